@@ -31,6 +31,11 @@ struct DevHam {
 
     const double *V = nullptr;   // V_eff, Nd
     const float *Vf = nullptr;   // V_eff rounded to float (FP32 filter)
+    // V_eff in the weights' units for the FP64 stencil: V vscale, vscale = -2 D h^2, as floor and
+    // 30-bit fraction; umin, umax: the floors' range (+-2^30 where V does not fit)
+    const int2 *uq = nullptr;
+    double vscale = 0;
+    int umin = 0, umax = 0;
 
     int natoms = 0;
     long nsup = 0;                   // support entries over all atoms
@@ -79,13 +84,14 @@ StepCoef<double> make_coef(const DevHam &H, double alpha, double shift, double b
 // scaled by a power of two per column, so each column needs a bound of its magnitude:
 // bY[c] = the largest high word (bits 32..62) of |y| over the column, as written by
 // colmax_f64 or by the launch that produced the block. bOut, if not null, is raised
-// (atomicMax) to the bound of the output's columns. u: alpha (V_eff - shift), Nd values
-// (from scaled_v; H.V itself when alpha = 1 and shift = 0).
+// (atomicMax) to the bound of the output's columns.
 cudaError_t stencil_f64(const DevHam &H, const double *Y, const double *Yprev, double *out,
-                        int ncols, long ld, double alpha, const double *u, double beta,
+                        int ncols, long ld, double alpha, double shift, double beta,
                         const unsigned *bY, unsigned *bOut, cudaStream_t st);
-cudaError_t scaled_v(const double *V, double alpha, double shift, double *u, long n,
-                     cudaStream_t st);
+// DevHam::uq from V (n values); lim[0] and lim[1] (device): lowered and raised to the
+// smallest and largest floor.
+cudaError_t potential_grid(const double *V, double vscale, int2 *uq, long n, int *lim,
+                           cudaStream_t st);
 // out += V_nl part from Cs = alpha chi^T Y (pairs), for FP64 outputs (nonlocal.cu); bOut
 // as for stencil_f64 (raised to the bound of the updated values), or null
 cudaError_t scatter_f64_df(const DevHam &H, const float2 *Cs, double *out, int ncols, long ld,

@@ -481,10 +481,10 @@ size_t sparc_request_bytes(const sparc_request *q)
     const int ns = q->ns;
     const size_t es = q->dtype == SPARC_F32 ? 4 : 8;
     const size_t na = q->natoms > 0 ? (size_t)q->natoms : 1;
-    // context: V_eff (FP64, FP32) and set-up scratch per node, projector entries (index,
+    // context: V_eff (FP64, FP32, integer units) and set-up scratch per node, projector entries (index,
     // chi and gamma chi in FP64 / FP32 / pairs, inverse map), bounded by the cube around
     // each support sphere
-    const size_t per_node = 8 + 4 + 4 * 8 + 8;
+    const size_t per_node = 8 + 4 + 8 + 4 * 8 + 8;
     const size_t per_entry = 4 + 4 + 32 + 32 + 16 + 16 + 32 + 4 + 4 + 16 + 32 + 16;
     const size_t entries = na * (size_t)nodes_in_support_box(q->h, 3.0);
     size_t b = per_node * (size_t)nd + per_entry * entries + 4096 * 64;
@@ -499,9 +499,8 @@ size_t sparc_request_bytes(const sparc_request *q)
     b += tc_slab_workspace(nd, ns, mixed);
     if (tc_slab_rows(nd, ns, mixed) < nd) b += sizeof(double) * 2 * (size_t)ns * ns;
     if (!mixed) {
-        // column bounds of the filter's blocks, alpha (V_eff - shift) of a step
+        // column bounds of the filter's blocks
         b += sizeof(unsigned) * ((size_t)(q->degree + 1) * ns + (size_t)ns);
-        b += 8 * (size_t)nd;
     }
     b += sizeof(double) * (4 * (size_t)ns * ns + 2 * (size_t)ns + (size_t)dense_work_elems(ns));
     b += sizeof(double) * (3 * (size_t)nd + kDotBlocks + 4096);

@@ -58,6 +58,7 @@ struct sparc_ctx {
     // owned tables
     double *V = nullptr;
     float *Vf = nullptr;
+    int2 *uq = nullptr;          // V_eff in the FP64 stencil's integer units
     int *atom_ptr = nullptr, *idx = nullptr, *ent_atom = nullptr;
     double *chi = nullptr, *gchi = nullptr;
     float *chi_f = nullptr, *gchi_f = nullptr;
@@ -81,7 +82,6 @@ struct sparc_ctx {
     void *lz = nullptr;      size_t lz_bytes = 0;    // Lanczos vectors and scalars
     void *bnd = nullptr;     size_t bnd_bytes = 0;   // column bounds of the FP64 filter's blocks
     void *bsc = nullptr;     size_t bsc_bytes = 0;   // column bounds of other FP64 H applications
-    void *vc = nullptr;      size_t vc_bytes = 0;    // alpha (V_eff - shift) of an FP64 step
     int *flags = nullptr;                            // device status words
     void *obs = nullptr;     size_t obs_bytes = 0;   // occupations, density and force data
     std::vector<double> gamma;                       // KB coefficients, 4 per atom (host)
@@ -249,20 +249,6 @@ sparc_status scratch_bounds(sparc_ctx *ctx, const T *Y, int ncols, long ld, unsi
     return SPARC_OK;
 }
 
-// alpha (V_eff - shift) for one FP64 step (formed on the context stream before the step;
-// V_eff itself for alpha = 1, shift = 0).
-sparc_status scaled_potential(sparc_ctx *ctx, double alpha, double shift, const double **u)
-{
-    if (alpha == 1.0 && shift == 0.0) {
-        *u = ctx->H.V;
-        return SPARC_OK;
-    }
-    TRY(ensure(ctx, ctx->vc, ctx->vc_bytes, sizeof(double) * (size_t)ctx->H.nd));
-    CK(scaled_v(ctx->H.V, alpha, shift, (double *)ctx->vc, ctx->H.nd, ctx->st));
-    *u = (const double *)ctx->vc;
-    return SPARC_OK;
-}
-
 // out = alpha ((H - shift) Y) - beta Yprev  (Yprev may alias out, may be null):
 // projection alpha chi^T Y, stencil step, nonlocal scatter-add. bY: column bounds of Y
 // (null: taken here by a pass over Y); bOut: raised to the bounds of out when not null.
@@ -276,13 +262,11 @@ sparc_status step_f64(sparc_ctx *ctx, const double *Y, const double *Yprev, doub
         TRY(scratch_bounds(ctx, Y, ncols, ld, &b));
         bY = b;
     }
-    const double *u = nullptr;
-    { PHASE(SPARC_PHASE_OTHER); TRY(scaled_potential(ctx, alpha, shift, &u)); }
     if (H.natoms > 0) {
         TRY(ensure_C(ctx, ncols));
         { PHASE(SPARC_PHASE_PROJECT); CK(project_f64_fx(H, Y, ncols, ld, alpha, bY, (float2 *)ctx->C, ctx->st)); }
     }
-    { PHASE(SPARC_PHASE_STENCIL); CK(stencil_f64(H, Y, Yprev, out, ncols, ld, alpha, u, beta, bY, bOut, ctx->st)); }
+    { PHASE(SPARC_PHASE_STENCIL); CK(stencil_f64(H, Y, Yprev, out, ncols, ld, alpha, shift, beta, bY, bOut, ctx->st)); }
     if (H.natoms > 0) { PHASE(SPARC_PHASE_SCATTER); CK(scatter_f64_df(H, (const float2 *)ctx->C, out, ncols, ld, bOut, ctx->st)); }
     return SPARC_OK;
 }
@@ -591,9 +575,9 @@ bool lap_weights_int(int no, double h, int *wint, double &wunit)
 void free_ctx(sparc_ctx *c)
 {
     if (!c) return;
-    void *ps[] = {c->V, c->Vf, c->atom_ptr, c->idx, c->ent_atom, c->chi, c->gchi, c->chi_f,
+    void *ps[] = {c->V, c->Vf, c->uq, c->atom_ptr, c->idx, c->ent_atom, c->chi, c->gchi, c->chi_f,
                   c->gchi_f, c->chi_q, c->chi_F, c->proj_order, c->uniq_node, c->uniq_ptr, c->ent_list, c->nl_atom, c->nl_gf, c->nl_gdf, c->C, c->hx, c->rotx, c->roth, c->part,
-                  c->tcws, c->dm, c->lz, c->bnd, c->bsc, c->vc, c->flags, c->obs, c->pois};
+                  c->tcws, c->dm, c->lz, c->bnd, c->bsc, c->flags, c->obs, c->pois};
     for (void *p : ps) dfree(p);
     for (cudaEvent_t e : c->prof.pool) cudaEventDestroy(e);
     for (cudaEvent_t e : c->prof.used) cudaEventDestroy(e);
@@ -790,9 +774,19 @@ sparc_status sparc_create(const sparc_grid *grid, const double *veff_host,
         CK(to_float(ctx->V, ctx->Vf, nd, ctx->st));
         H.V = ctx->V;
         H.Vf = ctx->Vf;
+        // the range words (flags 0, 1) are read at the end of the set-up
+        H.vscale = -2.0 / H.wunit;
+        TRY(dmalloc(ctx, ctx->uq, nd));
+        CK(potential_grid(ctx->V, H.vscale, ctx->uq, nd, ctx->flags, ctx->st));
+        CK(cudaMemcpyAsync(ctx->pin_i, ctx->flags, sizeof(int) * 2, cudaMemcpyDeviceToHost,
+                           ctx->st));
+        CK(cudaMemsetAsync(ctx->flags, 0, sizeof(int) * 2, ctx->st));
         TRY(build_tables(ctx, atoms));
         CK(cudaStreamSynchronize(ctx->st));
         CK(cudaGetLastError());
+        H.uq = ctx->uq;
+        H.umin = ctx->pin_i[0];
+        H.umax = ctx->pin_i[1];
         return SPARC_OK;
     };
     s = run();
