@@ -1,5 +1,5 @@
 // gram_df.cu -- FP64 subspace contractions in FP32-pair arithmetic (Sec. 3.4 projection
-// M_s = Y^T Y, H_s = Y^T (H Y), and the rotation of Eq. OrbitalTransformation).
+// M_s = Y^T Y, H_s = Y^T (H Y)).
 //
 // GB300's FP64 pipe issues at 1/64 of the FP32 rate, so a native FP64 Gram of a
 // 884736 x 128 block takes ~23 ms. Here every FP64 input is split into an FP32 pair
@@ -163,79 +163,5 @@ template cudaError_t gram_df_launch<float, float>(const float *, long, const flo
 template cudaError_t gram_df_launch<float, double>(const float *, long, const double *, long,
                                                    long, int, double *, double *, int, bool,
                                                    cudaStream_t);
-
-// ---- rotation out = A Q in FP32-pair arithmetic (FP64 blocks) ------------------------
-__global__ void __launch_bounds__(256)
-k_rotate_df(const double *__restrict__ A, long lda, long nd, int ns, const double *__restrict__ Q,
-            double *__restrict__ out, long ldo)
-{
-    __shared__ float2 As[GK][GT + 1];
-    __shared__ float2 Qs[GK][GT + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int j0 = blockIdx.x * GT;  // column tiles of a row tile run side by side (L2 reuse)
-    for (long rt = blockIdx.y; rt * GT < nd; rt += gridDim.y) {
-    const long r0 = rt * GT;
-    float sh[4][4], sl[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) sh[a][b] = sl[a][b] = 0.0f;
-    const float2 z = make_float2(0.0f, 0.0f);
-    for (int k0 = 0; k0 < ns; k0 += GK) {
-        {
-            const int rr = threadIdx.x & 63, kc = threadIdx.x >> 6;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int k = kc + 4 * u;
-                const long row = r0 + rr;
-                As[k][rr] = (row < nd && k0 + k < ns) ? split_double(A[row + (long)(k0 + k) * lda]) : z;
-            }
-        }
-        {
-            const int kk = threadIdx.x & 15, cc = threadIdx.x >> 4;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int c = cc + 16 * u;
-                Qs[kk][c] = (k0 + kk < ns && j0 + c < ns) ? split_double(Q[(k0 + kk) + (long)(j0 + c) * ns])
-                                                          : z;
-            }
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < GK; ++kk) {
-            float2 a[4], q[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = As[kk][ty + 16 * u];
-                q[u] = Qs[kk][tx + 16 * u];
-            }
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-#pragma unroll
-                for (int y = 0; y < 4; ++y) mac(a[x], q[y], sh[x][y], sl[x][y]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-            const long row = r0 + ty + 16 * x;
-            const int c = j0 + tx + 16 * y;
-            if (row < nd && c < ns) out[row + (long)c * ldo] = (double)sh[x][y] + (double)sl[x][y];
-        }
-    }
-}
-
-cudaError_t rotate_f64_df(const double *A, long lda, long nd, int ns, const double *Q, double *out,
-                          long ldo, cudaStream_t st)
-{
-    if (ns <= 0 || nd <= 0) return cudaSuccess;
-    const long gy = (nd + GT - 1) / GT;
-    dim3 grid((ns + GT - 1) / GT, (unsigned)(gy < 65535 ? gy : 65535));
-    k_rotate_df<<<grid, 256, 0, st>>>(A, lda, nd, ns, Q, out, ldo);
-    note_launch();
-    return cudaGetLastError();
-}
 
 }  // namespace sparc

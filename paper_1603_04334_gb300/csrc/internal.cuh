@@ -233,8 +233,6 @@ cudaError_t gram_f32_f64(const float *A, long lda, const double *B, long ldb, lo
 template <typename TA, typename TB>
 cudaError_t gram_df_launch(const TA *A, long lda, const TB *B, long ldb, long nd, int ns,
                            double *G, double *part, int nsplit, bool sym, cudaStream_t st);
-cudaError_t rotate_f64_df(const double *A, long lda, long nd, int ns, const double *Q, double *out,
-                          long ldo, cudaStream_t st);
 // FP64 Gram with a caller-chosen number of row slices (part: nsplit * ns * ns doubles).
 int gram_default_splits(int ns, long nd);
 // Tensor-core Gram of the mixed-precision form (gram_tc.cu): G = A^T B (ns x ns FP64,
@@ -292,9 +290,6 @@ cudaError_t gram_tc(const TA *A, long lda, const TB *B, long ldb, long nd, int n
                     void *ws, size_t ws_bytes, bool sym, int *err, cudaStream_t st);
 cudaError_t gram_f64_nsplit(const double *A, long lda, const double *B, long ldb, long nd, int ns,
                             double *G, double *part, int nsplit, cudaStream_t st);
-// out (nd x ns, ldo) = A (nd x ns, lda) Q (ns x ns, column-major FP64)
-cudaError_t rotate_f64(const double *A, long lda, long nd, int ns, const double *Q,
-                       double *out, long ldo, cudaStream_t st);
 
 // ---- dense.cu -------------------------------------------------------------------
 // Small dense Rayleigh-Ritz on the device (single CTA kernels), ns <= kMaxDense.
@@ -305,11 +300,11 @@ constexpr int kMaxDense = 1024;
 long dense_work_elems(int ns);
 cudaError_t dense_rr(double *M, double *Hs, int ns, double *ritz, double *Cf, double *work,
                      int *status, cudaStream_t st);
-// Symmetric eigensolve (cyclic Jacobi) of A (n x n, column-major, overwritten):
+// Symmetric eigensolve (cyclic Jacobi in one CTA) of A (n x n, column-major, n <= 64):
 // eigenvalues ascending in ev, eigenvectors (sign-fixed) in Q. n = *ns_dev when ns_dev is
-// not null (then n <= ns), else ns. work: dense_work_elems(ns).
-cudaError_t dense_syev(double *A, int ns, const int *ns_dev, double *ev, double *Q,
-                       double *work, int *status, cudaStream_t st);
+// not null (then n <= ns), else ns.
+cudaError_t dense_syev(const double *A, int ns, const int *ns_dev, double *ev, double *Q,
+                       int *status, cudaStream_t st);
 
 // ---- jacobi.cu --------------------------------------------------------------------
 // Grid-wide barrier state (zeroed before each cooperative launch).
@@ -324,13 +319,13 @@ struct GridBarrier {
 // sets *status = 3 if the sweeps do not converge; bar->err != 0 after a barrier timeout.
 cudaError_t jacobi_grid(double *A0, double *A1, double *V, double *diag, int n, GridBarrier *bar,
                         int *status, int *sweeps_out, cudaStream_t st);
-// Block Jacobi in FP32 (jacobi.cu): V = eigenvectors of the symmetric A (n x n, column-
-// major, overwritten by the nearly diagonal result); scratch of block_jacobi_f32_scratch(n)
-// bytes (device, 8-byte aligned); *sweeps_out (device) = sweeps used or -1. Synchronises
-// the stream once per sweep from the third on.
+// Block Jacobi in FP32 (jacobi.cu): V = approximate eigenvectors of the symmetric A64 (n x n,
+// column-major); A: n x n FP32 workspace; mx: a device word; scratch of
+// block_jacobi_f32_scratch(n) bytes (device, 8-byte aligned); *sweeps_out (device) = sweeps
+// used or -1. Synchronises the stream once per sweep from the fourth on.
 size_t block_jacobi_f32_scratch(int n);
-cudaError_t block_jacobi_f32(float *A, float *V, int n, void *scratch, int *sweeps_out,
-                             int max_sweeps, cudaStream_t st);
+cudaError_t block_jacobi_f32(const double *A64, float *A, float *V, int n, unsigned *mx,
+                             void *scratch, int *sweeps_out, int max_sweeps, cudaStream_t st);
 // Self-tests of the bounded waits (failure detection without a fault): a grid barrier
 // that can never complete (status <- 4 after its spin limit) and an mbarrier that never
 // completes (err <- 1 after its probe limit).
@@ -362,11 +357,13 @@ cudaError_t lanczos_bounds_final(const double *ev, const double *Q, const double
                                  const int *keff, double *out, cudaStream_t st);
 
 // ---- resid (gram.cu) --------------------------------------------------------------
-// resid[c] = || HX[:,c] - ritz[c] X[:,c] ||_2 (deterministic per-column reduction)
+// resid[c] = || HX[:,c] - ritz[c] X[:,c] ||_2 (deterministic per-column reduction); part:
+// resid_part_elems(ncols) doubles
+long resid_part_elems(int ncols);
 cudaError_t resid_f64(const double *X, const double *HX, long ld, long nd, int ncols,
-                      const double *ritz, double *resid, cudaStream_t st);
+                      const double *ritz, double *part, double *resid, cudaStream_t st);
 cudaError_t resid_f32(const float *X, const float *HX, long ld, long nd, int ncols,
-                      const double *ritz, double *resid, cudaStream_t st);
+                      const double *ritz, double *part, double *resid, cudaStream_t st);
 // flag |= 1 if any of n values is NaN or Inf
 cudaError_t check_finite(const double *a, long n, int *flag, cudaStream_t st);
 

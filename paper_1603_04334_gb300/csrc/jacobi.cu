@@ -11,17 +11,21 @@
 // of V in place (each (row, pair) belongs to one thread).
 //
 // Rotation angles follow Golub & Van Loan's symmetric Schur decomposition (Algorithm
-// 8.4.1); a rotation is skipped when |a_pq| <= 4 eps ||A||_F, and the sweeps stop after a
-// sweep that skipped all of them (as in dense.cu's single-CTA version). A round that
-// skips all of its rotations changes nothing, so it needs neither the update pass nor the
-// barrier (every CTA takes that decision from the same data).
+// 8.4.1; rotation.cuh); a rotation is skipped when |a_pq| <= 4 eps ||A||_F. Every sweep starts
+// with a scan of A for entries above that threshold: the rounds of those entries are the
+// ones the sweep visits (an entry that a rotation lifts above it later is found by the next
+// scan), and a scan that finds none ends the solve. After the refinement of dense.cu a few
+// entries at most are left, between eigenvalues too close for it: 128 states take 0.12 ms
+// where a sweep through all 127 rounds, with their angles and CTA barriers, took 0.4 to 0.9.
 //
 // The grid barrier is an arrival counter in global memory (grid.cuh); the kernel is launched
 // cooperatively (all CTAs co-resident), and every wait is bounded: after kBarrierSpins
 // polls the waiting CTA raises an error flag, every CTA leaves at its next barrier and the
 // host reports SPARC_ERR_TIMEOUT.
+#include "fx.cuh"
 #include "grid.cuh"
 #include "internal.cuh"
+#include "rotation.cuh"
 
 #include <atomic>
 
@@ -51,7 +55,6 @@ __device__ __forceinline__ void pair_of(int r, int k, int m, int &p, int &q)
     }
 }
 
-// Returns false (to every thread of the CTA) once any CTA has hit the spin limit.
 }  // namespace
 
 // T: the arithmetic (the eigensolve runs it in FP64), eps the unit roundoff of T.
@@ -63,7 +66,7 @@ k_jacobi_grid(T *A0, T *A1, T *V, T *diag, int n, GridBarrier *bar, int *status,
     __shared__ int sp[kMaxDense / 2], sq[kMaxDense / 2];
     __shared__ T sc[kMaxDense / 2], ss[kMaxDense / 2];
     __shared__ double red[NT / 32];
-    __shared__ int any_rot, round_rot;
+    __shared__ int flag[kMaxDense + 2], round_rot;
     if (*((volatile int *)status) != 0) return;  // the reduction step failed
     const unsigned nb = gridDim.x;
     const long nn = (long)n * n;
@@ -83,9 +86,24 @@ k_jacobi_grid(T *A0, T *A1, T *V, T *diag, int n, GridBarrier *bar, int *status,
     const int m = n + (n & 1), half = m / 2;
     int sweeps = -1;
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        if (threadIdx.x == 0) any_rot = 0;
+        // rounds with an entry above the threshold: i and j < m - 1 meet in the round r with
+        // 2 r = i + j modulo m - 1 (m / 2 is the inverse of 2), i and m - 1 in round i
+        for (int r = threadIdx.x; r < m; r += NT) flag[r] = 0;
         __syncthreads();
+        int found = 0, ri = threadIdx.x % n, rj = threadIdx.x / n;
+        for (long t = threadIdx.x; t < nn; t += NT) {
+            if (ri < rj && !(fabs(__ldcg(cur + t)) <= thr)) {
+                flag[rj == m - 1 ? ri : (int)((long)(ri + rj) * (m / 2) % (m - 1))] = 1;
+                found = 1;
+            }
+            for (ri += NT; ri >= n; ri -= n) ++rj;
+        }
+        if (!__syncthreads_or(found)) {
+            sweeps = sweep;
+            break;
+        }
         for (int r = 0; r < m - 1; ++r) {
+            if (!flag[r]) continue;
             if (threadIdx.x == 0) round_rot = 0;
             __syncthreads();
             for (int k = threadIdx.x; k < half; k += NT) {
@@ -97,11 +115,7 @@ k_jacobi_grid(T *A0, T *A1, T *V, T *diag, int n, GridBarrier *bar, int *status,
                     if (fabs(apq) > thr) {
                         const T app = __ldcg(cur + p + (long)p * n);
                         const T aqq = __ldcg(cur + q + (long)q * n);
-                        const T tau = (aqq - app) / ((T)2 * apq);
-                        const T t = (tau >= (T)0 ? (T)1 : (T)-1) / (fabs(tau) + sqrt((T)1 + tau * tau));
-                        c = (T)1 / sqrt((T)1 + t * t);
-                        s = t * c;
-                        any_rot = 1;
+                        jacobi_angle(app, aqq, apq, c, s);
                         round_rot = 1;
                     }
                 }
@@ -111,8 +125,9 @@ k_jacobi_grid(T *A0, T *A1, T *V, T *diag, int n, GridBarrier *bar, int *status,
                 ss[k] = s;
             }
             __syncthreads();
-            // a round without rotations leaves A and V as they are; every CTA computed the
-            // same angles from the same copy, so all of them skip it (and its barrier)
+            // an earlier round of the sweep may have taken the entry below the threshold: a
+            // round without rotations leaves A and V as they are, and every CTA, with the same
+            // angles from the same copy, skips it and its barrier
             if (!round_rot) continue;
             // 2 x 2 blocks: next = J_1^T cur J_2. A is symmetric, so block (k2, k1) of next is
             // the transpose of block (k1, k2): only k1 <= k2 is computed and written to both
@@ -158,12 +173,6 @@ k_jacobi_grid(T *A0, T *A1, T *V, T *diag, int n, GridBarrier *bar, int *status,
             T *t = cur;
             cur = nxt;
             nxt = t;
-        }
-        const int any = any_rot;
-        __syncthreads();
-        if (!any) {
-            sweeps = sweep + 1;
-            break;
         }
     }
     for (long i = gtid; i < n; i += gstride) diag[i] = __ldcg(cur + i + i * n);
@@ -244,26 +253,30 @@ cudaError_t barrier_selftest(GridBarrier *bar, int *status, cudaStream_t st)
 // The two-sided cyclic Jacobi method by blocks (the block form of the same Brent-Luk
 // round-robin ordering): the columns are cut into blocks of kBjB = 32, and in each round
 // the blocks are paired round-robin. For a pair (I, J) one CTA diagonalises the symmetric
-// subproblem S = A[I u J, I u J] (at most 64 x 64) in shared memory by kBjInner sweeps of
-// the scalar cyclic Jacobi (same angle formula and threshold as above) and stores the
-// accumulated rotation Q_IJ. A second kernel then applies all the round's rotations at
-// once: A[P, P'] <- Q_P^T A[P, P'] Q_P' for every pair of pairs (P <= P', the transpose
-// written to [P', P]) and V[R, P] <- V[R, P] Q_P for every 64-row block R, as 64 x 64
-// products in shared memory. Each tile is read and written by one CTA, so A and V are
+// subproblem S = A[I u J, I u J] (at most 64 x 64) in shared memory by one sweep of the scalar
+// cyclic Jacobi (same angle formula) and stores the accumulated rotation Q_IJ; when the pair is
+// the whole matrix, by as many sweeps as it takes. A second kernel then applies all the
+// round's rotations at once: A[P, P'] <- Q_P^T A[P, P'] Q_P' for every pair of pairs (P <= P',
+// the transpose written to [P', P]) and V[R, P] <- V[R, P] Q_P for every 64-row block R, as
+// 64 x 64 products in shared memory. Each tile is read and written by one CTA, so A and V are
 // updated in place. A sweep takes nb - 1 rounds of two launches for nb blocks (31 at
 // Ns = 1024, against 1023 barrier-separated rounds of the scalar form, each of which
-// streams all of A and V through L2). A sweep whose inner solves made no rotation ends
-// the solve: the kernels of later sweeps see the done flag and return at once.
+// streams all of A and V through L2). A is scaled to a largest entry in [1/2, 1); a rotation is
+// skipped below thr = 8 eps, and a sweep without a rotation above 8 thr ends the solve (the
+// FP64 refinement that follows converges quadratically from there; a sweep for the last bits
+// of FP32 would be one too many): the kernels of later sweeps see the done flag and
+// return at once.
 namespace {
 constexpr int kBjB = 32;                 // block size
 constexpr int kBjM = 2 * kBjB;           // largest subproblem
 constexpr int kBjLd = kBjM + 1;          // shared-memory row stride (no bank conflicts)
 constexpr int kBjThreads = 256;
-constexpr int kBjInner = 1;              // inner sweeps per subproblem and round
+constexpr int kBjSolveThreads = 1024;    // one 2 x 2 block of S per thread and round
+constexpr int kBjMaxInner = 20;
 
 struct BjState {
-    float thr;   // 4 eps ||A||_F
-    int rot;     // a rotation happened in the current sweep
+    float thr;   // 8 eps
+    int rot;     // a rotation above 8 thr happened in the current sweep
     int done;    // the solve has converged
     int sweeps;  // sweeps used
 };
@@ -288,23 +301,33 @@ __device__ __forceinline__ int bj_size(int blk, int n)
 }
 }  // namespace
 
-__global__ void __launch_bounds__(1024) k_bj_init(const float *__restrict__ A, float *V, int n,
-                                                  BjState *st, double eps)
+// *mx = max(*mx, high word of the largest |a|)
+__global__ void k_absmax(const double *__restrict__ a, long n, unsigned *mx)
 {
-    __shared__ double red[32];
-    double f = 0.0;
+    unsigned m = 0u;
+    for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
+         t += (long)gridDim.x * blockDim.x)
+        m = max(m, abs_hi_word(a[t]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) raise_bound(mx, m);
+}
+
+// A in FP32, scaled by a power of two to a largest entry in [1/2, 1) (eigenvectors do not
+// change), V = I and the solve's state.
+__global__ void k_bj_init(const double *__restrict__ A64, const unsigned *mx, float *A, float *V,
+                          int n, BjState *st)
+{
+    const unsigned m = *mx;
+    const int e = (int)(m >> 20);
+    const double sc = (e == 0 || e >= 0x7ff) ? 1.0 : ldexp(1.0, 1022 - e);
     const long nn = (long)n * n;
-    for (long t = threadIdx.x; t < nn; t += blockDim.x) {
-        f += (double)A[t] * (double)A[t];
+    for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < nn;
+         t += (long)gridDim.x * blockDim.x) {
+        A[t] = (float)(A64[t] * sc);
         V[t] = ((t % n) == (t / n)) ? 1.0f : 0.0f;
     }
-    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        st->thr = (float)(4.0 * eps * sqrt(s));
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->thr = 8.0f * 1.1920928955078125e-07f;
         st->rot = 0;
         st->done = 0;
         st->sweeps = -1;
@@ -323,92 +346,116 @@ __global__ void k_bj_sweep(BjState *st, int s, int phase)
     }
 }
 
-// Inner solve of each pair of round r: S = A[P, P] in shared memory, kBjInner cyclic
-// sweeps, Q (the accumulated rotation, kBjM x kBjM with an identity outside the subproblem)
-// to Qs[pair].
-__global__ void __launch_bounds__(kBjThreads)
-k_bj_solve(const float *__restrict__ A, int n, int nbe, int r, float *__restrict__ Qs,
+// Inner solve of each pair of round r: S = A[P, P] in shared memory, `inner` cyclic sweeps at
+// most, Q (the accumulated rotation, kBjM x kBjM with an identity outside the subproblem)
+// to Qs[pair]. Thread (k1, k2) updates the 2 x 2 block of pairs k1, k2 of S in place (both
+// sides at once: it reads and writes no other entry) and two rows of Q's column pair k2, so
+// a round is warp 0's angles and one update between two barriers. Bound by that chain
+// (barriers and the division / square root latency): 63 rounds in 53 us, against 164 us with
+// separate row and column passes over 256 threads and three barriers.
+__global__ void __launch_bounds__(kBjSolveThreads)
+k_bj_solve(const float *__restrict__ A, int n, int nbe, int r, int inner, float *__restrict__ Qs,
            BjState *st)
 {
     __shared__ float S[kBjM * kBjLd], Q[kBjM * kBjLd];
     __shared__ int sp[kBjB], sq[kBjB];
     __shared__ float sc[kBjB], ss[kBjB];
-    __shared__ int any;
+    __shared__ int round_rot, big_sweep, big_any;
     if (*(volatile int *)&st->done) return;
     int bi, bj;
     bj_pair(r, blockIdx.x, nbe, bi, bj);
     const int ni = bj_size(bi, n), nj = bj_size(bj, n), m = ni + nj;
     const float thr = st->thr;
-    for (int t = threadIdx.x; t < kBjM * kBjM; t += kBjThreads) {
+    const int tid = threadIdx.x, lane = tid & 31, k2 = tid >> 5;
+    for (int t = tid; t < kBjM * kBjM; t += kBjSolveThreads) {
         const int i = t % kBjM, j = t / kBjM;
         float v = 0.0f;
         if (i < m && j < m) v = A[bj_index(i, bi, ni, bj) + (long)bj_index(j, bi, ni, bj) * n];
         S[i + j * kBjLd] = v;
         Q[i + j * kBjLd] = i == j ? 1.0f : 0.0f;
     }
-    if (threadIdx.x == 0) any = 0;
-    __syncthreads();
+    if (tid == 0) big_any = 0;
+    // an odd m is padded by one zero row and column (m < kBjM then)
     const int me = m + (m & 1), half = me / 2;
-    for (int sw = 0; sw < kBjInner && m > 1; ++sw) {
+    for (int sw = 0; sw < inner && m > 1; ++sw) {
+        if (tid == 0) big_sweep = 0;
+        __syncthreads();
+        // pair `lane` of the round: (a, b) advance by one modulo me - 1
+        int a = lane, b = (lane == 0 ? me - 1 : me - 1 - lane);
         for (int rr = 0; rr < me - 1; ++rr) {
-            if (threadIdx.x < half) {
-                const int k = threadIdx.x;
-                int p, q;
-                pair_of(rr, k, me, p, q);
+            if (tid < 32) {
+                const int k = lane;
                 float c = 1.0f, s = 0.0f;
-                if (q < m) {
+                bool rot = false, big = false;
+                if (k < half) {
+                    const int p = min(a, b), q = max(a, b);
                     const float apq = S[p + q * kBjLd];
                     if (fabsf(apq) > thr) {
                         const float app = S[p + p * kBjLd], aqq = S[q + q * kBjLd];
-                        const float tau = (aqq - app) / (2.0f * apq);
-                        const float tt = (tau >= 0.0f ? 1.0f : -1.0f) /
-                                         (fabsf(tau) + sqrtf(1.0f + tau * tau));
-                        c = 1.0f / sqrtf(1.0f + tt * tt);
+                        // t = sgn(tau) |2 apq| / (|aqq - app| + sqrt((aqq - app)^2 + 4 apq^2)),
+                        // with the approximate reciprocals (P is made orthogonal in FP64)
+                        const float num = aqq - app, den = 2.0f * apq;
+                        const float h2 = fmaf(num, num, den * den);
+                        float tt = __fdividef(fabsf(den), fabsf(num) + h2 * rsqrtf(h2));
+                        if ((num < 0.0f) != (den < 0.0f) && num != 0.0f) tt = -tt;
+                        c = rsqrtf(fmaf(tt, tt, 1.0f));
                         s = tt * c;
-                        any = 1;
+                        rot = true;
+                        big = fabsf(apq) > 8.0f * thr;
+                    }
+                    sp[k] = p;
+                    sq[k] = q;
+                    sc[k] = c;
+                    ss[k] = s;
+                }
+                if (++a == me - 1) a = 0;
+                if (lane != 0 && ++b == me - 1) b = 0;
+                rot = __any_sync(0xffffffffu, rot);
+                big = __any_sync(0xffffffffu, big);
+                if (k == 0) {
+                    round_rot = rot;
+                    if (big) big_sweep = 1;
+                }
+            }
+            __syncthreads();
+            if (round_rot) {
+                if (lane < half && k2 < half) {
+                    const int p1 = sp[lane], q1 = sq[lane], p2 = sp[k2], q2 = sq[k2];
+                    const float c1 = sc[lane], s1 = ss[lane], c2 = sc[k2], s2 = ss[k2];
+                    const float app = S[p1 + p2 * kBjLd], apq = S[p1 + q2 * kBjLd];
+                    const float aqp = S[q1 + p2 * kBjLd], aqq = S[q1 + q2 * kBjLd];
+                    const float bpp = c1 * app - s1 * aqp, bpq = c1 * apq - s1 * aqq;
+                    const float bqp = s1 * app + c1 * aqp, bqq = s1 * apq + c1 * aqq;
+                    S[p1 + p2 * kBjLd] = c2 * bpp - s2 * bpq;
+                    S[p1 + q2 * kBjLd] = s2 * bpp + c2 * bpq;
+                    S[q1 + p2 * kBjLd] = c2 * bqp - s2 * bqq;
+                    S[q1 + q2 * kBjLd] = s2 * bqp + c2 * bqq;
+                }
+                if (k2 < half && ss[k2] != 0.0f) {
+                    const float c = sc[k2], s = ss[k2];
+                    float *vp = Q + sp[k2] * kBjLd, *vq = Q + sq[k2] * kBjLd;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int row = lane + 32 * u;
+                        const float x = vp[row], y = vq[row];
+                        vp[row] = c * x - s * y;
+                        vq[row] = s * x + c * y;
                     }
                 }
-                sp[k] = p;
-                sq[k] = q < m ? q : p;
-                sc[k] = c;
-                ss[k] = s;
-            }
-            __syncthreads();
-            // rows: S <- J^T S
-            for (int t = threadIdx.x; t < half * m; t += kBjThreads) {
-                const int k = t / m, col = t % m;
-                const float s = ss[k];
-                if (s == 0.0f) continue;
-                const float c = sc[k];
-                const int p = sp[k], q = sq[k];
-                const float ap = S[p + col * kBjLd], aq = S[q + col * kBjLd];
-                S[p + col * kBjLd] = c * ap - s * aq;
-                S[q + col * kBjLd] = s * ap + c * aq;
-            }
-            __syncthreads();
-            // columns: S <- S J, Q <- Q J
-            for (int t = threadIdx.x; t < half * m; t += kBjThreads) {
-                const int k = t / m, row = t % m;
-                const float s = ss[k];
-                if (s == 0.0f) continue;
-                const float c = sc[k];
-                const int p = sp[k], q = sq[k];
-                const float ap = S[row + p * kBjLd], aq = S[row + q * kBjLd];
-                S[row + p * kBjLd] = c * ap - s * aq;
-                S[row + q * kBjLd] = s * ap + c * aq;
-                const float vp = Q[row + p * kBjLd], vq = Q[row + q * kBjLd];
-                Q[row + p * kBjLd] = c * vp - s * vq;
-                Q[row + q * kBjLd] = s * vp + c * vq;
             }
             __syncthreads();
         }
+        if (!big_sweep) break;
+        if (tid == 0) big_any = 1;
+        __syncthreads();
     }
+    __syncthreads();
     float *qg = Qs + (long)blockIdx.x * kBjM * kBjM;
-    for (int t = threadIdx.x; t < kBjM * kBjM; t += kBjThreads) {
+    for (int t = tid; t < kBjM * kBjM; t += kBjSolveThreads) {
         const int i = t % kBjM, j = t / kBjM;
         qg[t] = Q[i + j * kBjLd];
     }
-    if (threadIdx.x == 0 && any) atomicExch(&st->rot, 1);
+    if (tid == 0 && big_any) atomicExch(&st->rot, 1);
 }
 
 // Application of round r's rotations. CTAs [0, npairs (npairs + 1) / 2): A tiles (P, P'),
@@ -547,23 +594,29 @@ size_t block_jacobi_f32_scratch(int n)
     return (size_t)(nbe / 2) * kBjM * kBjM * sizeof(float) + 256;
 }
 
-cudaError_t block_jacobi_f32(float *A, float *V, int n, void *scratch, int *sweeps_out,
-                             int max_sweeps, cudaStream_t st)
+cudaError_t block_jacobi_f32(const double *A64, float *A, float *V, int n, unsigned *mx,
+                             void *scratch, int *sweeps_out, int max_sweeps, cudaStream_t st)
 {
     if (n <= 0 || n > kMaxDense) return cudaErrorInvalidValue;
     const int nb = (n + kBjB - 1) / kBjB, nbe = nb + (nb & 1), npairs = nbe / 2;
     BjState *bs = reinterpret_cast<BjState *>(scratch);
     float *Qs = reinterpret_cast<float *>(reinterpret_cast<char *>(scratch) + 256);
-    k_bj_init<<<1, 1024, 0, st>>>(A, V, n, bs, 1.1920928955078125e-07);
+    const long nn = (long)n * n;
+    const int g = (int)((nn + 255) / 256 < 152 * 4 ? (nn + 255) / 256 : 152 * 4);
+    cudaError_t e = cudaMemsetAsync(mx, 0, sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    k_absmax<<<g, 256, 0, st>>>(A64, nn, mx);
     note_launch();
+    k_bj_init<<<g, 256, 0, st>>>(A64, mx, A, V, n, bs);
+    note_launch();
+    const int inner = nbe == 2 ? kBjMaxInner : 1;
     const int nrb = (n + kBjM - 1) / kBjM;
     const int napply = npairs * (npairs + 1) / 2 + npairs * nrb;
-    cudaError_t e;
     for (int s = 0; s < max_sweeps; ++s) {
         k_bj_sweep<<<1, 1, 0, st>>>(bs, s, 0);
         note_launch();
         for (int r = 0; r < nbe - 1; ++r) {
-            k_bj_solve<<<npairs, kBjThreads, 0, st>>>(A, n, nbe, r, Qs, bs);
+            k_bj_solve<<<npairs, kBjSolveThreads, 0, st>>>(A, n, nbe, r, inner, Qs, bs);
             note_launch();
             k_bj_apply<<<napply, kBjThreads, 0, st>>>(A, V, n, nbe, r, Qs, bs);
             note_launch();
@@ -571,8 +624,8 @@ cudaError_t block_jacobi_f32(float *A, float *V, int n, void *scratch, int *swee
         k_bj_sweep<<<1, 1, 0, st>>>(bs, s, 1);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (s >= 2) {
-            // from the third sweep on the host looks at the done flag (one small copy and a
+        if (s >= 3 || nbe == 2) {
+            // from the fourth sweep on the host looks at the done flag (one small copy and a
             // stream synchronisation per sweep) instead of queueing sweeps that would return
             int done = 0;
             if ((e = cudaMemcpyAsync(&done, &bs->done, sizeof(int), cudaMemcpyDeviceToHost,

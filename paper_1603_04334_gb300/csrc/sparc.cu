@@ -478,7 +478,7 @@ sparc_status rr_core(sparc_ctx *ctx, T *Yf, T *dst, double *HX, int ns, long ld,
                 for (long r0 = 0; r0 < nd; r0 += slab)
                     CK(rotate_tc(HX + r0, ld, nd - r0 < slab ? nd - r0 : slab, ns, d.Cf, hxr + r0, ld, ctx->tcws, ctx->tcws_bytes, ctx->H.err, ctx->st));
             }
-            { PHASE(SPARC_PHASE_OTHER); CK(resid_f64((const double *)xout, hxr, ld, nd, ns, d.ritz, d.resid, ctx->st)); }
+            { PHASE(SPARC_PHASE_OTHER); CK(resid_f64((const double *)xout, hxr, ld, nd, ns, d.ritz, d.work, d.resid, ctx->st)); }
         } else {
             float *hxr = (float *)ctx->roth;
             {
@@ -486,7 +486,7 @@ sparc_status rr_core(sparc_ctx *ctx, T *Yf, T *dst, double *HX, int ns, long ld,
                 for (long r0 = 0; r0 < nd; r0 += slab)
                     CK(rotate_tc23<double>(HX + r0, ld, nd - r0 < slab ? nd - r0 : slab, ns, d.Cf, hxr + r0, ld, ctx->tcws, ctx->tcws_bytes, ctx->H.err, ctx->st));
             }
-            { PHASE(SPARC_PHASE_OTHER); CK(resid_f32((const float *)xout, hxr, ld, nd, ns, d.ritz, d.resid, ctx->st)); }
+            { PHASE(SPARC_PHASE_OTHER); CK(resid_f32((const float *)xout, hxr, ld, nd, ns, d.ritz, d.work, d.resid, ctx->st)); }
         }
     }
     if (xout != dst) TRY(copy_block<T>(ctx, dst, xout, ns, ld));
@@ -991,12 +991,12 @@ sparc_status sparc_lanczos_bounds(sparc_ctx *ctx, int ksteps, unsigned long long
         return fail(ctx, SPARC_ERR_ARG, "ksteps must be in 1..%d (got %d)", kMaxLanczos, ksteps);
     const long nd = ctx->H.nd;
     const int K = kMaxLanczos;
-    const size_t nsc = 4 * (size_t)K + 8 + 2 * (size_t)K * K + (size_t)dense_work_elems(K);
+    const size_t nsc = 4 * (size_t)K + 8 + 2 * (size_t)K * K;
     const size_t tot = 3 * (size_t)nd + (size_t)kDotBlocks + nsc;
     TRY(ensure(ctx, ctx->lz, ctx->lz_bytes, tot * sizeof(double)));
     double *v = (double *)ctx->lz, *vp = v + nd, *w = vp + nd, *part = w + nd;
     double *alpha = part + kDotBlocks, *beta = alpha + K, *nrm2 = beta + K, *outb = nrm2 + 2,
-           *ev = outb + 4, *T = ev + K + 2, *Q = T + (size_t)K * K, *work = Q + (size_t)K * K;
+           *ev = outb + 4, *T = ev + K + 2, *Q = T + (size_t)K * K;
     int *stop = ctx->flags + 4, *keff = ctx->flags + 5, *status = ctx->flags + 6;
     CK(cudaMemsetAsync(ctx->flags + 4, 0, sizeof(int) * 3, ctx->st));
     CK(cudaMemsetAsync(vp, 0, sizeof(double) * nd, ctx->st));
@@ -1013,7 +1013,7 @@ sparc_status sparc_lanczos_bounds(sparc_ctx *ctx, int ksteps, unsigned long long
         { PHASE(SPARC_PHASE_OTHER); CK(lanczos_next(v, vp, w, nd, beta, j, stop, ctx->st)); }
     }
     { PHASE(SPARC_PHASE_OTHER); CK(lanczos_tridiag(alpha, beta, ksteps, stop, T, keff, ctx->st)); }
-    { PHASE(SPARC_PHASE_DENSE); CK(dense_syev(T, ksteps, keff, ev, Q, work, status, ctx->st)); }
+    { PHASE(SPARC_PHASE_DENSE); CK(dense_syev(T, ksteps, keff, ev, Q, status, ctx->st)); }
     { PHASE(SPARC_PHASE_OTHER); CK(lanczos_bounds_final(ev, Q, beta, ksteps, keff, outb, ctx->st)); }
     CK(cudaMemcpyAsync(ctx->pin, outb, sizeof(double) * 2, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaMemcpyAsync(ctx->pin_i, status, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
