@@ -556,8 +556,9 @@ k_chol_grid(double *M, double *Hs, int n, double *Lr, double *dinv, double *odia
     const unsigned nb = gridDim.x;
     const long gtid = (long)blockIdx.x * CT + threadIdx.x, gs = (long)nb * CT;
     const long nn = (long)n * n;
+    unsigned epoch = 0;
     auto sync = [&]() -> bool {
-        if (grid_barrier(bar, nb)) return true;
+        if (grid_barrier(bar, nb, epoch)) return true;
         if (threadIdx.x == 0) atomicExch(status, 4);
         return false;
     };

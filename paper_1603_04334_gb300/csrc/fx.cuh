@@ -1,5 +1,5 @@
 // fx.cuh -- per-column magnitude bounds of FP64 blocks and the fixed-point grid they
-// define, shared by the FP64 stencil (stencil_df.cu), the nonlocal projection and pair
+// define, shared by the FP64 stencil (stencil_df.cu, poisson.cu), the nonlocal projection and pair
 // scatter (nonlocal.cu) and the bound pass (bounds.cu). A bound is the largest high word
 // (bits 32..62) of |y| over a column; it only grows.
 #pragma once
@@ -62,6 +62,39 @@ __device__ __forceinline__ int2 fx_split(float y, int E)
     const int d = ((int)(unsigned)(N >> 23) ^ sm) - sm;
     const int r = ((int)((unsigned)N & 0x7fffffu) ^ sm) - sm;
     return make_int2(d, r);
+}
+
+// A value on the column's grid: .x = d, .y = the bits of r (y 2^(26-E) = d + 2^-32 r, |y| < 2^E).
+// With the significand at the top of 64 bits, y = (h:l) 2^(e-1086), N = (h:l) >> s with s =
+// 1028 + E - e (s >= 6 when |y| < 2^E) is |y| 2^(58-E): its high word is d (below 2^26), its low
+// word, rounded to FP32, r. Zero and subnormal y give 0; the sign is applied to both parts. The
+// rounding matters: a truncated y has an error of y's own sign, which in the potential term
+// (unlike in the Laplacian, whose weights sum to zero) does not cancel and which the filter
+// amplifies (10 times the error of a degree-20 filter with 23 truncated bits).
+__device__ __forceinline__ int2 grid_parts(unsigned h, unsigned l, int s, unsigned sign)
+{
+    const unsigned long long N = (((unsigned long long)h << 32) | l) >> min(s, 63);
+    const int sm = (int)sign >> 31;  // 0 or -1
+    const int d = ((int)(unsigned)(N >> 32) ^ sm) - sm;
+    const float r = __uint2float_rn((unsigned)N);
+    return make_int2(d, (int)(__float_as_uint(r) | (sign & 0x80000000u)));
+}
+
+__device__ __forceinline__ int2 to_grid(double y, int E)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(y);
+    const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
+    const int e = (int)((hw >> 20) & 0x7ffu);
+    const unsigned h = e ? __funnelshift_l(lw, hw, 11) | 0x80000000u : 0u;
+    return grid_parts(h, e ? lw << 11 : 0u, 1028 + E - e, hw);
+}
+
+// FP32 input: y = (h:0) 2^(e-190).
+__device__ __forceinline__ int2 to_grid(float y, int E)
+{
+    const unsigned u = __float_as_uint(y);
+    const int e = (int)((u >> 23) & 0xffu);
+    return grid_parts(e ? (u << 8) | 0x80000000u : 0u, 0u, 132 + E - e, u);
 }
 
 }  // namespace sparc

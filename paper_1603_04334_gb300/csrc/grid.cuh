@@ -10,39 +10,46 @@
 
 namespace sparc {
 
-constexpr unsigned long long kBarrierSpins = 1ull << 25;  // polls (each an L2 round trip + 32 ns)
+constexpr unsigned long long kBarrierSpins = 1ull << 25;  // polls (each an L2 round trip)
 
-// The count only grows (the host zeroes the barrier before each launch): a CTA arrives with
-// a release add, which returns the arrivals before it, and waits with acquire loads until
-// the count reaches the next multiple of nblocks. The last CTA to arrive thus opens the
-// barrier with its own add, with no reset on the critical path. Thread 0 arrives and waits
-// for its CTA, between two CTA barriers.
-__device__ __forceinline__ bool grid_barrier(GridBarrier *b, unsigned nblocks,
+// The count only grows (the host zeroes the barrier before each launch), and every CTA counts
+// the barriers it has passed in `epoch` (0 at the launch's start): a CTA arrives with a release
+// add that returns nothing, and waits with acquire loads until the count reaches epoch x
+// nblocks, so the last CTA to arrive opens the barrier with its own add and no CTA waits for
+// its own add's answer. Thread 0 arrives and waits for its CTA, between two CTA barriers, the
+// second of which hands its result to the others. The error flag is looked at every 64 polls:
+// two dependent L2 round trips a poll and one after it made a barrier 2 us, 1 us so.
+__device__ __forceinline__ bool grid_barrier(GridBarrier *b, unsigned nblocks, unsigned &epoch,
                                              unsigned long long spins = kBarrierSpins)
 {
+    ++epoch;
     __syncthreads();
+    int fail = 0;
     if (threadIdx.x == 0) {
-        unsigned old;
-        asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;"
-                     : "=r"(old) : "l"(&b->count) : "memory");
-        const unsigned target = (old / nblocks + 1u) * nblocks;
-        volatile int *ve = &b->err;
+        asm volatile("red.release.gpu.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
+        const unsigned target = epoch * nblocks;
         unsigned long long it = 0;
         for (;;) {
             unsigned c;
             asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(c) : "l"(&b->count) : "memory");
-            // leaves when every CTA has arrived, when another CTA has given up, or after
-            // `spins` polls (then it raises the flag itself)
-            if ((int)(c - target) >= 0 || *ve != 0) break;
-            if (++it > spins) {
-                atomicExch(&b->err, 1);
-                break;
+            if ((int)(c - target) >= 0) break;
+            // leaves when another CTA has given up, or after `spins` polls (then it raises the
+            // flag itself)
+            if ((++it & 63) == 0) {
+                if (*((volatile int *)&b->err) != 0) {
+                    fail = 1;
+                    break;
+                }
+                if (it > spins) {
+                    atomicExch(&b->err, 1);
+                    fail = 1;
+                    break;
+                }
+                __nanosleep(32);
             }
-            __nanosleep(32);
         }
     }
-    __syncthreads();
-    return *((volatile int *)&b->err) == 0;
+    return !__syncthreads_or(fail);
 }
 
 }  // namespace sparc

@@ -80,7 +80,8 @@ k_jacobi_grid(T *A0, T *A1, T *V, T *diag, int n, GridBarrier *bar, int *status,
     double fro = 0.0;
     for (int w = 0; w < NT / 32; ++w) fro += red[w];
     const T thr = (T)(4.0 * eps * sqrt(fro));
-    if (!grid_barrier(bar, nb)) return;
+    unsigned epoch = 0;
+    if (!grid_barrier(bar, nb, epoch)) return;
 
     T *cur = A0, *nxt = A1;
     const int m = n + (n & 1), half = m / 2;
@@ -169,7 +170,7 @@ k_jacobi_grid(T *A0, T *A1, T *V, T *diag, int n, GridBarrier *bar, int *status,
                 V[row + (long)p * n] = c * vp - s * vq;
                 V[row + (long)q * n] = s * vp + c * vq;
             }
-            if (!grid_barrier(bar, nb)) return;
+            if (!grid_barrier(bar, nb, epoch)) return;
             T *t = cur;
             cur = nxt;
             nxt = t;
@@ -231,7 +232,8 @@ cudaError_t jacobi_grid(double *A0, double *A1, double *V, double *diag, int n, 
 // the barrier (wrongly) completed.
 __global__ void __launch_bounds__(32) k_barrier_selftest(GridBarrier *bar, int *status)
 {
-    const bool ok = grid_barrier(bar, gridDim.x + 1u, 1ull << 20);
+    unsigned epoch = 0;
+    const bool ok = grid_barrier(bar, gridDim.x + 1u, epoch, 1ull << 20);
     if (threadIdx.x == 0 && !ok) atomicExch(status, 4);
 }
 

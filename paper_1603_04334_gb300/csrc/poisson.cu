@@ -2,7 +2,8 @@
 // PseudochargeDiscrete, Algorithm PseudochargeCalculation), multipole boundary values (Eq.
 // phi:BC:discrete, l_max = 6 as in Sec. 4), the charge correction (Eq. Phi:correction)
 // and the linear system -(1/4 pi) L_h phi = rho + b - d (Eq. FD:PoissonDiscrete) solved by
-// conjugate gradients with a Jacobi preconditioner, all in FP64 on the device.
+// conjugate gradients with a Jacobi preconditioner, all on the device in FP64 (the operator
+// as exact integer sums, below).
 //
 // The multipole terms use real solid harmonics R_lm(x) = |x|^l Y_lm(x/|x|), evaluated as
 // polynomials: with Pi_l^m(z, r^2) the associated-Legendre recurrence in solid form
@@ -14,7 +15,14 @@
 //
 // Every reduction (moments, CG dot products) runs in a fixed order: a block-level tree,
 // then one CTA over the block partials, so results repeat bit for bit.
+#include "fx.cuh"
+#include "grid.cuh"
 #include "internal.cuh"
+#include "rotation.cuh"
+
+#include <algorithm>
+#include <atomic>
+#include <cmath>
 
 namespace sparc {
 
@@ -24,7 +32,7 @@ constexpr int kNQ = (kLmax + 1) * (kLmax + 1);  // 49 moments
 constexpr int kPT = 256;                         // threads of the grid-wide kernels
 constexpr double kInv4Pi = 0.07957747154594767;  // 1 / (4 pi)
 constexpr double kSqrtPi = 1.7724538509055159;
-constexpr int kVecGrid = 152 * 8;                // CTAs of the vector kernels and dot products
+constexpr int kMomPer = 8;                       // nodes per thread of the moments
 }  // namespace
 
 // R_lm(x, y, z) for l <= 6 into S[l*l + l + m] (N: the 49 normalisation constants, same
@@ -122,28 +130,31 @@ k_pseudocharge(const double *__restrict__ Ve, double *__restrict__ b, int n0, in
     b[t] = -kInv4Pi * L;
 }
 
-// Block partials of sum (rho + b) R_lm(x - centre) over the grid: part[block * 49 + q].
+// Block partials of sum (rho + b) R_lm(x - centre) over the grid: part[block * 49 + q]. A
+// thread sums kMomPer nodes before the 49 block reductions.
 __global__ void __launch_bounds__(kPT)
 k_moments(const double *__restrict__ rho, const double *__restrict__ b, int n0, int n1, int n2,
           PoisCoef pc, double *__restrict__ part)
 {
     __shared__ double sh[kPT / 32][kNQ];
-    const long t = (long)blockIdx.x * kPT + threadIdx.x;
     const long nd = (long)n0 * n1 * n2;
-    double S[kNQ];
-    double f = 0.0;
-    if (t < nd) {
-        f = (rho ? rho[t] : 0.0) + b[t];
+    double A[kNQ];
+#pragma unroll
+    for (int q = 0; q < kNQ; ++q) A[q] = 0.0;
+    for (int u = 0; u < kMomPer; ++u) {
+        const long t = ((long)blockIdx.x * kMomPer + u) * kPT + threadIdx.x;
+        if (t >= nd) break;
+        double S[kNQ];
+        const double f = (rho ? rho[t] : 0.0) + b[t];
         const int i = (int)(t % n0), j = (int)((t / n0) % n1), k = (int)(t / ((long)n0 * n1));
         solid_harmonics(i * pc.h - pc.cx, j * pc.h - pc.cy, k * pc.h - pc.cz, pc.N, S);
-    } else {
 #pragma unroll
-        for (int q = 0; q < kNQ; ++q) S[q] = 0.0;
+        for (int q = 0; q < kNQ; ++q) A[q] = fma(f, S[q], A[q]);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < kNQ; ++q) {
-        double v = f * S[q];
+        double v = A[q];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if (lane == 0) sh[warp][q] = v;
@@ -156,23 +167,21 @@ k_moments(const double *__restrict__ rho, const double *__restrict__ b, int n0, 
     }
 }
 
-// out[q] = scale * sum_b part[b * stride + q] over nblk blocks (one CTA, fixed order).
+// out[q] = scale * sum_b part[b * nq + q] over nblk blocks (CTA q, fixed order).
 __global__ void __launch_bounds__(kPT)
 k_sum_partials(const double *__restrict__ part, int nblk, int nq, double scale, double *out)
 {
     __shared__ double sh[kPT];
-    for (int q = 0; q < nq; ++q) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < nblk; b += kPT) v += part[(long)b * nq + q];
-        sh[threadIdx.x] = v;
-        __syncthreads();
-        for (int s = kPT / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[q] = scale * sh[0];
+    const int q = blockIdx.x;
+    double v = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += kPT) v += part[(long)b * nq + q];
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int s = kPT / 2; s > 0; s >>= 1) {
+        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
         __syncthreads();
     }
+    if (threadIdx.x == 0) out[q] = scale * sh[0];
 }
 
 // phi at the nodes outside the grid that a grid node's stencil reaches: face f (0: i < 0,
@@ -259,156 +268,413 @@ k_poisson_rhs(const double *__restrict__ rho, const double *__restrict__ b,
     rhs[t] = (rho ? rho[t] : 0.0) + b[t] - d;
 }
 
-// out = -(1/4 pi) L_h in (zero Dirichlet), one node per thread; the FP64 stencil of a
-// single vector is light enough for the plain form.
-__global__ void __launch_bounds__(kPT)
-k_poisson_apply(const double *__restrict__ in, double *__restrict__ out, int n0, int n1, int n2,
-                PoisCoef pc, const int *done)
+// ---- conjugate gradients in one cooperative kernel ---------------------------------------
+// The Jacobi preconditioner of this operator is one number (its diagonal is constant), which
+// cancels from the iteration: x, r, alpha p and the iteration count are those of
+//   alpha = r.r / p.Ap;  x += alpha p;  r -= alpha A p;  beta = r'.r' / r.r;  p = r' + beta p.
+// Three phases per iteration, a grid barrier after each:
+//   A  A p on bricks of 16 x 16 x bz nodes, one or more per CTA, and partial sums of p.Ap;
+//   B  r -= alpha A p, partial sums of r.r and the largest |r|;
+//   C  x += alpha p, p = r + beta p, p's grid form and its largest magnitude.
+// The operator works on p's fixed-point grid (d, r) as the FP64 stencil does (stencil_df.cu):
+// exact integer neighbour sums and an FP32 remainder, two FP64 operations a node instead of 37.
+// Phase C writes that form, with the exponent from |p_new| <= max |r| + beta max |p|, so phase A
+// converts nothing. Every CTA adds the CTAs' partial sums itself, in the same order.
+//
+// Bound by latency: three barriers, the brick's loads from L2 and short FP64 chains (an FP64
+// warp instruction holds its quarter of the SM for 64 cycles). 64^3: 85 us an iteration with
+// seven launches (the FP64 operator 27 us, two dot products and their one-CTA sums 37 us), 19
+// us so.
+namespace {
+constexpr int kCgThreads = 512;
+constexpr int kBr = 16;                        // brick edge along x and y
+constexpr int kBrH = kBr + 2 * kRadius;        // with the halo
+constexpr int kCgSmemMax = 200 * 1024;
+constexpr int kCgMaxGrid = 152;                // one CTA per SM (all resident: grid barriers)
+constexpr int kCgPerLaunch = 512;              // iterations of one launch
+
+// shared memory of a brick bz planes high: the planes with their x and y halos, then the
+// columns without them, z halo included (so that every neighbour is at a constant offset)
+constexpr long cg_smem(int bz) { return 8L * (kBrH * kBrH * bz + kBr * kBr * (bz + 2 * kRadius)); }
+
+struct CgState {
+    double ff, rr;      // |f|^2, r.r
+    int E;              // p's grid exponent: |p| < 2^E
+    int done, iters;
+    GridBarrier bar;
+};
+
+struct CgArgs {
+    double *x, *r, *p, *Ap;
+    int2 *q;            // p on its grid
+    const double *f;
+    double *part;       // kCgMaxGrid sums
+    unsigned *pmax;     // kCgMaxGrid maxima
+    CgState *s;
+    int n0, n1, n2, bz;
+    int W[kRadius + 1];
+    float Wf[kRadius + 1];
+    double scale;       // -(1/4 pi) / (D h^2)
+    double tol2;
+    int first, last;    // iterations of this launch
+};
+
+// The CTA's sum of v and maximum of m into *part and *pmax, in a fixed order. An FP64 add
+// holds its quarter of the SM for 64 cycles whatever its active lanes, so the sum halves
+// through shared memory (20 warp-wide adds) rather than by shuffles in all 16 warps (84).
+__device__ __forceinline__ void cg_put(double v, unsigned m, double *part, unsigned *pmax)
 {
-    if (*(volatile const int *)done) return;
-    const long t = (long)blockIdx.x * kPT + threadIdx.x;
-    const long nd = (long)n0 * n1 * n2;
-    if (t >= nd) return;
-    const int i = (int)(t % n0), j = (int)((t / n0) % n1), k = (int)(t / ((long)n0 * n1));
-    const long pl = (long)n0 * n1;
-    double L = 6.0 * pc.w[0] * in[t];
-    for (int p = 1; p <= pc.radius; ++p) {
-        double s = 0.0;
-        if (i + p < n0) s += in[t + p];
-        if (i - p >= 0) s += in[t - p];
-        if (j + p < n1) s += in[t + (long)p * n0];
-        if (j - p >= 0) s += in[t - (long)p * n0];
-        if (k + p < n2) s += in[t + p * pl];
-        if (k - p >= 0) s += in[t - p * pl];
-        L += pc.w[p] * s;
+    __shared__ double sv[kCgThreads];
+    __shared__ unsigned sm[kCgThreads / 32];
+    const int tid = threadIdx.x;
+    sv[tid] = v;
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((tid & 31) == 0) sm[tid >> 5] = m;
+    __syncthreads();
+    for (int h = kCgThreads / 2; h >= 32; h >>= 1) {
+        if (tid < h) sv[tid] = v = v + sv[tid + h];
+        if (h > 32) __syncthreads();
     }
-    out[t] = -kInv4Pi * L;
+    if (tid < 32) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        m = __reduce_max_sync(0xffffffffu, tid < kCgThreads / 32 ? sm[tid] : 0u);
+        if (tid == 0) *part = v, *pmax = m;
+    }
 }
 
-// Block partials of a.b (and of c.c when c is not null): part[2 block], part[2 block + 1].
-__global__ void __launch_bounds__(kPT)
-k_dot2(const double *__restrict__ a, const double *__restrict__ b, const double *__restrict__ c,
-       long n, double *__restrict__ part, const int *done)
+// The CTA's maximum alone
+__device__ __forceinline__ void cg_put_max(unsigned m, unsigned *pmax)
 {
-    __shared__ double sh[2][kPT / 32];
-    if (*(volatile const int *)done) return;
-    double u = 0.0, v = 0.0;
-    for (long t = (long)blockIdx.x * kPT + threadIdx.x; t < n; t += (long)gridDim.x * kPT) {
-        u = fma(a[t], b[t], u);
-        if (c) v = fma(c[t], c[t], v);
+    __shared__ unsigned sm[kCgThreads / 32];
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = __reduce_max_sync(0xffffffffu, threadIdx.x < kCgThreads / 32 ? sm[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) *pmax = m;
     }
+}
+
+// The sum of part and the maxima of pa and pb over all CTAs (after a grid barrier), handed to
+// `fin` in thread 0, which leaves the iteration's scalars in shared memory: one thread does the
+// FP64 divisions. Ends with a CTA barrier.
+template <typename F>
+__device__ __forceinline__ void cg_get(const double *part, const unsigned *pa, const unsigned *pb,
+                                       F fin)
+{
+    if (threadIdx.x < 32) {
+        double t[kCgMaxGrid / 32 + 1];
+        unsigned x = 0u, y = 0u;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        u += __shfl_down_sync(0xffffffffu, u, o);
-        v += __shfl_down_sync(0xffffffffu, v, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = u;
-        sh[1][threadIdx.x >> 5] = v;
+        for (int k = 0; k <= kCgMaxGrid / 32; ++k) {
+            const int b = threadIdx.x + 32 * k;
+            const bool in = b < (int)gridDim.x;
+            t[k] = in ? __ldcg(part + b) : 0.0;
+            x = max(x, in ? __ldcg(pa + b) : 0u);
+            y = max(y, in ? __ldcg(pb + b) : 0u);
+        }
+        double u = t[0];
+#pragma unroll
+        for (int k = 1; k <= kCgMaxGrid / 32; ++k)
+            if (32 * k < (int)gridDim.x) u += t[k];
+        for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+        x = __reduce_max_sync(0xffffffffu, x);
+        y = __reduce_max_sync(0xffffffffu, y);
+        if (threadIdx.x == 0) fin(u, x, y);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double su = 0.0, sv = 0.0;
-        for (int w = 0; w < kPT / 32; ++w) {
-            su += sh[0][w];
-            sv += sh[1][w];
-        }
-        part[2 * blockIdx.x] = su;
-        part[2 * blockIdx.x + 1] = sv;
-    }
 }
 
-// CG scalars (device): s[0] = |f|^2, s[1 + (it & 1)] = r.z of iteration it, s[3] = p.Ap,
-// s[4] = r.r, s[5] = alpha.
-// Sums the dot partials in a fixed order. mode 0: s[3] = p.Ap. mode 1: s[1 + nxt] = r.z,
-// s[4] = r.r and done = (r.r <= tol^2 |f|^2), iters = it. mode 2: r.z and |f|^2 at the start.
-__global__ void __launch_bounds__(kPT)
-k_cg_scalars(const double *__restrict__ part, int nblk, double *s, int mode, int it,
-             double tol2, int *done, int *iters)
+// scale 2^(E - 32): the operator's factor for T in 1/64 of a grid unit
+__device__ __forceinline__ double cg_scale(double scale, int E)
 {
-    __shared__ double sh[2][kPT];
-    if (*(volatile const int *)done) return;
-    double u = 0.0, v = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += kPT) {
-        u += part[2 * b];
-        v += part[2 * b + 1];
-    }
-    sh[0][threadIdx.x] = u;
-    sh[1][threadIdx.x] = v;
-    __syncthreads();
-    for (int q = kPT / 2; q > 0; q >>= 1) {
-        if (threadIdx.x < q) {
-            sh[0][threadIdx.x] += sh[0][threadIdx.x + q];
-            sh[1][threadIdx.x] += sh[1][threadIdx.x + q];
+    const int e = E - 32 + 1023;
+    return e > 0 && e < 2047 ? scale * __hiloint2double(e << 20, 0) : ldexp(scale, E - 32);
+}
+
+// E with |y| < 2^E for |y| <= a + b c, from the high words of a and c (each at most 2^-20
+// above its value's truncation) and b >= 0
+__device__ __forceinline__ int cg_exponent(unsigned a, double b, unsigned c)
+{
+    const double x = __hiloint2double((int)a + 1, 0), y = __hiloint2double((int)c + 1, 0);
+    return bound_exponent(abs_hi_word(fma(b, y, x) * (1.0 + 0x1p-40)));
+}
+}  // namespace
+
+__global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgArgs g)
+{
+    extern __shared__ int2 sm[];
+    constexpr int R = kRadius, kU = 4, kL = 8, kWarps = kCgThreads / 32;
+    const unsigned nb = gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long nd = (long)g.n0 * g.n1 * g.n2, plane = (long)g.n0 * g.n1;
+    const long gt = (long)blockIdx.x * kCgThreads + tid, gs = (long)nb * kCgThreads;
+    CgState *s = g.s;
+    // sums and maxima of the phases: 0 p.Ap, 1 r.r and |r|, 2 |p|; each is written by its CTA
+    // and read by all after a barrier, and written again only two barriers later
+    double *part1 = g.part + kCgMaxGrid;
+    unsigned *pmax0 = g.pmax, *pmax1 = g.pmax + kCgMaxGrid, *pmax2 = g.pmax + 2 * kCgMaxGrid;
+    // the iteration's scalars; thread 0 writes them between barriers that all threads pass
+    // before they read or after they have read them
+    __shared__ struct {
+        double rr, ff, alpha, as, beta, sc, stop;  // sc: Ap = sc T; stop = tol^2 |f|^2
+        int E, done;
+    } S;
+    unsigned m, epoch = 0;
+    if (g.first == 0) {
+        // r = p = f, x = 0
+        double v = 0.0;
+        m = 0u;
+        for (long t = gt; t < nd; t += gs) {
+            const double f = g.f[t];
+            g.x[t] = 0.0;
+            g.r[t] = f;
+            g.p[t] = f;
+            v = fma(f, f, v);
+            m = max(m, abs_hi_word(f));
+        }
+        cg_put(v, m, part1 + blockIdx.x, pmax2 + blockIdx.x);
+        if (!grid_barrier(&s->bar, nb, epoch)) return;
+        cg_get(part1, pmax2, pmax2, [&](double u, unsigned x, unsigned) {
+            S.rr = S.ff = u;
+            S.stop = g.tol2 * u;
+            S.E = bound_exponent(x);
+            S.sc = cg_scale(g.scale, S.E);
+        });
+        if (S.rr == 0.0) {
+            if (gt == 0) s->ff = s->rr = 0.0, s->done = 1, s->iters = 0;
+            return;
+        }
+        for (long t = gt; t < nd; t += gs) g.q[t] = to_grid(g.p[t], S.E);
+        if (!grid_barrier(&s->bar, nb, epoch)) return;
+    } else {
+        if (tid == 0) {
+            S.rr = s->rr;
+            S.ff = s->ff;
+            S.stop = g.tol2 * S.ff;
+            S.E = s->E;
+            S.sc = cg_scale(g.scale, S.E);
         }
         __syncthreads();
     }
-    if (threadIdx.x != 0) return;
-    if (mode == 0) {
-        s[3] = sh[0][0];
-        s[5] = s[1 + (it & 1)] / s[3];
-    } else if (mode == 1) {
-        s[1 + ((it + 1) & 1)] = sh[0][0];
-        s[4] = sh[1][0];
-        *iters = it + 1;
-        if (s[4] <= tol2 * s[0]) *done = 1;
-    } else {
-        s[1] = sh[0][0];
-        s[0] = sh[1][0];
-        if (s[0] == 0.0) *done = 1;
+    const int gx = (g.n0 + kBr - 1) / kBr, gy = (g.n1 + kBr - 1) / kBr;
+    const int gz = (g.n2 + g.bz - 1) / g.bz;
+    const int nbrick = gx * gy * gz;
+    const int slab = kBrH * kBrH;                      // a plane with its halo
+    int2 *zc = sm + (long)slab * g.bz + R * kBr * kBr;  // columns; plane 0 (halo from -6 on)
+    int it = g.first, done = 0;
+    for (; it < g.last && !done; ++it) {
+        // ---- A: T = Ap / sc, Ap = -(1/4 pi) L_h p, and p.T
+        double v = 0.0;
+        for (int br = blockIdx.x; br < nbrick; br += nb) {
+            const int i0 = (br % gx) * kBr, j0 = (br / gx % gy) * kBr, k0 = br / (gx * gy) * g.bz;
+            const int bz = min(g.bz, g.n2 - k0);
+            __syncthreads();  // the previous brick's reads are done
+            auto at = [&](int i, int j, int k) -> int2 {
+                const bool in = i >= 0 && i < g.n0 && j >= 0 && j < g.n1 && k >= 0 && k < g.n2;
+                return in ? __ldcg(g.q + (i + (long)g.n0 * j + plane * k)) : make_int2(0, 0);
+            };
+            // rows of the brick with their x halo: a warp per row, 28 lanes (kL rows a trip, all
+            // their loads in flight); then, 16 lanes a row, the y halo and the z halo
+            for (int row0 = warp; row0 < bz * kBr; row0 += kL * kWarps) {
+                int2 w[kL];
+#pragma unroll
+                for (int u = 0; u < kL; ++u) {
+                    const int row = row0 + u * kWarps;
+                    w[u] = lane < kBrH && row < bz * kBr
+                               ? at(i0 - R + lane, j0 + row % kBr, k0 + row / kBr)
+                               : make_int2(0, 0);
+                }
+#pragma unroll
+                for (int u = 0; u < kL; ++u) {
+                    const int row = row0 + u * kWarps, y = row % kBr, z = row / kBr;
+                    if (lane < kBrH && row < bz * kBr) {
+                        sm[z * slab + (y + R) * kBrH + lane] = w[u];
+                        if (lane >= R && lane < R + kBr) zc[(z * kBr + y) * kBr + lane - R] = w[u];
+                    }
+                }
+            }
+            const int hx = tid % kBr, nyh = bz * 2 * R, nh = nyh + 2 * R * kBr;
+            for (int row0 = tid / kBr; row0 < nh; row0 += kL * (kCgThreads / kBr)) {
+                int2 w[kL];
+#pragma unroll
+                for (int u = 0; u < kL; ++u) {
+                    const int row = row0 + u * (kCgThreads / kBr);
+                    int y, z;  // the halo row in the brick's coordinates
+                    if (row < nyh) {
+                        z = row / (2 * R);
+                        y = row - z * (2 * R);
+                        y = y < R ? y - R : y - R + kBr;
+                    } else {
+                        z = (row - nyh) / kBr;
+                        y = (row - nyh) % kBr;
+                        z = z < R ? z - R : z - R + bz;
+                    }
+                    w[u] = row < nh ? at(i0 + hx, j0 + y, k0 + z) : make_int2(0, 0);
+                }
+#pragma unroll
+                for (int u = 0; u < kL; ++u) {
+                    const int row = row0 + u * (kCgThreads / kBr);
+                    if (row < nyh) {
+                        const int z = row / (2 * R), h = row - z * (2 * R);
+                        sm[z * slab + (h < R ? h : h + kBr) * kBrH + hx + R] = w[u];
+                    } else if (row < nh) {
+                        const int z = (row - nyh) / kBr, y = (row - nyh) % kBr;
+                        zc[((z < R ? z - R : z - R + bz) * kBr + y) * kBr + hx] = w[u];
+                    }
+                }
+            }
+            __syncthreads();
+            const int y = tid / kBr % kBr, zl = tid / (kBr * kBr);
+            if (i0 + hx < g.n0 && j0 + y < g.n1) {
+                constexpr int kZ = kCgThreads / (kBr * kBr);
+                const long o0 = (i0 + hx) + (long)g.n0 * (j0 + y) + plane * k0;
+                for (int z0 = zl; z0 < bz; z0 += kU * kZ) {
+                    double pv[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const int z = z0 + u * kZ;
+                        pv[u] = z < bz ? __ldcg(g.p + (o0 + plane * z)) : 0.0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const int z = z0 + u * kZ;
+                        if (z >= bz) break;
+                        const int2 *c = sm + z * slab + (y + R) * kBrH + hx + R;
+                        const int2 *cz = zc + (z * kBr + y) * kBr + hx;
+                        long long A = 0;
+                        float rs = 0.0f;
+#pragma unroll
+                        for (int r = R; r >= 1; --r) {
+                            const int2 xa = c[r], xb = c[-r], ya = c[r * kBrH], yb = c[-r * kBrH];
+                            const int2 za = cz[r * kBr * kBr], zb = cz[-r * kBr * kBr];
+                            const int sd = (xa.x + xb.x + ya.x) + (yb.x + za.x + zb.x);
+                            const float sr = ((__int_as_float(xa.y) + __int_as_float(xb.y)) +
+                                              (__int_as_float(ya.y) + __int_as_float(yb.y))) +
+                                             (__int_as_float(za.y) + __int_as_float(zb.y));
+                            A += (long long)g.W[r] * sd;
+                            rs = fmaf(g.Wf[r], sr, rs);
+                        }
+                        A += (long long)g.W[0] * c->x;
+                        rs = fmaf(g.Wf[0], __int_as_float(c->y), rs);
+                        // T in 1/64 of a unit (the r sum, below 2^25 units, fits 32 bits so)
+                        A = A * 64 + (long long)__float2int_rn(rs * 0x1p-26f);
+                        const double T = (double)A;
+                        g.Ap[o0 + plane * z] = T;
+                        v = fma(pv[u], T, v);
+                    }
+                }
+            }
+        }
+        cg_put(v, 0u, g.part + blockIdx.x, pmax0 + blockIdx.x);
+        if (!grid_barrier(&s->bar, nb, epoch)) return;
+        // ---- B: r -= alpha Ap, r.r, max |r|
+        cg_get(g.part, pmax0, pmax0, [&](double u, unsigned, unsigned) {
+            S.alpha = fast_quotient(S.rr, S.sc * u);
+            S.as = S.alpha * S.sc;
+        });
+        const double mas = -S.as;
+        v = 0.0;
+        m = 0u;
+        // (kU nodes a trip: their loads are in flight together)
+        for (long t0 = gt; t0 < nd; t0 += kU * gs) {
+            double a[kU], r[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const long t = t0 + u * gs;
+                a[u] = t < nd ? __ldcg(g.Ap + t) : 0.0;
+                r[u] = t < nd ? g.r[t] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const long t = t0 + u * gs;
+                if (t >= nd) break;
+                const double x = fma(mas, a[u], r[u]);
+                g.r[t] = x;
+                v = fma(x, x, v);
+                m = max(m, abs_hi_word(x));
+            }
+        }
+        cg_put(v, m, part1 + blockIdx.x, pmax1 + blockIdx.x);
+        if (!grid_barrier(&s->bar, nb, epoch)) return;
+        // ---- C: x += alpha p, p = r + beta p
+        cg_get(part1, pmax1, pmax2, [&](double u, unsigned maxr, unsigned maxp) {
+            S.beta = fast_quotient(u, S.rr);
+            S.rr = u;
+            S.done = !(u > S.stop);  // converged, or not a number
+            S.E = cg_exponent(maxr, S.beta, maxp);
+            S.sc = cg_scale(g.scale, S.E);
+        });
+        const double alpha = S.alpha, beta = S.beta;
+        const int E = S.E;
+        done = S.done;
+        m = 0u;
+        for (long t0 = gt; t0 < nd; t0 += kU * gs) {
+            double po[kU], x[kU], r[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const long t = t0 + u * gs;
+                po[u] = t < nd ? g.p[t] : 0.0;
+                x[u] = t < nd ? g.x[t] : 0.0;
+                r[u] = t < nd ? g.r[t] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const long t = t0 + u * gs;
+                if (t >= nd) break;
+                g.x[t] = fma(alpha, po[u], x[u]);
+                const double pn = fma(beta, po[u], r[u]);
+                g.p[t] = pn;
+                g.q[t] = to_grid(pn, E);
+                m = max(m, abs_hi_word(pn));
+            }
+        }
+        if (done) continue;
+        if (!grid_barrier(&s->bar, nb, epoch)) return;
+        // (after the barrier: other CTAs were reading the last maxima before it)
+        cg_put_max(m, pmax2 + blockIdx.x);
+    }
+    if (gt == 0) {
+        s->ff = S.ff;
+        s->rr = S.rr;
+        s->E = S.E;
+        s->done = done;
+        s->iters = it;
     }
 }
 
-// x += alpha p, r -= alpha Ap, z = r / diag.
-__global__ void __launch_bounds__(kPT)
-k_cg_update(double *__restrict__ x, double *__restrict__ r, double *__restrict__ z,
-            const double *__restrict__ p, const double *__restrict__ Ap, long n, double idiag,
-            const double *s, const int *done)
+namespace {
+long pois_partials(long nd)
 {
-    if (*(volatile const int *)done) return;
-    const double alpha = s[5];
-    for (long t = (long)blockIdx.x * kPT + threadIdx.x; t < n; t += (long)gridDim.x * kPT) {
-        x[t] = fma(alpha, p[t], x[t]);
-        const double rt = fma(-alpha, Ap[t], r[t]);
-        r[t] = rt;
-        z[t] = rt * idiag;
-    }
+    const long nblk = (nd + (long)kPT * kMomPer - 1) / ((long)kPT * kMomPer);
+    const long cg = 3 * kCgMaxGrid + (3 * kCgMaxGrid + 1) / 2;
+    return nblk * kNQ > cg ? nblk * kNQ : cg;
 }
-
-// p = z + beta p, beta = (r.z)_new / (r.z)_old.
-__global__ void __launch_bounds__(kPT)
-k_cg_direction(double *__restrict__ p, const double *__restrict__ z, long n, const double *s,
-               int it, const int *done)
-{
-    if (*(volatile const int *)done) return;
-    const double beta = s[1 + ((it + 1) & 1)] / s[1 + (it & 1)];
-    for (long t = (long)blockIdx.x * kPT + threadIdx.x; t < n; t += (long)gridDim.x * kPT)
-        p[t] = fma(beta, p[t], z[t]);
-}
-
-// r = f, z = f / diag, p = z, x = 0.
-__global__ void __launch_bounds__(kPT)
-k_cg_init(const double *__restrict__ f, double *__restrict__ x, double *__restrict__ r,
-          double *__restrict__ z, double *__restrict__ p, long n, double idiag)
-{
-    for (long t = (long)blockIdx.x * kPT + threadIdx.x; t < n; t += (long)gridDim.x * kPT) {
-        const double v = f[t];
-        x[t] = 0.0;
-        r[t] = v;
-        z[t] = v * idiag;
-        p[t] = v * idiag;
-    }
-}
+}  // namespace
 
 size_t poisson_workspace(int n0, int n1, int n2, int radius)
 {
     const long nd = (long)n0 * n1 * n2;
     const long ne = (long)(n0 + 2 * radius) * (n1 + 2 * radius) * (n2 + 2 * radius);
     const long nshell = 2L * radius * ((long)n1 * n2 + (long)n0 * n2 + (long)n0 * n1);
-    const long nblk = (nd + kPT - 1) / kPT;
-    const long nparts = nblk * kNQ > 2L * kVecGrid ? nblk * kNQ : 2L * kVecGrid;
-    // b, rhs, r, z, p, Ap; V_ext; shell; partials; Q (49) + scalars (8)
-    return sizeof(double) * (size_t)(6 * nd + ne + nshell + nparts + kNQ + 8) + 2 * sizeof(int);
+    // b, rhs, r, q, p, Ap; V_ext; shell; partials; Q (49); the CG state
+    return sizeof(double) * (size_t)(6 * nd + ne + nshell + pois_partials(nd) + kNQ) +
+           sizeof(CgState) + 64;
+}
+
+// Brick height: bricks one CTA takes per iteration x (its nodes + the halo's loads), fewest
+// node-times, within the shared memory.
+static int cg_brick_height(int n0, int n1, int n2)
+{
+    const long t = (long)((n0 + kBr - 1) / kBr) * ((n1 + kBr - 1) / kBr);
+    long best = -1;
+    int bz = 1;
+    for (int z = 1; z <= n2 && cg_smem(z) <= kCgSmemMax; ++z) {
+        const long per = (t * ((n2 + z - 1) / z) + kCgMaxGrid - 1) / kCgMaxGrid;
+        const long cost = per * (kBrH * kBrH * (long)z + 2 * kRadius * kBr * kBr + 1024);
+        if (best < 0 || cost < best) best = cost, bz = z;
+    }
+    return bz;
 }
 
 cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int natoms,
@@ -421,11 +687,11 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
     const long ne = (long)(n0 + 2 * Rr) * (n1 + 2 * Rr) * (n2 + 2 * Rr);
     const long nshell = 2L * Rr * ((long)n1 * n2 + (long)n0 * n2 + (long)n0 * n1);
     const long nblk = (nd + kPT - 1) / kPT;
-    const long nparts = nblk * kNQ > 2L * kVecGrid ? nblk * kNQ : 2L * kVecGrid;
+    const long nmom = (nd + (long)kPT * kMomPer - 1) / ((long)kPT * kMomPer);
     double *w = (double *)ws;
-    double *b = w, *rhs = b + nd, *r = rhs + nd, *z = r + nd, *p = z + nd, *Ap = p + nd;
-    double *Ve = Ap + nd, *pe = Ve + ne, *part = pe + nshell, *Q = part + nparts, *s = Q + kNQ;
-    int *done = (int *)(s + 8), *iters = done + 1;
+    double *b = w, *rhs = b + nd, *r = rhs + nd, *q = r + nd, *p = q + nd, *Ap = p + nd;
+    double *Ve = Ap + nd, *pe = Ve + ne, *part = pe + nshell, *Q = part + pois_partials(nd);
+    CgState *cs = (CgState *)(((uintptr_t)(Q + kNQ) + 15) & ~(uintptr_t)15);
 
     PoisCoef pc;
     for (int q = 0; q <= kRadius; ++q) pc.w[q] = H.w[q];
@@ -443,7 +709,6 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
             pc.N[l * l + l - m] = nlm;
         }
     }
-    const double idiag = 1.0 / (-kInv4Pi * 6.0 * H.w[0]);
     cudaError_t e;
     // pseudocharge, moments, boundary values, right-hand side
     k_vext<<<(unsigned)((ne + kPT - 1) / kPT), kPT, 0, st>>>(Ve, n0 + 2 * Rr, n1 + 2 * Rr,
@@ -452,9 +717,9 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
     note_launch();
     k_pseudocharge<<<(unsigned)nblk, kPT, 0, st>>>(Ve, b, n0, n1, n2, pc);
     note_launch();
-    k_moments<<<(unsigned)nblk, kPT, 0, st>>>(rho, b, n0, n1, n2, pc, part);
+    k_moments<<<(unsigned)nmom, kPT, 0, st>>>(rho, b, n0, n1, n2, pc, part);
     note_launch();
-    k_sum_partials<<<1, kPT, 0, st>>>(part, (int)nblk, kNQ, H.h * H.h * H.h, Q);
+    k_sum_partials<<<kNQ, kPT, 0, st>>>(part, (int)nmom, kNQ, H.h * H.h * H.h, Q);
     note_launch();
     k_phi_ext<<<(unsigned)((nshell + kPT - 1) / kPT), kPT, 0, st>>>(pe, n0, n1, n2, pc, Q,
                                                                     nshell);
@@ -467,43 +732,61 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
             return e;
     }
     // CG from phi = 0
-    const unsigned gv = kVecGrid;
-    if ((e = cudaMemsetAsync(done, 0, 2 * sizeof(int), st)) != cudaSuccess) return e;
-    k_cg_init<<<gv, kPT, 0, st>>>(rhs, phi, r, z, p, nd, idiag);
-    note_launch();
-    k_dot2<<<gv, kPT, 0, st>>>(r, z, rhs, nd, part, done);
-    note_launch();
-    k_cg_scalars<<<1, kPT, 0, st>>>(part, gv, s, 2, 0, tol * tol, done, iters);
-    note_launch();
-    int done_h = 0, it_h = 0;
-    const int kBatch = 16;  // iterations between host checks of the done flag
-    for (int it = 0; it < maxit; ++it) {
-        k_poisson_apply<<<(unsigned)nblk, kPT, 0, st>>>(p, Ap, n0, n1, n2, pc, done);
-        k_dot2<<<gv, kPT, 0, st>>>(p, Ap, nullptr, nd, part, done);
-        k_cg_scalars<<<1, kPT, 0, st>>>(part, gv, s, 0, it, 0.0, done, iters);
-        k_cg_update<<<gv, kPT, 0, st>>>(phi, r, z, p, Ap, nd, idiag, s, done);
-        k_dot2<<<gv, kPT, 0, st>>>(r, z, r, nd, part, done);
-        k_cg_scalars<<<1, kPT, 0, st>>>(part, gv, s, 1, it, tol * tol, done, iters);
-        k_cg_direction<<<gv, kPT, 0, st>>>(p, z, nd, s, it, done);
-        for (int q = 0; q < 7; ++q) note_launch();
-        if ((it + 1) % kBatch == 0 || it + 1 == maxit) {
-            if ((e = cudaMemcpyAsync(&done_h, done, sizeof(int), cudaMemcpyDeviceToHost, st)) !=
-                cudaSuccess)
-                return e;
-            if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-            if (done_h) break;
-        }
+    CgArgs g;
+    g.x = phi;
+    g.r = r;
+    g.p = p;
+    g.Ap = Ap;
+    g.q = (int2 *)q;
+    g.f = rhs;
+    g.part = part;
+    g.pmax = (unsigned *)(part + 3 * kCgMaxGrid);
+    g.s = cs;
+    g.n0 = n0;
+    g.n1 = n1;
+    g.n2 = n2;
+    g.bz = cg_brick_height(n0, n1, n2);
+    for (int t = 0; t <= kRadius; ++t) {
+        g.W[t] = H.wint[t];
+        g.Wf[t] = (float)H.wint[t];
     }
-    double sc[8];
-    if ((e = cudaMemcpyAsync(sc, s, sizeof(sc), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&it_h, iters, sizeof(int), cudaMemcpyDeviceToHost, st)) !=
-            cudaSuccess ||
-        (e = cudaMemcpyAsync(&done_h, done, sizeof(int), cudaMemcpyDeviceToHost, st)) !=
-            cudaSuccess)
-        return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    *iters_host = it_h;
-    *relres_host = sc[0] > 0.0 ? sqrt(sc[4] / sc[0]) : 0.0;
+    g.scale = -kInv4Pi * H.wunit;
+    g.tol2 = tol * tol;
+    static std::atomic<int> sms{0};  // set once (several host threads may launch)
+    if (!sms.load(std::memory_order_acquire)) {
+        int dev = 0, n = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+            return e;
+        if ((e = cudaFuncSetAttribute(k_cg, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kCgSmemMax)) != cudaSuccess)
+            return e;
+        sms.store(n, std::memory_order_release);
+    }
+    // enough CTAs for the bricks, and for the vector phases (four nodes per thread)
+    const long bricks = (long)((n0 + kBr - 1) / kBr) * ((n1 + kBr - 1) / kBr) * ((n2 + g.bz - 1) / g.bz);
+    const long vec = (nd + 4 * kCgThreads - 1) / (4 * kCgThreads);
+    const int grid = (int)std::min<long>(std::min(kCgMaxGrid, sms.load(std::memory_order_acquire)),
+                                         std::max(bricks, vec));
+    if ((e = cudaMemsetAsync(cs, 0, sizeof(CgState), st)) != cudaSuccess) return e;
+    CgState h;
+    for (int it = 0; it < maxit; it += kCgPerLaunch) {
+        g.first = it;
+        g.last = maxit - it < kCgPerLaunch ? maxit : it + kCgPerLaunch;
+        if ((e = cudaMemsetAsync(&cs->bar, 0, sizeof(GridBarrier), st)) != cudaSuccess) return e;
+        void *args[] = {&g};
+        e = cudaLaunchCooperativeKernel((const void *)k_cg, dim3(grid), dim3(kCgThreads), args,
+                                        (size_t)cg_smem(g.bz), st);
+        note_launch();
+        if (e != cudaSuccess) return e;
+        if ((e = cudaMemcpyAsync(&h, cs, sizeof h, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+            return e;
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        if (h.done || h.bar.err) break;
+    }
+    *iters_host = h.iters;
+    // a barrier that gave up counts as no convergence
+    *relres_host = h.bar.err ? INFINITY : h.ff > 0.0 ? std::sqrt(h.rr / h.ff) : h.rr;
     return cudaGetLastError();
 }
 

@@ -43,4 +43,13 @@ __device__ __forceinline__ double fast_reciprocal(double d)
     return y * __hiloint2double((2046 - e) << 20, 0);
 }
 
+// a / b to about an ulp (a short chain; b as for fast_reciprocal, else a plain division)
+__device__ __forceinline__ double fast_quotient(double a, double b)
+{
+    const double y = fast_reciprocal(fabs(b));
+    const double q = a * y, d = fabs(b);
+    const double z = isfinite(q) ? fma(y, fma(-q, d, a), q) : q;
+    return b < 0.0 ? -z : z;
+}
+
 }  // namespace sparc

@@ -52,39 +52,6 @@ struct FxCoef {
     double alpha, shift;  // the general form's potential factor
 };
 
-// A value on the column's grid: .x = d, .y = the bits of r (y 2^(26-E) = d + 2^-32 r, |y| < 2^E).
-// With the significand at the top of 64 bits, y = (h:l) 2^(e-1086), N = (h:l) >> s with s =
-// 1028 + E - e (s >= 6 when |y| < 2^E) is |y| 2^(58-E): its high word is d (below 2^26), its low
-// word, rounded to FP32, r. Zero and subnormal y give 0; the sign is applied to both parts. The
-// rounding matters: a truncated y has an error of y's own sign, which in the potential term
-// (unlike in the Laplacian, whose weights sum to zero) does not cancel and which the filter
-// amplifies (10 times the error of a degree-20 filter with 23 truncated bits).
-__device__ __forceinline__ int2 grid_parts(unsigned h, unsigned l, int s, unsigned sign)
-{
-    const unsigned long long N = (((unsigned long long)h << 32) | l) >> min(s, 63);
-    const int sm = (int)sign >> 31;  // 0 or -1
-    const int d = ((int)(unsigned)(N >> 32) ^ sm) - sm;
-    const float r = __uint2float_rn((unsigned)N);
-    return make_int2(d, (int)(__float_as_uint(r) | (sign & 0x80000000u)));
-}
-
-__device__ __forceinline__ int2 to_grid(double y, int E)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(y);
-    const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
-    const int e = (int)((hw >> 20) & 0x7ffu);
-    const unsigned h = e ? __funnelshift_l(lw, hw, 11) | 0x80000000u : 0u;
-    return grid_parts(h, e ? lw << 11 : 0u, 1028 + E - e, hw);
-}
-
-// FP32 input: y = (h:0) 2^(e-190).
-__device__ __forceinline__ int2 to_grid(float y, int E)
-{
-    const unsigned u = __float_as_uint(y);
-    const int e = (int)((u >> 23) & 0xffu);
-    return grid_parts(e ? (u << 8) | 0x80000000u : 0u, 0u, 132 + E - e, u);
-}
-
 __device__ __forceinline__ double as_f64(double y) { return y; }
 __device__ __forceinline__ double as_f64(float y) { return (double)y; }
 

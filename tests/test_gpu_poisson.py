@@ -115,3 +115,27 @@ def test_poisson_full_size_cluster96():
     got = phi.cpu().numpy()
     assert np.max(np.abs(got - ref)) <= 1e-6 * np.max(np.abs(ref))
     ctx.close()
+
+
+@pytest.mark.parametrize("n3,radius", [((7, 5, 9), 6), ((16, 17, 33), 6), ((50, 3, 18), 6),
+                                       ((33, 48, 64), 4), ((1, 1, 40), 6)])
+def test_poisson_brick_edges(n3, radius):
+    # grids below, at and beyond the operator's 16 x 16 bricks, thinner than the halo, and a
+    # smaller stencil radius (zero outer weights). The operator's grid form is scaled by a power
+    # of two from p's magnitude, so a density times 2^40 must take the same iterations and
+    # give the same potential times 2^40, bit for bit; at radius 6 the oracle's CG is the
+    # reference (tolerance as above).
+    h = 0.35
+    nd = n3[0] * n3[1] * n3[2]
+    g = np.random.default_rng(nd)
+    rho = g.uniform(0.0, 1.0, nd)
+    ctx = sparc.Context(n3, h, None, None, None, veff=np.zeros(nd), radius=radius)
+    phi, it, rel = ctx.poisson(torch.from_numpy(rho).to(DEV), tol=1e-12)
+    assert rel <= 1e-12
+    big = ctx.poisson(torch.from_numpy(rho * 2.0 ** 40).to(DEV), tol=1e-12)
+    assert big[1] == it and torch.equal(big[0], phi * 2.0 ** 40)   # exact scaling by 2^40
+    if radius == 6:
+        ref, _, _ = P.poisson_solve(rho, n3, h, np.zeros((0, 3)), np.zeros(0), 1.0, tol=1e-13)
+        got = phi.cpu().numpy()
+        assert np.max(np.abs(got - ref)) <= 1e-8 * np.max(np.abs(ref))
+    ctx.close()
