@@ -29,7 +29,7 @@ constexpr int kDefaultVariant = kTmaItemForm * 3;  // TMA, one CTA per item, who
 
 // Persistent grids: enough resident CTAs to fill the 152 SMs several times.
 constexpr int kGridStencil = 152 * 8;
-constexpr int kGridTma = 152 * 3;
+constexpr int kGridTma = 152 * 4;
 constexpr int kGridProject = 152 * 2;
 constexpr int kGridScatter = 152 * 6;
 

@@ -168,9 +168,11 @@ constexpr int kBatchNodes = 256;   // covered nodes per scatter work item
 cudaError_t stencil_f32(const DevHam &H, const float *Y, const float *Yprev, float *out,
                         int ncols, long ld, double alpha, double shift, double beta,
                         cudaStream_t st);
-void stencil_z_split(int n2, long tiles, int ncols, int &nzc, int &zchunk);
 // stencil_tma.cu: TMA-fed FP32 step for shapes with n0, ld multiples of 4 and 16-byte
-// aligned blocks (stencil_tma_ok); stencil_f32 picks it when it applies.
+// aligned blocks (stencil_tma_ok); stencil_f32 picks it when it applies, else the same step
+// fed by 4-byte asynchronous copies.
+cudaError_t stencil_f32_copy(const DevHam &H, const float *Y, const float *Yprev, float *out,
+                             int ncols, long ld, const StepCoef<float> &cf, cudaStream_t st);
 bool stencil_tma_ok(const DevHam &H, const void *Y, const void *Yprev, const void *out, long ld);
 cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev, float *out,
                             int ncols, long ld, const StepCoef<float> &cf, int *err,

@@ -137,19 +137,6 @@ __device__ __forceinline__ void stencil_tile(const T *__restrict__ Yc, const TO 
     }
 }
 
-template <typename T, typename TO, typename TC, int BX, int BY>
-__global__ void __launch_bounds__(BX *BY)
-k_stencil(const T *Y, const TO *Yprev, TO *out, const TC *__restrict__ V, int n0, int n1, int n2,
-          long ld, int nzc, int zchunk, StepCoef<TC> cf)
-{
-    const int col = blockIdx.z / nzc;
-    const int k0 = (blockIdx.z % nzc) * zchunk;
-    const int k1 = min(n2, k0 + zchunk);
-    stencil_tile<T, TO, TC, BX, BY>(Y + (long)col * ld, Yprev ? Yprev + (long)col * ld : nullptr,
-                                    out + (long)col * ld, V, n0, n1, n2, blockIdx.x * BX,
-                                    blockIdx.y * BY, k0, k1, cf);
-}
-
 // Work-list form for a batch of clusters: each CTA walks the items (cluster, column, tile,
 // z range) with a grid stride; a cluster's pointers, sizes and step coefficients come from
 // its BatchStencil entry.
@@ -165,35 +152,6 @@ k_batch_stencil(const BatchItem *__restrict__ items, int nitems, const BatchSten
                                                   C.out + off, C.V, C.n0, C.n1, C.n2, w.a * BX,
                                                   w.b * BY, w.k0, w.k1, C.cf);
     }
-}
-
-// Picks the number of z-chunks so that small problems still fill the 152 SMs.
-void stencil_z_split(int n2, long tiles, int ncols, int &nzc, int &zchunk)
-{
-    const long want = 152L * 8;
-    long per = tiles * ncols;
-    nzc = 1;
-    while (per * nzc < want && n2 / (nzc * 2) >= 16) nzc *= 2;
-    while ((long)nzc * ncols > 65535) nzc /= 2;
-    if (nzc < 1) nzc = 1;
-    zchunk = (n2 + nzc - 1) / nzc;
-}
-
-template <typename T, typename TO, typename TC>
-static cudaError_t launch(const DevHam &H, const T *Y, const TO *Yprev, TO *out, const TC *V,
-                          int ncols, long ld, const StepCoef<double> &cd, cudaStream_t st)
-{
-    constexpr int BX = 32, BY = 8;
-    if (ncols <= 0) return cudaSuccess;
-    if (ncols > 65535) return cudaErrorInvalidValue;
-    const int gx = (H.n0 + BX - 1) / BX, gy = (H.n1 + BY - 1) / BY;
-    int nzc, zchunk;
-    stencil_z_split(H.n2, (long)gx * gy, ncols, nzc, zchunk);
-    dim3 grid(gx, gy, ncols * nzc), block(BX, BY);
-    k_stencil<T, TO, TC, BX, BY><<<grid, block, 0, st>>>(Y, Yprev, out, V, H.n0, H.n1, H.n2,
-                                                         ld, nzc, zchunk, cast_coef<TC>(cd));
-    note_launch();
-    return cudaGetLastError();
 }
 
 int batch_stencil_shapes() { return 3; }
@@ -227,10 +185,9 @@ cudaError_t stencil_f32(const DevHam &H, const float *Y, const float *Yprev, flo
                         cudaStream_t st)
 {
     if (stencil_tma_ok(H, Y, Yprev, out, ld))
-        return stencil_f32_tma(H, Y, Yprev, out, ncols, ld,
-                               cast_coef<float>(make_coef(H, alpha, shift, beta)), H.err, st);
-    return launch<float, float, float>(H, Y, Yprev, out, H.Vf, ncols, ld,
-                                       make_coef(H, alpha, shift, beta), st);
+        return stencil_f32_tma(H, Y, Yprev, out, ncols, ld, coef_f32(H, alpha, shift, beta),
+                               H.err, st);
+    return stencil_f32_copy(H, Y, Yprev, out, ncols, ld, coef_f32(H, alpha, shift, beta), st);
 }
 
 }  // namespace sparc

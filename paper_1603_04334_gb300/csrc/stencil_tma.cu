@@ -18,8 +18,8 @@
 // plane. The arithmetic runs on packed FP32 pairs (two nodes per add or fused
 // multiply-add), each operation rounded as the scalar form would round it, and the plane
 // loop is unrolled 13 times, one copy per rotation of the queue, so the queue is never
-// shifted. The queue needs planes t .. t+6 of the ring, so with kStages = 10 the loads run
-// 3 planes ahead of the compute.
+// shifted. The queue needs planes t .. t+6 of the ring, so with kStages = 9 the loads run
+// 2 planes ahead of the compute.
 //
 // Y_{j-1} (one third of the step's traffic) rides in the same ring: the TMA load that
 // brings plane t of Y also brings the halo-free tile of Y_{j-1} at the plane whose compute
@@ -27,11 +27,12 @@
 // step is an asynchronous bulk copy. V_eff (one plane shared by all columns, L2-resident)
 // is prefetched into registers two planes ahead.
 //
-// Requirements (checked on the host, else the plain kernel of stencil.cu runs): n0 and ld
+// Requirements (checked on the host, else k_stencil_f32_copy runs): n0 and ld
 // multiples of 4 and 16-byte aligned block pointers (TMA strides and float4 accesses).
 #include "internal.cuh"
 
 #include <atomic>
+#include <type_traits>
 #include "tma.cuh"
 
 #include <cudaTypedefs.h>
@@ -45,10 +46,16 @@ constexpr int kBX = 4 * kTX; // 32 nodes along x
 constexpr int kR = kRadius;  // 6
 constexpr int kW = kBX + 16; // box width: 8 left (aligned) + 32 + 8 right
 constexpr int kH = kTY + 2 * kR;
-constexpr int kStages = 10;
+constexpr int kStages = 9;
+// Y_{j-1} tiles: one arrives with plane t and is used when that plane enters the z queue, kPrev
+// steps after it was issued (a plane stays kR steps longer), so they need fewer slots
+constexpr int kPrev = kStages - kR;
 constexpr int kPlaneBytes = kW * kH * 4;   // Y plane with halo
 constexpr int kTileBytes = kBX * kTY * 4;  // Y_{j-1} tile, no halo
-constexpr int kStageFloats = kW * kH + kBX * kTY;
+constexpr int kStageFloats = kW * kH;
+constexpr int kTileFloats = kBX * kTY;
+// 54.5 KB: four CTAs (16 warps) per SM; with a tile slot in each of ten stages it was three
+constexpr int kSmemBytes = kStages * kPlaneBytes + kPrev * kTileBytes;
 constexpr unsigned kWaitLimit = 1u << 22;
 }  // namespace
 
@@ -119,6 +126,7 @@ struct TmaThread {
     int i0, j0, k0, col;
     int sc;         // stage of the compute plane tc
     int sn;         // stage of plane tc + 6 (its centre enters the queue)
+    int sp;         // slot of its Y_{j-1} tile
     unsigned pn;    // parity of plane tc + 6's current use of its stage
     int tc;         // current compute plane
     int ty, tx, tid;
@@ -134,7 +142,9 @@ __device__ __forceinline__ void tma_issue(TmaThread &s, int t)
     float *dst = s.sm + (long)st * kStageFloats;
     mbar_arrive_expect_tx(&s.full[st], kPlaneBytes + (p ? kTileBytes : 0));
     tma_load_4d(dst, s.tmY, &s.full[st], s.i0 - 8, s.j0 - kR, s.k0 - kR + t, s.col);
-    if (p) tma_load_4d(dst + kH * kW, s.tmP, &s.full[st], s.i0, s.j0, s.k0 - 2 * kR + t, s.col);
+    if (p)
+        tma_load_4d(s.sm + kStages * kStageFloats + t % kPrev * kTileFloats, s.tmP, &s.full[st],
+                    s.i0, s.j0, s.k0 - 2 * kR + t, s.col);
 }
 
 template <int PH>
@@ -152,8 +162,8 @@ __device__ __forceinline__ bool plane_step(TmaThread &s, float4 (&q)[2 * kR + 1]
     plane_math<PH>(row, q, vv, cf, aA, aB);
     if (s.act && got) {
         if (s.hasP) {
-            const float4 pv =
-                *reinterpret_cast<const float4 *>(stn + kH * kW + s.ty * kBX + 4 * s.tx);
+            const float4 pv = *reinterpret_cast<const float4 *>(
+                s.sm + kStages * kStageFloats + s.sp * kTileFloats + s.ty * kBX + 4 * s.tx);
             aA = __ffma2_rn(cf.nbeta, lo2(pv), aA);
             aB = __ffma2_rn(cf.nbeta, hi2(pv), aB);
         }
@@ -170,6 +180,7 @@ __device__ __forceinline__ bool plane_step(TmaThread &s, float4 (&q)[2 * kR + 1]
         s.sn = 0;
         s.pn ^= 1u;
     }
+    if (++s.sp == kPrev) s.sp = 0;
     ++s.k;
     ++s.tc;
     s.p += s.plane;
@@ -180,12 +191,12 @@ __device__ __forceinline__ bool plane_step(TmaThread &s, float4 (&q)[2 * kR + 1]
 // after the barrier that ends the compute of plane tc, it refills that plane's stage with
 // plane tc + kStages. The plane loop is unrolled 13 times, one copy per rotation of the z
 // queue, so the queue is never shifted.
-__global__ void __launch_bounds__(kTX *kTY)
+__global__ void __launch_bounds__(kTX *kTY, 4)
 k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmP,
                   bool hasP, float *out, const float *__restrict__ V, int n0, int n1, int n2,
                   long ld, int nzc, int zchunk, StepCoef2 cf, int *err)
 {
-    // stage s: Y plane [kH][kW] then the Y_{j-1} tile [kTY][kBX]
+    // kStages Y planes [kH][kW], then kPrev Y_{j-1} tiles [kTY][kBX]
     extern __shared__ __align__(128) float sm[];
     __shared__ __align__(8) uint64_t full[kStages];
     __shared__ int timed_out;
@@ -246,6 +257,7 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
     s.sc = kR % kStages;
     s.sn = (2 * kR) % kStages;
     s.pn = (unsigned)(((2 * kR) / kStages) & 1);
+    s.sp = (2 * kR) % kPrev;
     s.tc = kR;
     float4 vv = make_float4(0.f, 0.f, 0.f, 0.f), v1 = vv;
     if (s.act) vv = *reinterpret_cast<const float4 *>(V + s.p);
@@ -278,6 +290,172 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
     }
 }
 
+// The same step for rows that TMA cannot address (n0 or ld not a multiple of 4, a block off a
+// 16-byte boundary): the ring is filled by 4-byte asynchronous copies (cp.async, zero-filled
+// outside the grid) that consecutive lanes issue along rows, and the output row goes through
+// shared memory so that its stores are consecutive too; the arithmetic and the queue are
+// those of k_stencil_f32_tma, plane by plane. One barrier per plane: it follows the wait for
+// this thread's copies of the step's planes and precedes the copies into the stage that the
+// previous step released. Bound by latency (about 80 thread instructions a node slot, issue
+// 46% busy at 12 warps per SM) where the row-per-thread
+// kernel it replaces needed 207: 75 x 61 x 53 x 40, 92 us -> 84 us a step.
+namespace {
+constexpr int kWarpsC = kTX * kTY / 32;
+}
+
+__device__ __forceinline__ void copy4(float *dst, const float *src, bool in)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(in ? 4 : 0)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(kTX *kTY, 4)
+k_stencil_f32_copy(const float *Yb, const float *Pb, float *out, const float *__restrict__ V,
+                   int n0, int n1, int n2, long ld, int nzc, int zchunk, StepCoef2 cf)
+{
+    extern __shared__ __align__(128) float sm[];
+    float *const prev = sm + kStages * kStageFloats;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kTX + tx;
+    const int lane = tid & 31, warp = tid >> 5;
+    const int i0 = blockIdx.x * kBX, j0 = blockIdx.y * kTY;
+    const int col = blockIdx.z / nzc;
+    const int k0 = (blockIdx.z % nzc) * zchunk, k1 = min(n2, k0 + zchunk);
+    const unsigned plane = (unsigned)n0 * (unsigned)n1;
+    const float *Y = Yb + (long)col * ld;
+    const float *P = Pb ? Pb + (long)col * ld : nullptr;
+    float *O = out + (long)col * ld;
+    // plane z of Y into stage st: the 32 columns of the tile for all 28 rows, a warp per row,
+    // then the 6 columns left and right of its 16 rows
+    const bool xin = i0 + lane < n0;
+    auto copy_plane = [&](int z, int st) {
+        const bool zin = z >= 0 && z < n2;
+        const float *src = Y + (zin ? (unsigned)z * plane : 0u);
+        float *dst = sm + st * kStageFloats;
+#pragma unroll
+        for (int u = 0; u < kH / kWarpsC; ++u) {
+            const int r = warp + u * kWarpsC, j = j0 - kR + r;
+            const bool in = zin && xin && j >= 0 && j < n1;
+            copy4(dst + r * kW + 8 + lane, src + (in ? (unsigned)(i0 + lane) + (unsigned)n0 * (unsigned)j : 0u), in);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int e = tid + u * kTX * kTY;
+            if (e < 2 * kR * kTY) {
+                const int r = e / (2 * kR), h = e - r * (2 * kR);
+                const int x = h < kR ? h - kR : h - kR + kBX, i = i0 + x, j = j0 + r;
+                const bool in = zin && i >= 0 && i < n0 && j < n1;
+                copy4(dst + (kR + r) * kW + 8 + x, src + (in ? (unsigned)i + (unsigned)n0 * (unsigned)j : 0u), in);
+            }
+        }
+    };
+    auto copy_prev = [&](int z, int slot) {
+        float *dst = prev + slot * kTileFloats;
+#pragma unroll
+        for (int u = 0; u < kTY / kWarpsC; ++u) {
+            const int r = warp + u * kWarpsC, j = j0 + r;
+            const bool in = xin && j < n1;
+            copy4(dst + r * kBX + lane,
+                  P + (in ? (unsigned)(i0 + lane) + (unsigned)n0 * (unsigned)j + (unsigned)z * plane : 0u), in);
+        }
+    };
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    // planes are numbered from k0 - 6; plane t goes to stage t % kStages, the Y_{j-1} tile of
+    // step t (compute plane t) to slot t % kPrev. Step t starts with planes t .. t + 6 and its
+    // tile present and issues plane t - 1 + kStages and the tile of step t + kPrev - 1.
+    const int T = (k1 - k0) + 2 * kR;
+    for (int t = 0; t < kStages; ++t) copy_plane(k0 - kR + t, t);  // (T >= 13)
+    commit();
+    const float *vp = V + ((unsigned)min(i0 + 4 * tx, n0 - 1) + (unsigned)n0 * (unsigned)min(j0 + ty, n1 - 1));
+    const int nv = min(n0 - 1 - min(i0 + 4 * tx, n0 - 1), 3);  // further nodes of the row
+    auto load_v = [&](int z) {
+        const float *q = vp + (unsigned)z * plane;
+        float4 v;
+        v.x = q[0];
+        v.y = q[min(1, nv)];
+        v.z = q[min(2, nv)];
+        v.w = q[nv];
+        return v;
+    };
+    float4 q[2 * kR + 1];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    auto center = [&](int st) {
+        return *reinterpret_cast<const float4 *>(sm + st * kStageFloats + (kR + ty) * kW + 8 + 4 * tx);
+    };
+    // planes 0 .. 5 only feed the queue: their stages take the planes up to 12, which step 6
+    // needs, and 13, with the first two tiles
+#pragma unroll
+    for (int t = 0; t < kStages; ++t) q[t] = center(t);
+    __syncthreads();
+    for (int t = kStages; t <= 2 * kR; ++t) copy_plane(k0 - kR + t, t % kStages);
+    if (P) copy_prev(k0, kR % kPrev);
+    commit();
+    if (2 * kR + 1 < T) copy_plane(k0 + kR + 1, (2 * kR + 1) % kStages);
+    if (P && k0 + 1 < k1) copy_prev(k0 + 1, (kR + 1) % kPrev);
+    commit();
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int t = kStages; t < 2 * kR; ++t) q[t] = center(t % kStages);
+    int sc = kR % kStages, sn = (2 * kR) % kStages, sp = kR % kPrev, k = k0;
+    float4 vv = load_v(k0), v1 = load_v(min(k0 + 1, k1 - 1));
+    auto step = [&](auto phase) {
+        constexpr int PH = decltype(phase)::value;
+        constexpr int Q = 2 * kR + 1;
+        const int tc = k - k0 + kR;
+        // all but the newest group are here; every thread is done with the previous step
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        {
+            const int t = tc - 1 + kStages;  // into the stage of plane tc - 1
+            if (t < T) copy_plane(k0 - kR + t, sc == 0 ? kStages - 1 : sc - 1);
+            if (P && k + kPrev - 1 < k1) copy_prev(k + kPrev - 1, sp == 0 ? kPrev - 1 : sp - 1);
+            commit();
+        }
+        const float4 v2 = load_v(min(k + 2, k1 - 1));
+        q[(PH + 2 * kR) % Q] = center(sn);
+        const float *row = sm + sc * kStageFloats + (kR + ty) * kW + 4 * tx;
+        float2 aA, aB;
+        plane_math<PH>(row, q, vv, cf, aA, aB);
+        // the tile's slot takes the result in place of Y_{j-1}: a warp writes its four rows as
+        // its threads own them and stores them row by row
+        float *const ot = prev + sp * kTileFloats;
+        float4 *const mine = reinterpret_cast<float4 *>(ot + ty * kBX + 4 * tx);
+        if (P) {
+            const float4 pv = *mine;
+            aA = __ffma2_rn(cf.nbeta, lo2(pv), aA);
+            aB = __ffma2_rn(cf.nbeta, hi2(pv), aB);
+        }
+        *mine = make_float4(aA.x, aA.y, aB.x, aB.y);
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = 4 * warp + u;
+            if (xin && j0 + r < n1)
+                O[(unsigned)(i0 + lane) + (unsigned)n0 * (unsigned)(j0 + r) + (unsigned)k * plane] =
+                    ot[r * kBX + lane];
+        }
+        vv = v1;
+        v1 = v2;
+        if (++sc == kStages) sc = 0;
+        if (++sn == kStages) sn = 0;
+        if (++sp == kPrev) sp = 0;
+        ++k;
+    };
+#define SPARC_COPY_STEP(PH)                                                              \
+    if (k >= k1) break;                                                                  \
+    step(std::integral_constant<int, PH>{});
+    for (;;) {
+        SPARC_COPY_STEP(0) SPARC_COPY_STEP(1) SPARC_COPY_STEP(2) SPARC_COPY_STEP(3)
+        SPARC_COPY_STEP(4) SPARC_COPY_STEP(5) SPARC_COPY_STEP(6) SPARC_COPY_STEP(7)
+        SPARC_COPY_STEP(8) SPARC_COPY_STEP(9) SPARC_COPY_STEP(10) SPARC_COPY_STEP(11)
+        SPARC_COPY_STEP(12)
+    }
+#undef SPARC_COPY_STEP
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
 // Work-list form for a batch of clusters: a persistent CTA walks its items (cluster,
 // column, 32 x 16 tile, z range) in order, and its ring runs on across item boundaries: the
 // planes of all its items form one sequence (item i contributes (k1 - k0) + 12 planes),
@@ -285,7 +463,7 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
 // consumers take the planes in the same order. Each cluster's tensor maps (Y_j with halo,
 // Y_{j-1} tile) live in device memory, its sizes, pointers and coefficients in its
 // BatchTma entry. Same per-point arithmetic as k_stencil_f32_tma.
-__global__ void __launch_bounds__(kTX *kTY)
+__global__ void __launch_bounds__(kTX *kTY, 4)
 k_batch_stencil_tma(const BatchItem *__restrict__ items, int nitems, const BatchTma *cs, int *err)
 {
     extern __shared__ __align__(128) float sm[];
@@ -324,7 +502,9 @@ k_batch_stencil_tma(const BatchItem *__restrict__ items, int nitems, const Batch
             float *st = sm + (long)s * kStageFloats;
             mbar_arrive_expect_tx(&full[s], kPlaneBytes + (p ? kTileBytes : 0));
             tma_load_4d(st, p_mY, &full[s], p_x - 8, p_y - kR, p_z + p_t, p_col);
-            if (p) tma_load_4d(st + kH * kW, p_mP, &full[s], p_x, p_y, p_z - kR + p_t, p_col);
+            if (p)
+                tma_load_4d(sm + kStages * kStageFloats + issued % kPrev * kTileFloats, p_mP,
+                            &full[s], p_x, p_y, p_z - kR + p_t, p_col);
             ++issued;
             if (++p_t == p_T) {
                 p_t = 0;
@@ -410,8 +590,8 @@ k_batch_stencil_tma(const BatchItem *__restrict__ items, int nitems, const Batch
                 float4 o = make_float4(acc[0], acc[1], acc[2], acc[3]);
                 if (hasP) {
                     const float4 pv = *reinterpret_cast<const float4 *>(
-                        sm + ((g0 + tc + kR) % kStages) * kStageFloats + kH * kW + ty * kBX +
-                        4 * tx);
+                        sm + kStages * kStageFloats + (g0 + tc + kR) % kPrev * kTileFloats +
+                        ty * kBX + 4 * tx);
                     o.x -= cf.beta * pv.x;
                     o.y -= cf.beta * pv.y;
                     o.z -= cf.beta * pv.z;
@@ -493,7 +673,7 @@ cudaError_t batch_stencil_tma(const BatchItem *items, int nitems, const BatchTma
 {
     if (nitems <= 0) return cudaSuccess;
     static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
-    const int smem = kStages * kStageFloats * 4;
+    const int smem = kSmemBytes;
     if (!attr_set.load(std::memory_order_acquire)) {
         cudaError_t e = cudaFuncSetAttribute(k_batch_stencil_tma,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -512,6 +692,54 @@ bool stencil_tma_ok(const DevHam &H, const void *Y, const void *Yprev, const voi
            al(H.Vf) && H.n0 <= (1 << 24) && H.n1 <= (1 << 24);
 }
 
+// z ranges per column of the two kernels above: 608 CTAs (four per SM) run at a time, each for
+// its planes plus about eight plane-times for the twelve it reads ahead; the count with the
+// fewest plane-times over all waves, of at least eight planes each.
+static void f32_z_split(int n2, long tiles, int ncols, int &nzc, int &zchunk)
+{
+    constexpr int kFill = 8, kMinPlanes = 8;
+    const long per = tiles * ncols;
+    long best = -1;
+    nzc = 1;
+    zchunk = n2;
+    for (int z = 1; z == 1 || (n2 / z >= kMinPlanes && (long)z * ncols <= 65535); ++z) {
+        const int zc = (n2 + z - 1) / z, used = (n2 + zc - 1) / zc;
+        const long cost = (per * used + 607) / 608 * (zc + kFill);
+        if (best < 0 || cost < best) best = cost, nzc = used, zchunk = zc;
+    }
+}
+
+static StepCoef2 pair_coef(const StepCoef<float> &cf)
+{
+    StepCoef2 c2;
+    for (int r = 0; r <= kR; ++r) c2.w[r] = make_float2(cf.w[r], cf.w[r]);
+    c2.c0 = make_float2(cf.c0, cf.c0);
+    c2.alpha = make_float2(cf.alpha, cf.alpha);
+    c2.nbeta = make_float2(-cf.beta, -cf.beta);
+    return c2;
+}
+
+cudaError_t stencil_f32_copy(const DevHam &H, const float *Y, const float *Yprev, float *out,
+                             int ncols, long ld, const StepCoef<float> &cf, cudaStream_t st)
+{
+    if (ncols <= 0) return cudaSuccess;
+    if (ncols > 65535) return cudaErrorInvalidValue;
+    static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
+    if (!attr_set.load(std::memory_order_acquire)) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            k_stencil_f32_copy, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e != cudaSuccess) return e;
+        attr_set.store(true, std::memory_order_release);
+    }
+    const int gx = (H.n0 + kBX - 1) / kBX, gy = (H.n1 + kTY - 1) / kTY;
+    int nzc, zchunk;
+    f32_z_split(H.n2, (long)gx * gy, ncols, nzc, zchunk);
+    k_stencil_f32_copy<<<dim3(gx, gy, ncols * nzc), dim3(kTX, kTY), kSmemBytes, st>>>(
+        Y, Yprev, out, H.Vf, H.n0, H.n1, H.n2, ld, nzc, zchunk, pair_coef(cf));
+    note_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev, float *out,
                             int ncols, long ld, const StepCoef<float> &cf, int *err,
                             cudaStream_t st)
@@ -519,7 +747,7 @@ cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev,
     cudaError_t e = get_encoder();
     if (e != cudaSuccess) return e;
     static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
-    const int smem = kStages * kStageFloats * 4;
+    const int smem = kSmemBytes;
     if (!attr_set.load(std::memory_order_acquire)) {
         e = cudaFuncSetAttribute(k_stencil_f32_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  smem);
@@ -547,16 +775,11 @@ cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev,
     }
     const int gx = (H.n0 + kBX - 1) / kBX, gy = (H.n1 + kTY - 1) / kTY;
     int nzc, zchunk;
-    stencil_z_split(H.n2, (long)gx * gy, ncols, nzc, zchunk);
-    StepCoef2 c2;
-    for (int r = 0; r <= kR; ++r) c2.w[r] = make_float2(cf.w[r], cf.w[r]);
-    c2.c0 = make_float2(cf.c0, cf.c0);
-    c2.alpha = make_float2(cf.alpha, cf.alpha);
-    c2.nbeta = make_float2(-cf.beta, -cf.beta);
+    f32_z_split(H.n2, (long)gx * gy, ncols, nzc, zchunk);
     dim3 grid(gx, gy, ncols * nzc);
     k_stencil_f32_tma<<<grid, dim3(kTX, kTY), smem, st>>>(mapY, mapP, Yprev != nullptr, out,
                                                           H.Vf, H.n0, H.n1, H.n2, ld, nzc,
-                                                          zchunk, c2, err);
+                                                          zchunk, pair_coef(cf), err);
     note_launch();
     return cudaGetLastError();
 }
