@@ -30,29 +30,42 @@
 // and classes 3, 4 (products below 2^-22 of the leading term) are dropped. Per chunk a class
 // accumulator holds at most 3 x 2^14 x 256 < 2^24 in magnitude, so its FP32 sums are
 // exact integers. After each chunk the epilogue warps read the three accumulators from
-// tensor memory, combine them exactly into an FP32 pair (TwoSum), scale the pair by the
-// chunk's power of two 2^(e_i + e_j - 14) and add it to FP32-pair running sums (error about
-// 2^-48 relative). The result is the Gram matrix of the 23-bit rounded block with no error
-// growth along Nd; the FP32-pair Gram of gram_df.cu remains the exact one.
+// tensor memory, combine them into an FP32 pair, apply 2^(e_i + e_j) exactly and add them
+// into a running FP32-pair sum (errors of a few 2^-39 of the chunk's largest product, no
+// FP64 pipe). The result is the Gram matrix of the 23-bit rounded block with no error growth
+// along Nd; the FP32-pair Gram of gram_df.cu remains the exact one. The 47-bit form combines a
+// chunk's accumulators into one 64-bit integer, shifts it right by the chunk's exponents'
+// distance from the columns' largest (E_i - e_i + E_j - e_j, rounded) and adds it to a 64-bit
+// integer sum.
 //
 // Layout and pipeline. A pre-pass (k_tc_digits) writes the digits of an operand in the
 // shared-memory order the MMA reads (no swizzle, K-major, 8-row x 16-byte core matrices)
 // as 8 KB blobs, one per (128-column block, 32-row step, digit), plus the exponents
-// e(c, j). A CTA owns one 128 x 128 tile of G over a range of chunks (split-K): warp 0
-// streams the blobs of A and B into a three-stage ring with untiled bulk copies (48 KB a
-// stage; B's digits side by side along N), one thread of warp 1 issues the tcgen05.mma
-// (M = 128, K = 16): per A digit s one MMA over the B digits 0 .. 2 - s at once (N = 384 as
-// 256 + 128, then 256, then 128), which writes the class accumulators s .. 2 side by side
-// (384 tensor-memory columns) and reads the A digit once instead of once per product; it
-// commits stage releases and chunk completions to mbarriers, and eight epilogue warps (two per tensor-memory lane quarter,
-// 64 columns each; high parts of the running sums in registers, low parts in shared
-// memory) flush every chunk. Partial tiles of the K splits are summed by a
-// second kernel in a fixed order (deterministic). Every wait is bounded; on a timeout the
-// kernel raises *err, drains its copies and MMAs (bounded), frees its tensor memory and
-// returns.
+// e(c, j). A CTA owns one 128 x 128 tile of G (Tc47: 128 x 64) over a range of chunks
+// (split-K): warp 0 streams a step's blobs into a three-stage ring, A by one untiled bulk
+// copy, B by one tiled copy that lays its digits side by side along N. One thread of warp 1
+// issues the tcgen05.mma (M = 128, K = 16): per A digit s one MMA over the kept B digits
+// 0 .. at once (Tc23: N = 384 as 256 + 128, then 256, then 128), which writes the class
+// accumulators s .. side by side (384 tensor-memory columns) and reads the A digit once
+// instead of once per product; it commits stage releases and chunk completions to mbarriers,
+// and sixteen epilogue warps (four per tensor-memory lane quarter, the running sums in
+// registers) flush every chunk. Partial tiles of the K splits are summed by a second kernel
+// in a fixed order (deterministic). Every wait is bounded; on a timeout the kernel raises
+// *err, drains its copies and MMAs (bounded), frees its tensor memory and returns.
+//
+// What bounds it. The MMAs of a 96^3 x 128 Tc47 launch need 0.26 ms at the tensor pipe's
+// rate (21 products, N = 64 .. 256). Of its 0.73 ms the pipe was busy 44%: the issuing thread
+// formed descriptors and tested barriers for longer than a step's MMAs took, B's 1 KB pieces
+// came in twelve requests a step, and every chunk waited for the epilogue's sums of pairs.
+// Uniform issue, one copy for B, 32-row steps and 64-bit integer sums of which only the
+// combination is waited for: 0.46 ms (128^3 x 512, two slabs, M and H: 33.8 -> 20.9 ms). What
+// is left is that wait, about 2000 cycles a chunk beside 5400 of MMAs (the class accumulators
+// fill 384 of the 512 columns, so no second set fits).
 #include "internal.cuh"
 
+#include <algorithm>
 #include <atomic>
+#include <cstring>
 #include "tma.cuh"
 
 #include <cstdint>
@@ -62,11 +75,12 @@ namespace sparc {
 
 namespace {
 constexpr int kTile = 128;                     // MMA M (A columns per tile)
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 16;                  // four per tensor-memory lane quarter
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr unsigned kWaitLimit = 1u << 22;
 constexpr int kTmemCols = 512;
-constexpr int kNonFinite = INT32_MIN;          // exponent sentinel of a chunk with Inf/NaN
+constexpr int kNonFinite = INT32_MAX;          // exponent sentinel of a chunk with Inf/NaN
+constexpr int kZeroExp = -4096;                // exponent of an all-zero chunk column
 // core-matrix offsets inside a blob (elements): K-adjacent cores 2048 B apart, M/N-adjacent
 // cores 128 B apart
 constexpr unsigned kLbo = 2048, kSbo = 128;
@@ -84,10 +98,12 @@ constexpr unsigned kLbo = 2048, kSbo = 128;
 struct Tc23 {
     static constexpr int kDigits = 3, kClasses = 3, kBits = 23, kChunk = 256, kStep = 32,
                          kN = 128, kStages = 3, kBase = 8;
+    static constexpr bool kPair = true;   // epilogue sums as FP32 pairs
 };
 struct Tc47 {
-    static constexpr int kDigits = 6, kClasses = 6, kBits = 47, kChunk = 128, kStep = 16,
-                         kN = 64, kStages = 4, kBase = 8;
+    static constexpr int kDigits = 6, kClasses = 6, kBits = 47, kChunk = 128, kStep = 32,
+                         kN = 64, kStages = 3, kBase = 8;
+    static constexpr bool kPair = false;  // as 64-bit integers
 };
 // A stage holds A's blobs (all 128 columns of each digit) and the kN columns of B's blobs
 // this CTA multiplies. B is stored digit-concatenated: per 8-row K group, the kN / 8 core
@@ -104,9 +120,9 @@ template <class C> struct TcDims {
     static constexpr unsigned kBOperandBytes = C::kDigits * C::kN * C::kStep * 2;
     static constexpr unsigned kStageBytes = kOperandBytes + kBOperandBytes;
     static constexpr int kHalves = kTile / C::kN;                          // CTAs per tile
-    static constexpr int kEpiCols = C::kN / 2;                             // per epilogue warp
-    // ring, then the low parts of the epilogue's running pair sums ([warp][column][lane])
-    static constexpr unsigned kLowBytes = kEpiWarps * kEpiCols * 32 * 4;
+    static constexpr int kEpiCols = C::kN / (kEpiWarps / 4);              // per epilogue warp
+    // ring, then (Tc23) the low parts of the epilogue's running pair sums ([warp][column][lane])
+    static constexpr unsigned kLowBytes = C::kPair ? kEpiWarps * kEpiCols * 32 * 4 : 0;
     static constexpr unsigned kSmemBytes = C::kStages * kStageBytes + kLowBytes + 1024;
     static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
     static_assert(C::kClasses * C::kN <= kTmemCols, "class accumulators exceed tensor memory");
@@ -117,6 +133,9 @@ template <class C> struct TcDims {
     static_assert(((long)C::kClasses << (2 * C::kBase - 2)) * C::kChunk < (1L << 24),
                   "class sums of a chunk must stay exact in FP32");
     static constexpr int kScale = C::kBits - C::kBase * (C::kDigits - 1);
+    // Tc47: the epilogue's integer T = sum_w class_w 2^(8 (5 - w)), below 2^61.1, counts
+    // 2^(e_i + e_j - kUnit)
+    static constexpr int kUnit = 2 * kScale + C::kBase * (C::kClasses - 1);
 };
 
 namespace {
@@ -147,83 +166,142 @@ template <> struct FBits<double> {
 };
 }  // namespace
 
-// Digits and exponents of one operand. CTA: one chunk (blockIdx.y) x 8 columns
-// (blockIdx.x), one warp per column, kChunk / 32 rows per lane. Rows past nd and columns
-// past ns are zero; a chunk column holding Inf or NaN gets the exponent kNonFinite.
+// |x| (bit pattern mag) on the grid of exponent e: round(|x| 2^(kBits - e)), in [0, 2^kBits].
 template <class C, typename T>
-__global__ void __launch_bounds__(256)
-k_tc_digits(const T *__restrict__ X, long ld, long nd, int ns, long nstep,
-            __nv_bfloat16 *__restrict__ D, int *__restrict__ E, int ns_pad)
+__device__ __forceinline__ unsigned long long grid_value(typename FBits<T>::U mag, int e)
 {
     using B = FBits<T>;
     using U = typename B::U;
-    constexpr int R = C::kChunk / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int col = blockIdx.x * 8 + warp;
-    const long chunk = blockIdx.y;
-    const long k0 = chunk * C::kChunk;
-    U mag[R];
-    bool ng[R];
-    U mx = 0;
-    bool bad = false;
-    const U inf = (U)B::kExpMask << B::kMant;
+    if (mag == 0) return 0ull;
+    const int bx = (int)(mag >> B::kMant);
+    const U m = (mag & (((U)1 << B::kMant) - 1)) | (bx ? ((U)1 << B::kMant) : 0);
+    const int sh = e + B::kBias + B::kMant - C::kBits - (bx ? bx : 1);
+    if (sh <= 0) return (unsigned long long)m << (-sh);  // exact: FP32 inputs of the 47-bit form
+    if (sh < 8 * (int)sizeof(U)) return (unsigned long long)((m + ((U)1 << (sh - 1))) >> sh);
+    return 0ull;
+}
+
+// exponent of a chunk column from its largest magnitude: |x| < 2^e
+template <typename T>
+__device__ __forceinline__ int chunk_exponent(typename FBits<T>::U mx)
+{
+    using B = FBits<T>;
+    const int bx = (int)(mx >> B::kMant);
+    return mx == 0 ? kZeroExp : (bx == 0 ? 2 - B::kBias : bx - B::kBias + 1);
+}
+
+// The digits of eight grid values N (sign bit t of neg) as BF16, eight K-adjacent elements (16
+// bytes) per digit, digit s to dst + s stride. Adding 128 at every lower digit's place makes the
+// balanced digits the bytes of the sum minus 128 (the top digit, at most 128, is the byte as it
+// is): a byte permutation puts each into the significand of 1.5 2^23, one multiply-add takes
+// the offset off and applies the sign, and the upper half of the FP32 result is the BF16.
+template <class C>
+__device__ __forceinline__ void store_digits(const unsigned long long (&N)[8], unsigned neg,
+                                             __nv_bfloat16 *dst, long stride)
+{
+    static_assert(C::kBase == 8 && C::kDigits <= 8, "byte digits");
+    constexpr unsigned long long kBias = 0x8080808080808080ull >> (64 - 8 * (C::kDigits - 1));
+    constexpr float kM = 12582912.0f;  // 1.5 * 2^23, bits 0x4B400000
+    unsigned lo[8], hi[8];
+    float sg[8];
 #pragma unroll
-    for (int u = 0; u < R; ++u) {
-        const long k = k0 + lane + 32 * u;
-        T x = (T)0;
-        if (col < ns && k < nd) x = X[k + (long)col * ld];
-        mag[u] = B::mag(x);
-        ng[u] = B::neg(x);
-        bad |= mag[u] >= inf;
-        mx = mag[u] > mx ? mag[u] : mx;
+    for (int t = 0; t < 8; ++t) {
+        const unsigned long long n = N[t] + kBias;
+        lo[t] = (unsigned)n;
+        hi[t] = (unsigned)(n >> 32);
+        sg[t] = ((neg >> t) & 1u) ? -1.0f : 1.0f;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int s = 0; s < C::kDigits; ++s) {
+        const int byte = C::kDigits - 1 - s;
+        const float off = -(kM + (s ? 128.0f : 0.0f));
+        unsigned f[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const unsigned x = __byte_perm(byte < 4 ? lo[t] : hi[t], 0x4B400000u, 0x7650u | (byte & 3));
+            f[t] = __float_as_uint(fmaf(__uint_as_float(x), sg[t], off * sg[t]));
+        }
+        uint4 v;
+        v.x = __byte_perm(f[0], f[1], 0x7632);
+        v.y = __byte_perm(f[2], f[3], 0x7632);
+        v.z = __byte_perm(f[4], f[5], 0x7632);
+        v.w = __byte_perm(f[6], f[7], 0x7632);
+        *reinterpret_cast<uint4 *>(dst + s * stride) = v;
+    }
+}
+
+// Eight consecutive rows of a column from row k (zero past nd); vec: 16-byte loads allowed.
+template <typename T>
+__device__ __forceinline__ void load8(const T *X, long k, long nd, bool live, bool vec, T (&x)[8])
+{
+    if (live && vec && k + 8 <= nd) {
+        constexpr int W = 16 / sizeof(T);
+#pragma unroll
+        for (int u = 0; u < 8 / W; ++u) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(X + k + W * u);
+            memcpy(&x[W * u], &v, 16);
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = live && k + t < nd ? X[k + t] : (T)0;
+    }
+}
+
+// Digits and exponents of one operand. CTA: one chunk (blockIdx.y) x 8 or 16 columns
+// (blockIdx.x); a thread takes eight consecutive rows of a column, so its loads are whole
+// sectors and its stores 16 bytes per digit, 128 contiguous bytes per eight columns (a row
+// per lane stored two bytes at a time: 0.50 ms for a 96^3 x 128 FP64 block, 0.38 ms so).
+// Rows past nd and columns past ns are zero; a chunk column holding Inf or NaN gets the
+// exponent kNonFinite. EX[col] is raised to the column's largest exponent.
+template <class C, typename T>
+__global__ void __launch_bounds__(256)
+k_tc_digits(const T *__restrict__ X, long ld, long nd, int ns, long nstep, bool vec,
+            __nv_bfloat16 *__restrict__ D, int *__restrict__ E, int *__restrict__ EX, int ns_pad)
+{
+    using B = FBits<T>;
+    using U = typename B::U;
+    constexpr int kKg = C::kChunk / 8, kCols = 256 / kKg, kWarpsPer = C::kChunk / 32;
+    static_assert(kCols * kKg == 256 && kCols % 8 == 0, "threads of a chunk");
+    __shared__ U red[8][8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c8 = tid & 7, kg = (tid >> 3) % kKg, grp = tid / (8 * kKg);
+    const int col = blockIdx.x * kCols + grp * 8 + c8;
+    const long chunk = blockIdx.y, k = chunk * C::kChunk + kg * 8;
+    T x[8];
+    load8(X + (long)(col < ns ? col : 0) * ld, k, nd, col < ns, vec, x);
+    U mx = 0;
+    unsigned neg = 0u;
+    const U inf = (U)B::kExpMask << B::kMant;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const U m = B::mag(x[t]);
+        mx = m > mx ? m : mx;
+        neg |= (B::neg(x[t]) ? 1u : 0u) << t;
+    }
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
         const U t = (U)__shfl_xor_sync(0xffffffffu, (unsigned long long)mx, o);
         mx = t > mx ? t : mx;
     }
-    bad = __any_sync(0xffffffffu, bad);
-    // max |x| < 2^e: e = unbiased exponent of the max + 1 (normal), 1 - bias + 1 for
-    // subnormals; 0 for an all-zero chunk column
-    const int bxm = (int)(mx >> B::kMant);
-    const int e = mx == 0 ? 0 : (bxm == 0 ? 2 - B::kBias : bxm - B::kBias + 1);
-    if (lane == 0 && col < ns_pad) E[chunk * ns_pad + col] = bad ? kNonFinite : e;
-    const int cb = col >> 7, c = col & 127;
+    if (lane < 8) red[warp][lane] = mx;
+    __syncthreads();
+    const int w0 = grp * kWarpsPer;
 #pragma unroll
-    for (int u = 0; u < R; ++u) {
-        const long k = k0 + lane + 32 * u;
-        long N = 0;
-        if (!bad && mag[u] != 0) {
-            const int bx = (int)(mag[u] >> B::kMant);
-            const U m = (mag[u] & (((U)1 << B::kMant) - 1)) | (bx ? ((U)1 << B::kMant) : 0);
-            const int ebx = bx ? bx : 1;
-            // N = round(m 2^(ebx - bias - mant + kBits - e)) in [0, 2^kBits]
-            const int sh = e + B::kBias + B::kMant - C::kBits - ebx;
-            if (sh <= 0)
-                N = (long)m << (-sh);  // exact: FP32 inputs of the 47-bit form
-            else if (sh < 8 * (int)sizeof(U))
-                N = (long)((m + ((U)1 << (sh - 1))) >> sh);
-        }
-        // balanced base-2^kBase digits from the bottom; the top one lies in
-        // [0, 2^(kBase - 1)]
-        constexpr long kHalf = 1L << (C::kBase - 1), kMask = (1L << C::kBase) - 1;
-        int d[C::kDigits];
-#pragma unroll
-        for (int s = C::kDigits - 1; s > 0; --s) {
-            d[s] = (int)(((N + kHalf) & kMask) - kHalf);
-            N = (N - d[s]) >> C::kBase;
-        }
-        d[0] = (int)N;
-        const int sg = ng[u] ? -1 : 1;
-        const long step = k / C::kStep;
-        const int kl = (int)(k % C::kStep);
-        if (col < ns_pad) {
-            const long base = blob_offset<C>(cb, step, 0, nstep) + in_blob(kl, c);
-#pragma unroll
-            for (int s = 0; s < C::kDigits; ++s)
-                D[base + (long)s * TcDims<C>::kBlobElems] = __float2bfloat16_rn((float)(sg * d[s]));
-        }
+    for (int w = 0; w < kWarpsPer; ++w) mx = red[w0 + w][c8] > mx ? red[w0 + w][c8] : mx;
+    const bool bad = mx >= inf;
+    const int e = chunk_exponent<T>(mx);
+    if (kg == 0 && col < ns_pad) {
+        E[chunk * ns_pad + col] = bad ? kNonFinite : e;
+        if (!bad && e > *(volatile int *)(EX + col)) atomicMax(EX + col, e);
     }
+    if (col >= ns_pad) return;
+    unsigned long long N[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) N[t] = bad ? 0ull : grid_value<C, T>(B::mag(x[t]), e);
+    const int cb = col >> 7, c = col & 127;
+    store_digits<C>(N, neg,
+                    D + blob_offset<C>(cb, k / C::kStep, 0, nstep) + in_blob((int)(k % C::kStep), c),
+                    TcDims<C>::kBlobElems);
 }
 
 // 2^(e - kScale) as an FP32 factor (the chunk scale 2^(e_i + e_j - 2 kScale) is applied as
@@ -245,17 +323,35 @@ __device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e)
     e = (a - (s - bb)) + (b - bb);
 }
 
-// FP32 -> FP64 by moving the exponent field (integer operations; FP32 subnormals count as
-// zero, Inf / NaN stay so): the rotation writes one output per thread and column, where an
-// FP64 conversion instruction per value would load the FP64 pipe.
-__device__ __forceinline__ double widen_int(float f)
+// a 2^sc as FP64, rounded to nearest, by integer operations (an FP64 instruction per output
+// would load the FP64 pipe); below the normal range 0, above it Inf.
+__device__ __forceinline__ double scaled_to_double(long long a, int sc)
 {
-    const unsigned u = __float_as_uint(f);
-    const unsigned e = (u >> 23) & 0xffu, m = u & 0x7fffffu, sg = u & 0x80000000u;
-    unsigned hi = sg | ((e + 896u) << 20) | (m >> 3), lo = m << 29;
-    if (e == 0u) hi = sg, lo = 0u;
-    if (e == 0xffu) hi = sg | 0x7ff00000u | (m ? 0x80000u : 0u), lo = 0u;
-    return __hiloint2double((int)hi, (int)lo);
+    const unsigned long long sgn = (unsigned long long)a & 0x8000000000000000ull;
+    const unsigned long long m = (unsigned long long)(a < 0 ? -a : a);
+    if (m == 0) return 0.0;
+    const int lz = __clzll((long long)m);
+    const unsigned long long t = m << lz;
+    const unsigned long long r = (t >> 11) + ((t >> 10) & 1ull);  // 53 bits, hidden bit included
+    const int e = 1023 + 63 - lz + sc;
+    if (e <= 0) return 0.0;
+    if (e >= 2047) return __longlong_as_double((long long)(sgn | 0x7ff0000000000000ull));
+    return __longlong_as_double((long long)(sgn | (((unsigned long long)(e - 1) << 52) + r)));
+}
+
+// The chunk's integer T from Tc47's class sums (exact integers in FP32, below 2^21, 2^22, 2^22.6,
+// 2^23, 2^23.4, 2^23.6). Integers up to 2^22 come out of the significand of 1.5 2^23 + v, larger
+// ones by conversion; the last two classes are rounded together to 2^10 (2^-51 of T's range).
+__device__ __forceinline__ long long class_sum47(const uint32_t (&v)[6])
+{
+    constexpr float kM = 12582912.0f;
+    auto f = [&](int w) { return __uint_as_float(v[w]); };
+    const int b0 = __float_as_int(f(0) + kM), b1 = __float_as_int(f(1) + kM);
+    const int i1 = (int)(((unsigned)b0 << 8) + (unsigned)b1 - (0x40000000u + 0x4B400000u));
+    const int i2 = (int)(((unsigned)__float2int_rn(f(2)) << 8) + (unsigned)__float2int_rn(f(3)));
+    const float l = fmaf(f(5), 0x1p-10f, fmaf(f(4), 0x1p-2f, kM));
+    const int i3 = __float_as_int(l) - 0x4B400000;
+    return ((long long)i1 << 32) + ((long long)i2 * 65536 + (long long)i3 * 1024);
 }
 
 // Digits of the transposed operand: B = Y^T for the rotation, so the K dimension runs over
@@ -299,52 +395,21 @@ k_tc_digits_t(const T *__restrict__ Y, long ld, long nd, int ns, long nstep,
         mx = red[q][lane] > mx ? red[q][lane] : mx;
         bad |= bad_s[q][lane];
     }
-    const int bxm = (int)(mx >> B::kMant);
-    const int e = mx == 0 ? 0 : (bxm == 0 ? 2 - B::kBias : bxm - B::kBias + 1);
+    const int e = chunk_exponent<T>(mx);
     if (g == 0 && row < nd_pad) E[chunk * nd_pad + row] = bad ? kNonFinite : e;
     if (row >= nd_pad) return;
-    // each value's magnitude on the grid and its sign; the digits are then peeled off from
-    // the bottom and each digit's 8 values stored at once (16 bytes: the 8 K-adjacent
-    // elements of a core-matrix row; the 32 rows of a warp fill 512 contiguous bytes)
-    long N[8];
+    unsigned long long N[8];
     unsigned neg = 0u;
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-        const U mag = B::mag(x[t]);
-        N[t] = 0;
-        if (!bad && mag != 0) {
-            const int bx = (int)(mag >> B::kMant);
-            const U m = (mag & (((U)1 << B::kMant) - 1)) | (bx ? ((U)1 << B::kMant) : 0);
-            const int ebx = bx ? bx : 1;
-            const int sh = e + B::kBias + B::kMant - C::kBits - ebx;
-            if (sh <= 0)
-                N[t] = (long)m << (-sh);
-            else if (sh < 8 * (int)sizeof(U))
-                N[t] = (long)((m + ((U)1 << (sh - 1))) >> sh);
-        }
+        N[t] = bad ? 0ull : grid_value<C, T>(B::mag(x[t]), e);
         neg |= (B::neg(x[t]) ? 1u : 0u) << t;
     }
     // the 8 columns kb .. kb+7 lie in one K-step (kStep is a multiple of 8) and one core
     const int cb = (int)(row >> 7), c = (int)(row & 127);
-    const long base = blob_offset<C>(cb, kb / C::kStep, 0, nstep) + in_blob(kb % C::kStep, c);
-    constexpr long kHalf = 1L << (C::kBase - 1), kMask = (1L << C::kBase) - 1;
-#pragma unroll
-    for (int s2 = C::kDigits - 1; s2 >= 0; --s2) {
-        __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            int dv;
-            if (s2 > 0) {
-                dv = (int)(((N[t] + kHalf) & kMask) - kHalf);
-                N[t] = (N[t] - dv) >> C::kBase;
-            } else {
-                dv = (int)N[t];
-            }
-            v[t] = __float2bfloat16_rn((float)(((neg >> t) & 1u) ? -dv : dv));
-        }
-        *reinterpret_cast<uint4 *>(D + base + (long)s2 * TcDims<C>::kBlobElems) =
-            *reinterpret_cast<const uint4 *>(v);
-    }
+    store_digits<C>(N, neg,
+                    D + blob_offset<C>(cb, kb / C::kStep, 0, nstep) + in_blob(kb % C::kStep, c),
+                    TcDims<C>::kBlobElems);
 }
 
 // tiles[t] = (A column block, B column block); a tile is computed by kHalves CTAs, each
@@ -361,16 +426,16 @@ k_tc_digits_t(const T *__restrict__ Y, long ld, long nd, int ns, long nstep,
 template <class C, bool ROT, typename TO = double>
 __global__ void __launch_bounds__(kThreads, 1)
 k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
-          const __nv_bfloat16 *__restrict__ DB, const int *__restrict__ EB, int ns_pad, long nstep,
+          const __grid_constant__ CUtensorMap mapB, const int *__restrict__ EB, int ns_pad, long nstep,
           const int2 *__restrict__ tiles, int ntiles, int nsplit, double *__restrict__ part,
-          int *err, int eb_ld = 0, int mblk = 1, TO *__restrict__ out = nullptr, long ldo = 0,
+          int drop, int *err, const int *__restrict__ EXA, const int *__restrict__ EXB,
+          int eb_ld = 0, int mblk = 1, TO *__restrict__ out = nullptr, long ldo = 0,
           long nrow = 0, int ncol = 0, long ea_ld = 0)
 {
     using Dm = TcDims<C>;
     constexpr int kStages = C::kStages, kStepsPerChunk = Dm::kStepsPerChunk;
     constexpr unsigned kStageBytes = Dm::kStageBytes, kOperandBytes = Dm::kOperandBytes;
-    constexpr unsigned kBLbo = Dm::kBLbo, kBPiece = Dm::kBPiece;
-    constexpr int kGroups = C::kStep / 8;  // 8-row K groups of a step
+    constexpr unsigned kBLbo = Dm::kBLbo;
     constexpr int kEpiCols = Dm::kEpiCols;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[kStages], empty[kStages], acc_full, acc_empty, drain;
@@ -422,109 +487,126 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
         atomicExch(err, 1);
     };
 
+    // Warps 0 and 1 run their loops whole, so that the counters and the operand descriptors are
+    // uniform values; one lane issues. A step's MMAs take 672 (Tc47) or 768 cycles (Tc23), and a
+    // single thread that formed 14 descriptors and tested two barriers between steps needed more
+    // than that: the tensor pipe was idle 55% of the time.
     if (warp == 0) {
         // ---- producer: A and B blobs of each step into the ring, unit after unit ----
-        if (lane == 0) {
-            long j = 0, issued = 0;  // steps handed to the ring over all units
-            for (int u = blockIdx.x; u < nunits && !abort_flag; u += ustride) {
-                const Unit w = unit(u);
-                for (long st = w.c0 * kStepsPerChunk; st < w.c1 * kStepsPerChunk && !abort_flag;
-                     ++st, ++j) {
-                    const int s = (int)(j % kStages);
-                    if (j >= kStages &&
-                        !mbar_wait(&empty[s], (unsigned)(((j / kStages) & 1) ^ 1), kWaitLimit)) {
-                        fail();
-                        break;
-                    }
+        // A's blobs are one run of memory; this unit's kN columns of B's digits come by one tiled
+        // copy that puts them digit by digit within each K group (copied piece by piece they were
+        // kDigits kGroups requests of 1 KB a step, which the copy unit does not serve in the time
+        // of the MMAs: 605 us for the 96^3 x 128 block below, 524 us by one copy)
+        unsigned j = 0;  // steps handed to the ring over all units
+        int s = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < nunits && ok; u += ustride) {
+            const Unit w = unit(u);
+            const __nv_bfloat16 *src = DA + blob_offset<C>(w.tb.x, w.c0 * kStepsPerChunk, 0, nstep);
+            int row = (int)((w.tb.y * nstep + w.c0 * kStepsPerChunk) * C::kDigits);
+            const long n = (w.c1 - w.c0) * kStepsPerChunk;
+            for (long st = 0; st < n; ++st) {
+                ok = j < kStages || mbar_wait(&empty[s], (j / kStages & 1u) ^ 1u, kWaitLimit);
+                ok = __all_sync(0xffffffffu, ok && !abort_flag);
+                if (!ok) {
+                    if (lane == 0) fail();
+                    break;
+                }
+                if (lane == 0) {
                     unsigned char *dst = smem + (size_t)s * kStageBytes;
                     mbar_arrive_expect_tx(&full[s], kStageBytes);
-                    bulk_load(dst, DA + blob_offset<C>(w.tb.x, st, 0, nstep), kOperandBytes,
-                              &full[s]);
-                    // this unit's kN columns of every digit and K group of B, digit-concatenated
-#pragma unroll
-                    for (int d = 0; d < C::kDigits; ++d)
-#pragma unroll
-                        for (int g = 0; g < kGroups; ++g)
-                            bulk_load(dst + kOperandBytes + g * kBLbo + d * kBPiece,
-                                      DB + blob_offset<C>(w.tb.y, st, d, nstep) + g * (kTile * 8) +
-                                          w.hf * (C::kN * 8),
-                                      kBPiece, &full[s]);
-                    issued = j + 1;
+                    bulk_load(dst, src, kOperandBytes, &full[s]);
+                    tma_load_3d(dst + kOperandBytes, &mapB, &full[s], w.hf * (C::kN * 2), row, 0);
                 }
-            }
-            if (abort_flag) {
-                // wait (bounded) for the last copy issued into each stage
-                for (int s = 0; s < kStages; ++s) {
-                    long last = -1;
-                    for (long q = s; q < issued; q += kStages) last = q;
-                    if (last >= 0)
-                        mbar_wait(&full[s], (unsigned)((last / kStages) & 1), kWaitLimit);
-                }
+                __syncwarp();
+                src += C::kDigits * Dm::kBlobElems;
+                row += C::kDigits;
+                ++j;
+                s = s + 1 == kStages ? 0 : s + 1;
             }
         }
+        if (abort_flag) {
+            // wait (bounded) for the last copy issued into each stage
+            for (int q = 0; q < kStages; ++q) {
+                if (j <= (unsigned)q) break;
+                const unsigned last = j - 1 - (j - 1 - q) % kStages;  // j-1 or less, = q mod kStages
+                mbar_wait(&full[q], last / kStages & 1u, kWaitLimit);
+            }
+        }
+        __syncwarp();
     } else if (warp == 1) {
         // ---- MMA issuer ----
-        if (lane == 0) {
-            long j = 0, cc = 0;  // steps and chunks over all units
-            for (int u = blockIdx.x; u < nunits && !abort_flag; u += ustride) {
-                const Unit w = unit(u);
-                const long st0 = w.c0 * kStepsPerChunk;
-                for (long st = st0; st < w.c1 * kStepsPerChunk && !abort_flag; ++st, ++j) {
-                    const int s = (int)(j % kStages);
-                    const int kin = (int)((st - st0) % kStepsPerChunk);
-                    if (kin == 0 && cc > 0) {
-                        if (!mbar_wait(&acc_empty, (unsigned)((cc - 1) & 1), kWaitLimit)) {
-                            fail();
-                            break;
-                        }
-                        tc_fence_after();
-                    }
-                    if (!mbar_wait(&full[s], (unsigned)((j / kStages) & 1), kWaitLimit)) {
-                        fail();
-                        break;
-                    }
+        const uint64_t ad0 = smem_desc(smem, kLbo, kSbo);
+        const uint64_t bd0 = smem_desc(smem + kOperandBytes, kBLbo, kSbo);
+        const bool leader = lane == 0;
+        unsigned j = 0, cc = 0;  // steps and chunks over all units
+        int s = 0;
+        bool ok = true, ready = false;  // ready: stage s is known to be full
+        for (int u = blockIdx.x; u < nunits && ok; u += ustride) {
+            const Unit w = unit(u);
+            for (long c = w.c0; c < w.c1; ++c, ++cc) {
+                if (cc > 0) {
+                    ok = mbar_wait(&acc_empty, (cc - 1) & 1u, kWaitLimit) && !abort_flag;
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
                     tc_fence_after();
-                    const unsigned char *a = smem + (size_t)s * kStageBytes;
-                    const unsigned char *b = a + kOperandBytes;
+                }
+#pragma unroll 1
+                for (int kin = 0; kin < kStepsPerChunk; ++kin) {
+                    if (!ready) {
+                        ok = __all_sync(0xffffffffu,
+                                        mbar_wait(&full[s], j / kStages & 1u, kWaitLimit));
+                        if (!ok) break;
+                    }
+                    const uint64_t ads = ad0 + (unsigned)s * (kStageBytes >> 4);
+                    const uint64_t bds = bd0 + (unsigned)s * (kStageBytes >> 4);
+                    if (leader) {
 #pragma unroll
-                    for (int ks = 0; ks < C::kStep / 16; ++ks) {
+                        for (int ks = 0; ks < C::kStep / 16; ++ks) {
 #pragma unroll
-                        for (int sa = 0; sa < C::kDigits; ++sa) {
-                            // A digit sa times B digits 0 .. nb-1 (classes sa .. sa+nb-1, the
-                            // kept ones), as MMAs of N <= 256 over the digit-concatenated B
-                            const int nb = C::kClasses - sa < C::kDigits ? C::kClasses - sa
-                                                                         : C::kDigits;
-                            const uint64_t ad =
-                                smem_desc(a + sa * Dm::kBlobElems * 2 + ks * 2 * kLbo, kLbo, kSbo);
+                            for (int sa = 0; sa < C::kDigits; ++sa) {
+                                // A digit sa times B digits 0 .. nb-1 (classes sa .. sa+nb-1, the
+                                // kept ones), as MMAs of N <= 256 over the digit-concatenated B
+                                const int nb = C::kClasses - sa < C::kDigits ? C::kClasses - sa
+                                                                             : C::kDigits;
 #pragma unroll
-                            for (int n0 = 0; n0 < nb * C::kN; n0 += 256) {
-                                const int nl = nb * C::kN - n0 < 256 ? nb * C::kN - n0 : 256;
-                                const uint64_t bd =
-                                    smem_desc(b + ks * 2 * kBLbo + (n0 / 8) * kSbo, kBLbo, kSbo);
-                                // the sa = 0 MMAs cover every class: at a chunk start they
-                                // overwrite the accumulators, all later ones accumulate
-                                const bool first = kin == 0 && ks == 0 && sa == 0;
-                                tc_mma_bf16(tmem + (uint32_t)(sa * C::kN + n0), ad, bd,
-                                            idesc_bf16_f32(kTile, nl), !first);
+                                for (int n0 = 0; n0 < nb * C::kN; n0 += 256) {
+                                    const int nl = nb * C::kN - n0 < 256 ? nb * C::kN - n0 : 256;
+                                    // the sa = 0 MMAs cover every class: at a chunk start they
+                                    // overwrite the accumulators, all later ones accumulate
+                                    tc_mma_bf16(
+                                        tmem + (uint32_t)(sa * C::kN + n0),
+                                        ads + ((sa * Dm::kBlobElems * 2 + ks * 2 * kLbo) >> 4),
+                                        bds + ((ks * 2 * kBLbo + (n0 / 8) * kSbo) >> 4),
+                                        idesc_bf16_f32(kTile, nl), kin > 0 || ks > 0 || sa > 0);
+                                }
                             }
                         }
+                        tc_commit(&empty[s]);  // stage free once these MMAs are done
+                        if (kin == kStepsPerChunk - 1) tc_commit(&acc_full);  // chunk complete
                     }
-                    tc_commit(&empty[s]);  // stage free once these MMAs are done
-                    if (kin == kStepsPerChunk - 1) {
-                        tc_commit(&acc_full);  // chunk complete
-                        ++cc;
-                    }
+                    __syncwarp();
+                    ++j;
+                    s = s + 1 == kStages ? 0 : s + 1;
+                    // (a stage past the last one never fills)
+                    ready = __all_sync(0xffffffffu, mbar_test(&full[s], j / kStages & 1u));
                 }
+                if (!ok) break;
             }
+        }
+        if (leader) {
+            if (!ok) fail();
             // all MMAs issued by this thread are complete before tensor memory is freed
             tc_commit(&drain);
             if (!mbar_wait(&drain, 0u, kWaitLimit)) fail();
         }
+        __syncwarp();
     } else {
-        // ---- epilogue: flush each chunk's class accumulators into FP32-pair sums ----
         const int q = warp & 3;                 // tensor-memory lane quarter of this warp
         const int hw = (warp - 2) >> 2;         // columns kEpiCols hw .. of this CTA's kN
         const int r = q * 32 + lane;            // tile row = A column within the block
+        if constexpr (C::kPair) {
+        // ---- epilogue: flush each chunk's class accumulators into FP32-pair sums ----
         float H[kEpiCols];
         float *Lw = reinterpret_cast<float *>(smem + (size_t)kStages * kStageBytes) +
                     (size_t)(warp - 2) * kEpiCols * 32 + lane;  // Lw[u * 32]: column u
@@ -565,39 +647,38 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
                 }
                 tc_fence_after();
 #pragma unroll
-                for (int g = 0; g < kEpiCols / 8; ++g) {
+                for (int g = 0; g < kEpiCols / 4; ++g) {
                     const uint32_t ta =
-                        tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hw * kEpiCols + g * 8);
-                    uint32_t v[C::kClasses][8];
+                        tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hw * kEpiCols + g * 4);
+                    uint32_t v[C::kClasses][4];
 #pragma unroll
                     for (int cl = 0; cl < C::kClasses; ++cl)
-                        tmem_ld8(ta + (uint32_t)(cl * C::kN), v[cl]);
+                        tmem_ld4(ta + (uint32_t)(cl * C::kN), v[cl]);
                     tmem_wait_ld();
+                    if (g == kEpiCols / 4 - 1) {
+                        // all sums are in registers: the next chunk's MMAs may start
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&acc_empty);
+                    }
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) {
-                        // sum_w class_w 2^(-8 w) as a pair (each class value an exact integer)
-                        float h = __uint_as_float(v[0][x]), l = 0.0f;
-                        float wt = 1.0f;
-#pragma unroll
-                        for (int cl = 1; cl < C::kClasses; ++cl) {
-                            wt *= 1.0f / (float)(1 << C::kBase);  // 2^-kBase
-                            float t, e2;
-                            two_sum_f(h, __uint_as_float(v[cl][x]) * wt, t, e2);
-                            h = t;
-                            l += e2;
-                        }
+                    for (int x = 0; x < 4; ++x) {
+                        // class_0 + class_1 2^-8 + class_2 2^-16 as a pair: h rounds the
+                        // first two, and h - class_0 is exact (a multiple of 2^-8 below 2^16),
+                        // so the rest of class_1 is too; l is rounded to 2^-17 or better,
+                        // 2^-39 of the largest sum
+                        const float c0 = __uint_as_float(v[0][x]), c1 = __uint_as_float(v[1][x]);
+                        const float h = fmaf(c1, 0x1p-8f, c0);
+                        const float l = fmaf(__uint_as_float(v[2][x]), 0x1p-16f,
+                                             fmaf(c1, 0x1p-8f, c0 - h));
                         const float f =
-                            fA * __shfl_sync(0xffffffffu, fb[(g * 8 + x) / 32], (g * 8 + x) % 32);
-                        const float ph = h * f, pl = l * f;
+                            fA * __shfl_sync(0xffffffffu, fb[(g * 4 + x) / 32], (g * 4 + x) % 32);
                         float sh, se;
-                        two_sum_f(H[g * 8 + x], ph, sh, se);
-                        H[g * 8 + x] = sh;
-                        Lw[(g * 8 + x) * 32] += se + pl;
+                        two_sum_f(H[g * 4 + x], h * f, sh, se);
+                        H[g * 4 + x] = sh;
+                        Lw[(g * 4 + x) * 32] += fmaf(l, f, se);
                     }
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&acc_empty);
             }
             if (!ok) break;
             if (ROT) {
@@ -608,10 +689,7 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
 #pragma unroll
                     for (int x = 0; x < kEpiCols; ++x) {
                         if (j0 + x >= ncol) continue;
-                        if constexpr (sizeof(TO) == 4)
-                            o[(long)x * ldo] = H[x] + Lw[x * 32];  // the pair rounded to FP32
-                        else
-                            o[(long)x * ldo] = widen_int(H[x]) + widen_int(Lw[x * 32]);
+                        o[(long)x * ldo] = H[x] + Lw[x * 32];  // the pair rounded to FP32
                     }
                 }
             } else {
@@ -620,6 +698,107 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
 #pragma unroll
                 for (int x = 0; x < kEpiCols; ++x) o[x] = (double)H[x] + (double)Lw[x * 32];
             }
+        }
+        } else {
+        // ---- epilogue: each chunk's class accumulators into 64-bit integer sums ----
+        long long S[kEpiCols];
+        long cc = 0;  // chunks over all units
+        bool ok = true;
+        // the chunk exponents are loaded one chunk ahead (they do not depend on the MMAs):
+        // this thread's A column, and one of the warp's B columns per lane (lane mod kEpiCols),
+        // whose shifts reach the other lanes by shuffle
+        const long eb_stride = ROT ? eb_ld : ns_pad;
+        for (int u = blockIdx.x; u < nunits && ok; u += ustride) {
+            const Unit w = unit(u);
+            const long colA = (long)w.tb.x * kTile + r;
+            const long colB = (long)w.tb.y * kTile + w.hf * C::kN + hw * kEpiCols + lane % kEpiCols;
+            const int *ebw = EB + colB;
+#pragma unroll
+            for (int x = 0; x < kEpiCols; ++x) S[x] = 0;
+            // largest exponents over the chunks (the rotation's few chunks are looked at here)
+            int xa = kZeroExp, xb = kZeroExp, bad = 0;
+            if (ROT) {
+                for (long c = w.c0; c < w.c1; ++c) {
+                    const int e = EA[c * ea_stride + colA];
+                    xa = max(xa, e == kNonFinite ? kZeroExp : e);
+                    const int f = ebw[c * eb_stride];
+                    xb = max(xb, f == kNonFinite ? kZeroExp : f);
+                }
+            } else {
+                xa = max(xa, EXA[colA]);
+                xb = max(xb, EXB[colB]);
+            }
+            int ea_n = EA[w.c0 * ea_stride + colA], eb_n = ebw[w.c0 * eb_stride];
+            for (long c = w.c0; c < w.c1; ++c, ++cc) {
+                // shifts less one, and flags of chunks holding Inf or NaN (bit 0 this row's, bit 1
+                // the lane's column)
+                if (ea_n == kNonFinite) bad |= 1, ea_n = xa;
+                const int sa = xa - ea_n + drop - 1;
+                if (eb_n == kNonFinite) bad |= 2, eb_n = xb;
+                const int sb = xb - eb_n;
+                if (c + 1 < w.c1) {
+                    ea_n = EA[(c + 1) * ea_stride + colA];
+                    eb_n = ebw[(c + 1) * eb_stride];
+                }
+                ok = mbar_wait(&acc_full, (unsigned)(cc & 1), kWaitLimit) && !abort_flag;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) {
+                    if (lane == 0) fail();
+                    break;
+                }
+                tc_fence_after();
+                // all of the chunk's integers first, so that the next chunk's MMAs may start ...
+                long long T[kEpiCols];
+#pragma unroll
+                for (int g = 0; g < kEpiCols / 4; ++g) {
+                    const uint32_t ta =
+                        tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hw * kEpiCols + g * 4);
+                    uint32_t v[C::kClasses][4];
+#pragma unroll
+                    for (int cl = 0; cl < C::kClasses; ++cl)
+                        tmem_ld4(ta + (uint32_t)(cl * C::kN), v[cl]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        uint32_t vx[C::kClasses];
+#pragma unroll
+                        for (int cl = 0; cl < C::kClasses; ++cl) vx[cl] = v[cl][x];
+                        T[g * 4 + x] = class_sum47(vx);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty);
+                // ... then, beside them, T 2^-(sh + 1), rounded, into the sums
+#pragma unroll
+                for (int x = 0; x < kEpiCols; ++x) {
+                    const int sh = sa + __shfl_sync(0xffffffffu, sb, x);
+                    S[x] += ((T[x] >> min((unsigned)sh, 62u)) + 1) >> 1;
+                }
+            }
+            if (!ok) break;
+            const int unit_e = xa - Dm::kUnit + drop;  // 2^(unit_e + xb): the value of one
+            const long i = (long)w.tb.x * kTile + r;
+            const long j0 = (long)w.tb.y * kTile + w.hf * C::kN + hw * kEpiCols;
+            TO *o = ROT ? out + i + j0 * ldo : nullptr;
+            double *pt = ROT ? nullptr
+                             : part + ((long)w.split * ntiles + w.tile) * kTile * kTile +
+                                   (long)r * kTile + w.hf * C::kN + hw * kEpiCols;
+#pragma unroll
+            for (int x = 0; x < kEpiCols; ++x) {
+                const int sc = unit_e + __shfl_sync(0xffffffffu, xb, x);
+                const int fb = __shfl_sync(0xffffffffu, bad, x);
+                const bool nan = (bad & 1) || (fb & 2);
+                if (ROT) {
+                    if (i >= nrow || j0 + x >= ncol) continue;
+                    o[(long)x * ldo] = nan ? __longlong_as_double(0x7ff8000000000000ll)
+                                           : scaled_to_double(S[x], sc);
+                } else {
+                    pt[x] = nan ? __longlong_as_double(0x7ff8000000000000ll)
+                                : scaled_to_double(S[x], sc);
+                }
+            }
+        }
         }
     }
     tc_fence_before();
@@ -655,9 +834,17 @@ __global__ void k_gram_tc_reduce(const double *__restrict__ part, const int2 *__
 namespace {
 struct TcPlan {
     int ns_pad, nblk, ntiles, nsplit;
+    int drop;  // right shift of a chunk's integer: the chunks of a unit add up below 2^63
     long nstep, nchunk;
     size_t digits_bytes, exps_bytes, part_bytes, tiles_bytes;
 };
+
+int log2_ceil(long n)
+{
+    int b = 0;
+    while ((1L << b) < n) ++b;
+    return b;
+}
 
 template <class C>
 TcPlan tc_plan(long nd, int ns, bool sym)
@@ -683,8 +870,9 @@ TcPlan tc_plan(long nd, int ns, bool sym)
         if (best < 0 || cost < best) best = cost, best_s = s;
     }
     p.nsplit = (int)best_s;
+    p.drop = std::max(1, log2_ceil((p.nchunk + best_s - 1) / best_s));
     p.digits_bytes = (size_t)C::kDigits * p.ns_pad * p.nstep * C::kStep * 2;
-    p.exps_bytes = (size_t)p.nchunk * p.ns_pad * sizeof(int);
+    p.exps_bytes = (size_t)(p.nchunk + 1) * p.ns_pad * sizeof(int);  // then the largest per column
     p.part_bytes = (size_t)p.nsplit * p.ntiles * kTile * kTile * sizeof(double);
     p.tiles_bytes = (size_t)p.ntiles * sizeof(int2);
     return p;
@@ -708,15 +896,49 @@ size_t gram_tc_workspace(long nd, int ns, bool same_operand, bool sym)
 }
 size_t gram_tc47_workspace(long nd, int ns) { return tc_workspace<Tc47>(nd, ns, false, true); }
 
+// 16-byte loads along a column
+template <typename T>
+static bool tc_vec(const T *X, long ld)
+{
+    return ((uintptr_t)X & 15u) == 0 && ld % (long)(16 / sizeof(T)) == 0;
+}
+
 template <class C, typename T>
 static cudaError_t tc_digits(const T *X, long ld, long nd, int ns, const TcPlan &p,
                              __nv_bfloat16 *D, int *E, cudaStream_t st)
 {
     if (p.nchunk > 65535) return cudaErrorInvalidValue;
-    dim3 grid(p.ns_pad / 8, (unsigned)p.nchunk);
-    k_tc_digits<C, T><<<grid, 256, 0, st>>>(X, ld, nd, ns, p.nstep, D, E, p.ns_pad);
+    int *EX = E + p.nchunk * p.ns_pad;
+    const cudaError_t e = cudaMemsetAsync(EX, 0x80, sizeof(int) * (size_t)p.ns_pad, st);
+    if (e != cudaSuccess) return e;
+    dim3 grid(p.ns_pad / (2048 / C::kChunk), (unsigned)p.nchunk);
+    k_tc_digits<C, T><<<grid, 256, 0, st>>>(X, ld, nd, ns, p.nstep, tc_vec(X, ld), D, E, EX,
+                                            p.ns_pad);
     note_launch();
     return cudaGetLastError();
+}
+
+// A digit buffer of nblk column blocks as (16-byte units of a K group's 128 columns taken as
+// 8-byte words, digit of a step, K group of a step), with the box of one CTA's B operand. The
+// box starts at a multiple of its width, so the x coordinate is a multiple of 1 KB.
+template <class C>
+static cudaError_t tc_map(CUtensorMap &m, const __nv_bfloat16 *D, long nblk, long nstep)
+{
+    constexpr int kGroups = C::kStep / 8;
+    PFN_cuTensorMapEncodeTiled_v12000 enc;
+    const cudaError_t e = tensor_map_encoder(enc);
+    if (e != cudaSuccess) return e;
+    const long rows = nblk * nstep * C::kDigits;
+    if (rows > 0x7fffffffL) return cudaErrorInvalidValue;
+    cuuint64_t dims[3] = {kTile * 2, (cuuint64_t)rows, kGroups};
+    cuuint64_t strides[2] = {(cuuint64_t)TcDims<C>::kBlobElems * 2, kTile * 16};
+    cuuint32_t box[3] = {C::kN * 2, C::kDigits, kGroups}, estr[3] = {1, 1, 1};
+    return enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, (void *)D, dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+               ? cudaSuccess
+               : cudaErrorInvalidValue;
 }
 
 // Tile list (host-built, uploaded) and the kernel's shared-memory attribute.
@@ -745,11 +967,14 @@ static cudaError_t tc_run(const TcPlan &p, const __nv_bfloat16 *DA, const int *E
                           double *part, int ns, bool sym, double *G, int *err, cudaStream_t st)
 {
     const int ctas = p.ntiles * p.nsplit * TcDims<C>::kHalves;
-    k_gram_tc<C, false><<<ctas, kThreads, TcDims<C>::kSmemBytes, st>>>(DA, EA, DB, EB, p.ns_pad, p.nstep,
-                                                                tiles, p.ntiles, p.nsplit, part,
-                                                                err);
+    CUtensorMap mapB;
+    cudaError_t e = tc_map<C>(mapB, DB, p.nblk, p.nstep);
+    if (e != cudaSuccess) return e;
+    k_gram_tc<C, false><<<ctas, kThreads, TcDims<C>::kSmemBytes, st>>>(
+        DA, EA, mapB, EB, p.ns_pad, p.nstep, tiles, p.ntiles, p.nsplit, part, p.drop, err,
+        EA + p.nchunk * p.ns_pad, EB + p.nchunk * p.ns_pad);
     note_launch();
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_gram_tc_reduce<<<152 * 4, 256, 0, st>>>(part, tiles, p.ntiles, p.nsplit, ns, sym, G);
     note_launch();
@@ -868,7 +1093,7 @@ RotPlan rot_plan(long nd, int ns)
     p.nchunk = (ns + C::kChunk - 1) / C::kChunk;
     p.nstep = p.nchunk * TcDims<C>::kStepsPerChunk;
     p.da_bytes = (size_t)C::kDigits * p.ns_pad * p.nstep * C::kStep * 2;
-    p.ea_bytes = (size_t)p.nchunk * p.ns_pad * sizeof(int);
+    p.ea_bytes = (size_t)(p.nchunk + 1) * p.ns_pad * sizeof(int);
     p.db_bytes = (size_t)C::kDigits * p.nd_pad * p.nstep * C::kStep * 2;
     p.eb_bytes = (size_t)p.nchunk * p.nd_pad * sizeof(int);
     return p;
@@ -911,8 +1136,12 @@ cudaError_t rotate_tc_impl(const TY *Y, long ldy, long nd, int ns, const double 
         attr_set.store(true, std::memory_order_release);
     }
     {   // A = C: K = Ns rows, M = Ns columns
-        dim3 grid(p.ns_pad / 8, (unsigned)p.nchunk);
-        k_tc_digits<C, double><<<grid, 256, 0, st>>>(Cm, ns, ns, ns, p.nstep, DA, EA, p.ns_pad);
+        dim3 grid(p.ns_pad / (2048 / C::kChunk), (unsigned)p.nchunk);
+        int *EX = EA + p.nchunk * p.ns_pad;  // (not used by the rotation)
+        if ((e = cudaMemsetAsync(EX, 0x80, sizeof(int) * (size_t)p.ns_pad, st)) != cudaSuccess)
+            return e;
+        k_tc_digits<C, double><<<grid, 256, 0, st>>>(Cm, ns, ns, ns, p.nstep, tc_vec(Cm, ns), DA, EA,
+                                                     EX, p.ns_pad);
         note_launch();
     }
     {   // B = Y^T: K = Ns (Y's columns), N = Nd (Y's rows)
@@ -922,11 +1151,13 @@ cudaError_t rotate_tc_impl(const TY *Y, long ldy, long nd, int ns, const double 
         note_launch();
     }
     const unsigned grid = (unsigned)(ctas < 152 ? ctas : 152);  // persistent, one per SM
+    CUtensorMap mapB;
+    if ((e = tc_map<C>(mapB, DA, p.mblk, p.nstep)) != cudaSuccess) return e;
     // A: Y's digits (nblk row blocks, exponent stride nd_pad); B: C's (mblk column blocks,
     // the fastest tile index)
     k_gram_tc<C, true, TO><<<grid, kThreads, TcDims<C>::kSmemBytes, st>>>(
-        DB, EB, DA, EA, p.ns_pad, p.nstep, nullptr, (int)(p.mblk * p.nblk), 1, nullptr, err,
-        p.ns_pad, p.mblk, out, ldo, nd, ns, p.nd_pad);
+        DB, EB, mapB, EA, p.ns_pad, p.nstep, nullptr, (int)(p.mblk * p.nblk), 1, nullptr,
+        std::max(1, log2_ceil(p.nchunk)), err, nullptr, nullptr, p.ns_pad, p.mblk, out, ldo, nd, ns, p.nd_pad);
     note_launch();
     return cudaGetLastError();
 }

@@ -622,26 +622,12 @@ k_batch_stencil_tma(const BatchItem *__restrict__ items, int nitems, const Batch
     }
 }
 
-static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> g_encode{nullptr};
-
-static cudaError_t get_encoder()
-{
-    if (g_encode.load(std::memory_order_acquire)) return cudaSuccess;
-    cudaDriverEntryPointQueryResult q;
-    void *fn = nullptr;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
-                                                     cudaEnableDefault, &q);
-    if (e != cudaSuccess) return e;
-    if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    g_encode.store((PFN_cuTensorMapEncodeTiled_v12000)fn, std::memory_order_release);
-    return cudaSuccess;
-}
-
 // The two tensor maps of a block: with the halo box (the Y_j loads) and with the tile box
 // (the Y_{j-1} loads); maps[0], maps[1].
 cudaError_t encode_f32_maps(const DevHam &H, const float *base, int ncols, long ld, void *maps)
 {
-    cudaError_t e = get_encoder();
+    PFN_cuTensorMapEncodeTiled_v12000 enc;
+    const cudaError_t e = tensor_map_encoder(enc);
     if (e != cudaSuccess) return e;
     CUtensorMap *m = reinterpret_cast<CUtensorMap *>(maps);
     cuuint64_t dims[4] = {(cuuint64_t)H.n0, (cuuint64_t)H.n1, (cuuint64_t)H.n2, (cuuint64_t)ncols};
@@ -650,7 +636,6 @@ cudaError_t encode_f32_maps(const DevHam &H, const float *base, int ncols, long 
     cuuint32_t estr[4] = {1, 1, 1, 1};
     cuuint32_t boxY[4] = {(cuuint32_t)kW, (cuuint32_t)kH, 1, 1};
     cuuint32_t boxP[4] = {(cuuint32_t)kBX, (cuuint32_t)kTY, 1, 1};
-    const PFN_cuTensorMapEncodeTiled_v12000 enc = g_encode.load(std::memory_order_acquire);
     if (enc(&m[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (void *)base, dims, strides, boxY,
                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
@@ -744,7 +729,8 @@ cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev,
                             int ncols, long ld, const StepCoef<float> &cf, int *err,
                             cudaStream_t st)
 {
-    cudaError_t e = get_encoder();
+    PFN_cuTensorMapEncodeTiled_v12000 enc;
+    cudaError_t e = tensor_map_encoder(enc);
     if (e != cudaSuccess) return e;
     static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
     const int smem = kSmemBytes;
@@ -762,9 +748,9 @@ cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev,
                                  (cuuint64_t)ld * 4};
         cuuint32_t box[4] = {bx, by, 1, 1};
         cuuint32_t estr[4] = {1, 1, 1, 1};
-        return g_encode.load(std::memory_order_acquire)(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (void *)base, dims, strides, box,
-                        estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (void *)base, dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     };
     CUtensorMap mapY, mapP;
     if (encode(&mapY, Y, kW, kH) != CUDA_SUCCESS) return cudaErrorInvalidValue;

@@ -1,14 +1,33 @@
 // tma.cuh -- inline-PTX helpers for TMA tile loads and mbarriers (sm_90+ / sm_103a).
 //
-// Only what the stencil kernels use: mbarrier init / expect-tx / bounded parity wait,
-// and the 4-D tiled cp.async.bulk.tensor load into this CTA's shared memory. Every wait
+// Only what the stencil and contraction kernels use: mbarrier init / expect-tx / bounded parity
+// wait, and the 4-D and 3-D tiled cp.async.bulk.tensor loads into this CTA's shared memory. Every wait
 // is bounded by the caller (no unbounded spin).
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <cudaTypedefs.h>
+#include <atomic>
 #include <cstdint>
 
 namespace sparc {
+
+// cuTensorMapEncodeTiled of the installed driver (looked up once per process).
+inline cudaError_t tensor_map_encoder(PFN_cuTensorMapEncodeTiled_v12000 &enc)
+{
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> known{nullptr};
+    enc = known.load(std::memory_order_acquire);
+    if (enc) return cudaSuccess;
+    cudaDriverEntryPointQueryResult q;
+    void *fn = nullptr;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
+                                                           cudaEnableDefault, &q);
+    if (e != cudaSuccess) return e;
+    if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
+    enc = (PFN_cuTensorMapEncodeTiled_v12000)fn;
+    known.store(enc, std::memory_order_release);
+    return cudaSuccess;
+}
 
 __device__ __forceinline__ unsigned smem_u32(const void *p)
 {
@@ -92,6 +111,17 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, u
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
         " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
         "l"((unsigned long long)map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w)
+        : "memory");
+}
+
+// 3-D tiled load.
+__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar,
+                                            int x, int y, int z)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
+        "l"((unsigned long long)map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
         : "memory");
 }
 
@@ -185,6 +215,15 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
                    "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+
+// Four of them.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr)
                  : "memory");
 }
