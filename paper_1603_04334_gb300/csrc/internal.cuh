@@ -381,7 +381,8 @@ cudaError_t density(const T *X, long ld, int ncols, long nd, const double *g, do
                     double *rho, cudaStream_t st);
 // Weights w~_p of Eq. (gradient:approximate) for radius n_o (1/h included), zero beyond.
 struct GradCoef {
-    double w[kRadius + 1];
+    int iw[kRadius + 1];  // whole numbers; iw[p] scale is the weight of x(s + p) - x(s - p)
+    double scale;
 };
 GradCoef grad_coef(int radius, double h);
 // Non-local force of Eq. (NonlocForce:Discrete): f (3 natoms) from the columns X, occupations
