@@ -336,21 +336,20 @@ cudaError_t mbar_selftest(int *err, cudaStream_t st);
 
 // ---- lanczos.cu -------------------------------------------------------------------
 constexpr int kDotBlocks = 608;
-// r = <x, y> (FP64, deterministic two-level reduction); part: kDotBlocks doubles.
-cudaError_t dot_f64(const double *x, const double *y, long n, double *part, double *r,
-                    cudaStream_t st);
+// *r = <x, y> or 1 / sqrt(<x, y>) (FP64, deterministic two-level reduction); part: kDotBlocks
+// doubles, ticket: zero before the first call (and left so).
+cudaError_t dot_f64(const double *x, const double *y, long n, double *part, unsigned *ticket,
+                    bool rsqrt, double *r, cudaStream_t st);
 cudaError_t lanczos_start(double *v, long n, unsigned long long seed, cudaStream_t st);
-// v *= 1/sqrt(*nrm2)
-cudaError_t scale_rsqrt(double *v, long n, const double *nrm2, cudaStream_t st);
-// w = w - alpha[j] v - beta[j-1] vp   (beta term skipped when j == 0); skipped if *stop
+// v *= *f; *b raised to the column bound of the result
+cudaError_t lanczos_scale(double *v, long n, const double *f, unsigned *b, cudaStream_t st);
+// w -= alpha_j v + beta_{j-1} vp; beta_j = ||w||, *inv = 1 / beta_j, *stop
 cudaError_t lanczos_orth(double *w, const double *v, const double *vp, long n,
-                         const double *alpha, const double *beta, int j, const int *stop,
-                         cudaStream_t st);
-// beta[j] = sqrt(*nrm2); if beta[j] == 0 or non-finite: *stop = j+1 (once)
-cudaError_t lanczos_beta(double *beta, int j, const double *nrm2, int *stop, cudaStream_t st);
-// vp = v; v = w / beta[j] (skipped if *stop)
-cudaError_t lanczos_next(double *v, double *vp, const double *w, long n, const double *beta,
-                         int j, const int *stop, cudaStream_t st);
+                         const double *alpha, double *beta, int j, double *part, unsigned *ticket,
+                         double *inv, int *stop, cudaStream_t st);
+// vp = v, v = w *inv; b: the bounds of the old v and (raised) of the new one
+cudaError_t lanczos_next(double *v, double *vp, const double *w, long n, const double *inv,
+                         unsigned *b, const int *stop, cudaStream_t st);
 // T (k x k) from alpha, beta, using keff = (*stop ? *stop : k)
 cudaError_t lanczos_tridiag(const double *alpha, const double *beta, int k, const int *stop,
                             double *T, int *keff, cudaStream_t st);

@@ -9,6 +9,15 @@
 // Start vector: v0[p] = u(splitmix64(seed ^ p)) - 0.5 with u(z) = (z >> 11) 2^-53, the
 // SplitMix64 generator as published by Vigna (mixing constants of Stafford's Mix13).
 // Dot products are two-level fixed-order reductions, so results are reproducible.
+//
+// On one vector every kernel is short (a 64^3 step's six take 5 to 20 us each), so a step is as
+// few launches as its global sums allow: apply, <w, v>, the subtraction with ||w||^2, the scaling.
+// The CTA that finishes last adds the partial sums and forms the scalars that follow from them
+// (a reciprocal or square root in every thread holds the FP64 pipe longer than the vector
+// update itself), and the scaling takes the new vector's magnitude bound for the next apply. Ten
+// steps on 64^3, 20 atoms: 0.95 ms as eleven launches a step with a separate bound pass (20 us)
+// and reduction launches, 0.62 ms so.
+#include "fx.cuh"
 #include "internal.cuh"
 
 namespace sparc {
@@ -36,14 +45,13 @@ cudaError_t lanczos_start(double *v, long n, unsigned long long seed, cudaStream
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256)
-k_dot_part(const double *__restrict__ x, const double *__restrict__ y, long n, double *part)
+namespace {
+// This CTA's partial sum into part; true in the CTA that stored last, with the sum of all the
+// partials (in a fixed order) in `total` of thread 0. ticket returns to zero.
+__device__ __forceinline__ bool sum_by_last(double s, double *part, unsigned *ticket, double &total)
 {
     __shared__ double red[8];
-    double s = 0.0;
-    for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-         p += (long)gridDim.x * blockDim.x)
-        s += x[p] * y[p];
+    __shared__ bool last;
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -51,100 +59,148 @@ k_dot_part(const double *__restrict__ x, const double *__restrict__ y, long n, d
         double t = 0.0;
         for (int w = 0; w < 8; ++w) t += red[w];
         part[blockIdx.x] = t;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
-}
-
-__global__ void __launch_bounds__(256) k_dot_final(const double *part, int nb, double *r)
-{
-    __shared__ double red[8];
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nb; b += 256) s += part[b];
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    s = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) s += __ldcg(part + b);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < 8; ++w) t += red[w];
-        *r = t;
+        total = 0.0;
+        for (int w = 0; w < 8; ++w) total += red[w];
+        *ticket = 0u;
+    }
+    return true;
+}
+
+// Raises *b by the largest high word m of the CTA's threads (all CTAs raise one word: by warps,
+// the reads of it took longer than the vector update).
+__device__ __forceinline__ void raise_by_cta(unsigned *b, unsigned m)
+{
+    __shared__ unsigned red[8];
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+        if (m) raise_bound(b, m);
     }
 }
+}  // namespace
 
-cudaError_t dot_f64(const double *x, const double *y, long n, double *part, double *r,
-                    cudaStream_t st)
+// *r = <x, y>, or 1 / sqrt(<x, y>) (RSQRT).
+template <bool RSQRT>
+__global__ void __launch_bounds__(256)
+k_dot(const double *__restrict__ x, const double *__restrict__ y, long n, double *part,
+      unsigned *ticket, double *r)
 {
-    k_dot_part<<<kDotBlocks, 256, 0, st>>>(x, y, n, part);
-    note_launch();
-    k_dot_final<<<1, 256, 0, st>>>(part, kDotBlocks, r);
-    note_launch();
-    return cudaGetLastError();
-}
-
-__global__ void k_scale_rsqrt(double *v, long n, const double *nrm2)
-{
-    const double f = 1.0 / sqrt(*nrm2);
+    double s = 0.0, t;
     for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
          p += (long)gridDim.x * blockDim.x)
-        v[p] *= f;
+        s += x[p] * y[p];
+    if (sum_by_last(s, part, ticket, t) && threadIdx.x == 0) *r = RSQRT ? 1.0 / sqrt(t) : t;
 }
 
-cudaError_t scale_rsqrt(double *v, long n, const double *nrm2, cudaStream_t st)
+cudaError_t dot_f64(const double *x, const double *y, long n, double *part, unsigned *ticket,
+                    bool rsqrt, double *r, cudaStream_t st)
 {
-    k_scale_rsqrt<<<152 * 8, 256, 0, st>>>(v, n, nrm2);
+    if (rsqrt)
+        k_dot<true><<<kDotBlocks, 256, 0, st>>>(x, y, n, part, ticket, r);
+    else
+        k_dot<false><<<kDotBlocks, 256, 0, st>>>(x, y, n, part, ticket, r);
     note_launch();
     return cudaGetLastError();
 }
 
-__global__ void k_lanczos_orth(double *w, const double *v, const double *vp, long n,
-                               const double *alpha, const double *beta, int j, const int *stop)
+// v *= *f, *b raised to the new values' bound
+__global__ void __launch_bounds__(256)
+k_lanczos_scale(double *__restrict__ v, long n, const double *f, unsigned *b)
+{
+    const double s = *f;
+    unsigned m = 0u;
+#pragma unroll 4
+    for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
+         p += (long)gridDim.x * blockDim.x) {
+        const double x = v[p] * s;
+        v[p] = x;
+        m = max(m, abs_hi_word(x));
+    }
+    raise_by_cta(b, m);
+}
+
+cudaError_t lanczos_scale(double *v, long n, const double *f, unsigned *b, cudaStream_t st)
+{
+    k_lanczos_scale<<<152 * 2, 256, 0, st>>>(v, n, f, b);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// w -= alpha_j v + beta_{j-1} vp; beta_j = ||w||, inv = 1 / beta_j; stop = j + 1 where beta_j is
+// zero or not finite.
+__global__ void __launch_bounds__(256)
+k_lanczos_orth(double *__restrict__ w, const double *__restrict__ v,
+               const double *__restrict__ vp, long n, const double *alpha,
+               double *beta, int j, double *part, unsigned *ticket, double *inv, int *stop)
 {
     if (*stop) return;
     const double a = alpha[j];
     const double b = j > 0 ? beta[j - 1] : 0.0;
-    for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-         p += (long)gridDim.x * blockDim.x)
-        w[p] = w[p] - a * v[p] - b * vp[p];
-}
-
-cudaError_t lanczos_orth(double *w, const double *v, const double *vp, long n,
-                         const double *alpha, const double *beta, int j, const int *stop,
-                         cudaStream_t st)
-{
-    k_lanczos_orth<<<152 * 8, 256, 0, st>>>(w, v, vp, n, alpha, beta, j, stop);
-    note_launch();
-    return cudaGetLastError();
-}
-
-__global__ void k_lanczos_beta(double *beta, int j, const double *nrm2, int *stop)
-{
-    if (*stop) return;
-    const double b = sqrt(*nrm2);
-    beta[j] = b;
-    if (!(b > 0.0) || !isfinite(b)) *stop = j + 1;
-}
-
-cudaError_t lanczos_beta(double *beta, int j, const double *nrm2, int *stop, cudaStream_t st)
-{
-    k_lanczos_beta<<<1, 1, 0, st>>>(beta, j, nrm2, stop);
-    note_launch();
-    return cudaGetLastError();
-}
-
-__global__ void k_lanczos_next(double *v, double *vp, const double *w, long n,
-                               const double *beta, int j, const int *stop)
-{
-    if (*stop) return;
-    const double f = 1.0 / beta[j];
+    double s = 0.0, t;
     for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
          p += (long)gridDim.x * blockDim.x) {
-        vp[p] = v[p];
-        v[p] = w[p] * f;
+        double x = w[p] - a * v[p];
+        if (j > 0) x -= b * vp[p];  // (vp is not set before the first step)
+        w[p] = x;
+        s += x * x;
+    }
+    if (sum_by_last(s, part, ticket, t) && threadIdx.x == 0) {
+        const double bj = sqrt(t);
+        beta[j] = bj;
+        *inv = 1.0 / bj;
+        if (!(bj > 0.0) || !isfinite(bj)) *stop = j + 1;
     }
 }
 
-cudaError_t lanczos_next(double *v, double *vp, const double *w, long n, const double *beta,
-                         int j, const int *stop, cudaStream_t st)
+cudaError_t lanczos_orth(double *w, const double *v, const double *vp, long n,
+                         const double *alpha, double *beta, int j, double *part, unsigned *ticket,
+                         double *inv, int *stop, cudaStream_t st)
 {
-    k_lanczos_next<<<152 * 8, 256, 0, st>>>(v, vp, w, n, beta, j, stop);
+    k_lanczos_orth<<<kDotBlocks, 256, 0, st>>>(w, v, vp, n, alpha, beta, j, part, ticket, inv, stop);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// vp = v, v = w inv; b[1] raised to the new v's bound (after a stop v and its bound b[0] stay)
+__global__ void __launch_bounds__(256)
+k_lanczos_next(double *__restrict__ v, double *__restrict__ vp, const double *__restrict__ w, long n, const double *inv, unsigned *b,
+               const int *stop)
+{
+    if (*stop) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) b[1] = b[0];
+        return;
+    }
+    const double f = *inv;
+    unsigned m = 0u;
+#pragma unroll 4
+    for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
+         p += (long)gridDim.x * blockDim.x) {
+        vp[p] = v[p];
+        const double x = w[p] * f;
+        v[p] = x;
+        m = max(m, abs_hi_word(x));
+    }
+    raise_by_cta(b + 1, m);
+}
+
+cudaError_t lanczos_next(double *v, double *vp, const double *w, long n, const double *inv,
+                         unsigned *b, const int *stop, cudaStream_t st)
+{
+    k_lanczos_next<<<152 * 2, 256, 0, st>>>(v, vp, w, n, inv, b, stop);
     note_launch();
     return cudaGetLastError();
 }

@@ -11,6 +11,8 @@
 #include "fx.cuh"
 #include "internal.cuh"
 
+#include <type_traits>
+
 namespace sparc {
 
 template <typename T>
@@ -227,7 +229,7 @@ cudaError_t chi_fixed(int natoms, const int *atom_ptr, const double *chi, int4 *
 // mixed-precision Rayleigh-Ritz step applies H in FP64). bY: the columns' bounds.
 // Grid as k_project: x = atom (in the spatial order), y = column block.
 template <typename T, int CB, int NT>
-__global__ void __launch_bounds__(NT, 3)
+__global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1)
 k_project_fx(const T *__restrict__ Y, long ld, int ncols, const int *__restrict__ atom_ptr,
              const int *__restrict__ idx, const int4 *__restrict__ chi_q,
              const int *__restrict__ chi_F, const unsigned *__restrict__ bY, double alpha,
@@ -325,12 +327,25 @@ static cudaError_t project_fx(const DevHam &H, const T *Y, int ncols, long ld, d
                               const unsigned *bY, float2 *C, cudaStream_t st)
 {
     if (H.natoms == 0 || ncols <= 0) return cudaSuccess;
-    constexpr int CB = 2, NT = 256;
-    dim3 grid(H.natoms, (ncols + CB - 1) / CB);
-    if (grid.y > 65535 || !bY) return cudaErrorInvalidValue;
-    k_project_fx<T, CB, NT><<<grid, NT, 0, st>>>(Y, ld, ncols, H.atom_ptr, H.idx, H.chi_q,
-                                                 H.chi_F, bY, alpha, C, H.proj_order);
-    note_launch();
+    if (!bY) return cudaErrorInvalidValue;
+    auto launch = [&](auto cb, auto nt) {
+        constexpr int CB = decltype(cb)::value, NT = decltype(nt)::value;
+        const dim3 grid(H.natoms, (ncols + CB - 1) / CB);
+        if (grid.y > 65535) return cudaErrorInvalidValue;
+        k_project_fx<T, CB, NT><<<grid, NT, 0, st>>>(Y, ld, ncols, H.atom_ptr, H.idx, H.chi_q,
+                                                     H.chi_F, bY, alpha, C, H.proj_order);
+        note_launch();
+        return cudaSuccess;
+    };
+    // Two columns a CTA of 256 threads, three CTAs an SM. A single vector (the Lanczos steps) has
+    // one CTA per atom, whose time is its trips over the support: 1024 threads make a quarter of
+    // them (20 atoms, 4189 entries each: 18.9 us with 256 threads and two columns, 11.5 us so).
+    cudaError_t e;
+    if (ncols == 1)
+        e = launch(std::integral_constant<int, 1>{}, std::integral_constant<int, 1024>{});
+    else
+        e = launch(std::integral_constant<int, 2>{}, std::integral_constant<int, 256>{});
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -496,16 +511,17 @@ cudaError_t scatter_f32(const DevHam &H, const float *Cs, float *out, int ncols,
 namespace {
 constexpr int kScatDfNodes = 256;
 constexpr int kScatDfCols = 4;    // columns per group
-constexpr int kScatDfGroups = 4;  // column groups per thread
+constexpr int kScatDfGroups = 4;  // column groups per thread, most
 }  // namespace
 
+template <int NG>
 __global__ void __launch_bounds__(kScatDfNodes, 4)
 k_scatter_df(double *out, long ld, int ncols, long nuniq, const int *__restrict__ uniq_node,
              const int *__restrict__ uniq_ptr, const int *__restrict__ nl_atom,
              const float2 *__restrict__ g, const float2 *__restrict__ Cs, unsigned *bOut)
 {
     constexpr int K = kScatDfCols;
-    const int c0 = blockIdx.x * K * kScatDfGroups;
+    const int c0 = blockIdx.x * K * NG;
     // both loops are uniform over the CTA: every lane reaches the bound reductions
     for (long ub = blockIdx.y; ub * kScatDfNodes < nuniq; ub += gridDim.y) {
         const long u = ub * kScatDfNodes + threadIdx.x;
@@ -520,11 +536,11 @@ k_scatter_df(double *out, long ld, int ncols, long nuniq, const int *__restrict_
 #pragma unroll
         for (int k = 0; k < K; ++k) o[k] = (live && c0 + k < ncols) ? ob[(long)(c0 + k) * ld] : 0.0;
 #pragma unroll 1
-        for (int gi = 0; gi < kScatDfGroups; ++gi) {
+        for (int gi = 0; gi < NG; ++gi) {
             const int cg = c0 + gi * K;
             if (cg >= ncols) break;
             const int cn = cg + K;
-            const bool more = gi + 1 < kScatDfGroups && cn < ncols;
+            const bool more = gi + 1 < NG && cn < ncols;
             double on[K];
 #pragma unroll
             for (int k = 0; k < K; ++k)
@@ -570,10 +586,21 @@ cudaError_t scatter_f64_df(const DevHam &H, const float2 *Cs, double *out, int n
 {
     if (H.natoms == 0 || H.nuniq == 0 || ncols <= 0) return cudaSuccess;
     const long nb = (H.nuniq + kScatDfNodes - 1) / kScatDfNodes;
-    constexpr int cpb = kScatDfCols * kScatDfGroups;
-    dim3 grid((unsigned)((ncols + cpb - 1) / cpb), (unsigned)(nb < 65535 ? nb : 65535));
-    k_scatter_df<<<grid, kScatDfNodes, 0, st>>>(out, ld, ncols, H.nuniq, H.uniq_node, H.uniq_ptr,
-                                              H.nl_atom, H.nl_gdf, Cs, bOut);
+    auto launch = [&](auto ng) {
+        constexpr int NG = decltype(ng)::value, cpb = kScatDfCols * NG;
+        dim3 grid((unsigned)((ncols + cpb - 1) / cpb), (unsigned)(nb < 65535 ? nb : 65535));
+        k_scatter_df<NG><<<grid, kScatDfNodes, 0, st>>>(out, ld, ncols, H.nuniq, H.uniq_node,
+                                                        H.uniq_ptr, H.nl_atom, H.nl_gdf, Cs, bOut);
+    };
+    // A thread's groups follow one another, so while a launch of one group a thread is a few
+    // waves of the chip (four CTAs an SM), it is the shorter: 24^3 x 12, 4 atoms 13.5 -> 7.6 us;
+    // 70 x 61 x 53 x 33, 12 atoms (2.3 waves) 26.3 -> 18.6 us; 96^3 x 128, 40 atoms (27 waves)
+    // 133 us with four groups, whose output reads run ahead, 146 us with one.
+    const long groups = (ncols + kScatDfCols - 1) / kScatDfCols;
+    if (nb * groups <= 4 * 4 * 152)
+        launch(std::integral_constant<int, 1>{});
+    else
+        launch(std::integral_constant<int, kScatDfGroups>{});
     note_launch();
     return cudaGetLastError();
 }

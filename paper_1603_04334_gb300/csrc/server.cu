@@ -503,7 +503,7 @@ size_t sparc_request_bytes(const sparc_request *q)
         b += sizeof(unsigned) * ((size_t)(q->degree + 1) * ns + (size_t)ns);
     }
     b += sizeof(double) * (4 * (size_t)ns * ns + 2 * (size_t)ns + (size_t)dense_work_elems(ns));
-    b += sizeof(double) * (3 * (size_t)nd + kDotBlocks + 4096);
+    b += sizeof(double) * (3 * (size_t)nd + kDotBlocks + 8704);
     // the request's two orbital blocks
     b += 2 * es * (size_t)nd * ns;
     return b + b / 16;  // allocation granularity

@@ -991,26 +991,27 @@ sparc_status sparc_lanczos_bounds(sparc_ctx *ctx, int ksteps, unsigned long long
         return fail(ctx, SPARC_ERR_ARG, "ksteps must be in 1..%d (got %d)", kMaxLanczos, ksteps);
     const long nd = ctx->H.nd;
     const int K = kMaxLanczos;
-    const size_t nsc = 4 * (size_t)K + 8 + 2 * (size_t)K * K;
+    const size_t nsc = 5 * (size_t)K + 8 + 2 * (size_t)K * K;
     const size_t tot = 3 * (size_t)nd + (size_t)kDotBlocks + nsc;
     TRY(ensure(ctx, ctx->lz, ctx->lz_bytes, tot * sizeof(double)));
     double *v = (double *)ctx->lz, *vp = v + nd, *w = vp + nd, *part = w + nd;
-    double *alpha = part + kDotBlocks, *beta = alpha + K, *nrm2 = beta + K, *outb = nrm2 + 2,
-           *ev = outb + 4, *T = ev + K + 2, *Q = T + (size_t)K * K;
+    // beta (K), then the ticket and the K + 1 vectors' bounds in K doubles: zeroed together
+    double *alpha = part + kDotBlocks, *beta = alpha + K, *zero_end = beta + 2 * K,
+           *inv = zero_end, *outb = inv + 2, *ev = outb + 4, *T = ev + K + 2,
+           *Q = T + (size_t)K * K;
+    unsigned *ticket = (unsigned *)(beta + K), *bnd = ticket + 1;
+    static_assert(2 * kMaxLanczos >= kMaxLanczos + 2, "ticket and bounds fit K doubles");
     int *stop = ctx->flags + 4, *keff = ctx->flags + 5, *status = ctx->flags + 6;
     CK(cudaMemsetAsync(ctx->flags + 4, 0, sizeof(int) * 3, ctx->st));
-    CK(cudaMemsetAsync(vp, 0, sizeof(double) * nd, ctx->st));
-    CK(cudaMemsetAsync(beta, 0, sizeof(double) * K, ctx->st));
+    CK(cudaMemsetAsync(beta, 0, (size_t)((char *)zero_end - (char *)beta), ctx->st));
     { PHASE(SPARC_PHASE_OTHER); CK(lanczos_start(v, nd, seed, ctx->st)); }
-    { PHASE(SPARC_PHASE_OTHER); CK(dot_f64(v, v, nd, part, nrm2, ctx->st)); }
-    { PHASE(SPARC_PHASE_OTHER); CK(scale_rsqrt(v, nd, nrm2, ctx->st)); }
+    { PHASE(SPARC_PHASE_OTHER); CK(dot_f64(v, v, nd, part, ticket, true, inv, ctx->st)); }
+    { PHASE(SPARC_PHASE_OTHER); CK(lanczos_scale(v, nd, inv, bnd, ctx->st)); }
     for (int j = 0; j < ksteps; ++j) {
-        TRY(step_f64(ctx, v, nullptr, w, 1, nd, 1.0, 0.0, 0.0));
-        { PHASE(SPARC_PHASE_OTHER); CK(dot_f64(w, v, nd, part, alpha + j, ctx->st)); }
-        { PHASE(SPARC_PHASE_OTHER); CK(lanczos_orth(w, v, vp, nd, alpha, beta, j, stop, ctx->st)); }
-        { PHASE(SPARC_PHASE_OTHER); CK(dot_f64(w, w, nd, part, nrm2, ctx->st)); }
-        { PHASE(SPARC_PHASE_OTHER); CK(lanczos_beta(beta, j, nrm2, stop, ctx->st)); }
-        { PHASE(SPARC_PHASE_OTHER); CK(lanczos_next(v, vp, w, nd, beta, j, stop, ctx->st)); }
+        TRY(step_f64(ctx, v, nullptr, w, 1, nd, 1.0, 0.0, 0.0, bnd + j));
+        { PHASE(SPARC_PHASE_OTHER); CK(dot_f64(w, v, nd, part, ticket, false, alpha + j, ctx->st)); }
+        { PHASE(SPARC_PHASE_OTHER); CK(lanczos_orth(w, v, vp, nd, alpha, beta, j, part, ticket, inv, stop, ctx->st)); }
+        { PHASE(SPARC_PHASE_OTHER); CK(lanczos_next(v, vp, w, nd, inv, bnd + j, stop, ctx->st)); }
     }
     { PHASE(SPARC_PHASE_OTHER); CK(lanczos_tridiag(alpha, beta, ksteps, stop, T, keff, ctx->st)); }
     { PHASE(SPARC_PHASE_DENSE); CK(dense_syev(T, ksteps, keff, ev, Q, status, ctx->st)); }
