@@ -356,60 +356,72 @@ __device__ __forceinline__ long long class_sum47(const uint32_t (&v)[6])
 
 // Digits of the transposed operand: B = Y^T for the rotation, so the K dimension runs over
 // Y's columns and each Y row gets its own exponent per chunk of kChunk columns. CTA: 32
-// rows (lanes) x the chunk's kChunk / 8 groups of 8 columns (warps): loads are coalesced
-// across lanes, the row's largest entry is reduced through shared memory, and each thread
-// writes its 8 values of a digit as one 16-byte store (the 8 K-adjacent elements of a core
-// matrix row are contiguous, and the 32 rows of a warp fill 512 contiguous bytes). Rows past
-// nd and columns past ns are zero.
+// rows (lanes) x 16 warps, each with one or two groups of 8 columns: loads are coalesced
+// across lanes, the row's largest entry (as the word that holds its exponent) is found by shared
+// memory maxima, and each thread writes its 8 values of a digit as one 16-byte store (the 8
+// K-adjacent elements of a core matrix row are contiguous, and the 32 rows of a warp fill 512
+// contiguous bytes). Rows past nd and columns past ns are zero. Bounded by its reads and writes;
+// with every thread reading all warps' 64-bit maxima, and the 256-column chunks in CTAs of 1024
+// threads of which one fits an SM, 2.7 ms for half of 128^3 x 512 FP64 to 23 bits, 1.23 ms so.
+constexpr int kDigitTWarps = 16;
 template <class C, typename T>
-__global__ void __launch_bounds__(32 * (C::kChunk / 8))
+__global__ void __launch_bounds__(32 * kDigitTWarps)
 k_tc_digits_t(const T *__restrict__ Y, long ld, long nd, int ns, long nstep,
               __nv_bfloat16 *__restrict__ D, int *__restrict__ E, long nd_pad)
 {
     using B = FBits<T>;
     using U = typename B::U;
-    constexpr int G = C::kChunk / 8;  // column groups (warps)
-    __shared__ U red[G][32];
-    __shared__ int bad_s[G][32];
+    constexpr int P = C::kChunk / 8 / kDigitTWarps;  // column groups of a thread
+    static_assert(P * 8 * kDigitTWarps == C::kChunk, "whole groups");
+    constexpr int kWordShift = 8 * (int)sizeof(T) - 32;
+    __shared__ unsigned red[32];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    if (g == 0) red[lane] = 0u;
     const long row = (long)blockIdx.x * 32 + lane;
     const long chunk = blockIdx.y;
-    const int kb = (int)(chunk * C::kChunk) + g * 8;  // first column of this thread's group
     const bool live = row < nd;
-    T x[8];
+    T x[P][8];
     U mx = 0;
-    int bad = 0;
-    const U inf = (U)B::kExpMask << B::kMant;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        x[t] = (live && kb + t < ns) ? Y[row + (long)(kb + t) * ld] : (T)0;
-        const U m = B::mag(x[t]);
-        bad |= m >= inf;
-        mx = m > mx ? m : mx;
+    for (int q = 0; q < P; ++q) {
+        const int kb = (int)(chunk * C::kChunk) + (g + kDigitTWarps * q) * 8;
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+            x[q][t] = (live && kb + t < ns) ? Y[row + (long)(kb + t) * ld] : (T)0;
     }
-    red[g][lane] = mx;
-    bad_s[g][lane] = bad;
+#pragma unroll
+    for (int q = 0; q < P; ++q)
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const U m = B::mag(x[q][t]);
+            mx = m > mx ? m : mx;
+        }
+    // the word with the exponent; a value below its last bit counts as that bit (not zero)
+    const unsigned word = (unsigned)(mx >> kWordShift);
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < G; ++q) {
-        mx = red[q][lane] > mx ? red[q][lane] : mx;
-        bad |= bad_s[q][lane];
-    }
-    const int e = chunk_exponent<T>(mx);
+    atomicMax(&red[lane], word ? word : mx != 0 ? 1u : 0u);
+    __syncthreads();
+    const unsigned top = red[lane];
+    const bool bad = top >= (unsigned)(((U)B::kExpMask << B::kMant) >> kWordShift);
+    const int e = top == 1u ? 2 - B::kBias : chunk_exponent<T>((U)top << kWordShift);
     if (g == 0 && row < nd_pad) E[chunk * nd_pad + row] = bad ? kNonFinite : e;
     if (row >= nd_pad) return;
-    unsigned long long N[8];
-    unsigned neg = 0u;
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        N[t] = bad ? 0ull : grid_value<C, T>(B::mag(x[t]), e);
-        neg |= (B::neg(x[t]) ? 1u : 0u) << t;
-    }
-    // the 8 columns kb .. kb+7 lie in one K-step (kStep is a multiple of 8) and one core
     const int cb = (int)(row >> 7), c = (int)(row & 127);
-    store_digits<C>(N, neg,
-                    D + blob_offset<C>(cb, kb / C::kStep, 0, nstep) + in_blob(kb % C::kStep, c),
-                    TcDims<C>::kBlobElems);
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+        unsigned long long N[8];
+        unsigned neg = 0u;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            N[t] = bad ? 0ull : grid_value<C, T>(B::mag(x[q][t]), e);
+            neg |= (B::neg(x[q][t]) ? 1u : 0u) << t;
+        }
+        // the 8 columns kb .. kb+7 lie in one K-step (kStep is a multiple of 8) and one core
+        const int kb = (int)(chunk * C::kChunk) + (g + kDigitTWarps * q) * 8;
+        store_digits<C>(N, neg,
+                        D + blob_offset<C>(cb, kb / C::kStep, 0, nstep) + in_blob(kb % C::kStep, c),
+                        TcDims<C>::kBlobElems);
+    }
 }
 
 // tiles[t] = (A column block, B column block); a tile is computed by kHalves CTAs, each
@@ -1146,7 +1158,7 @@ cudaError_t rotate_tc_impl(const TY *Y, long ldy, long nd, int ns, const double 
     }
     {   // B = Y^T: K = Ns (Y's columns), N = Nd (Y's rows)
         dim3 grid((unsigned)(p.nd_pad / 32), (unsigned)p.nchunk);
-        k_tc_digits_t<C, TY><<<grid, 32 * (C::kChunk / 8), 0, st>>>(Y, ldy, nd, ns, p.nstep, DB,
+        k_tc_digits_t<C, TY><<<grid, 32 * kDigitTWarps, 0, st>>>(Y, ldy, nd, ns, p.nstep, DB,
                                                                     EB, p.nd_pad);
         note_launch();
     }

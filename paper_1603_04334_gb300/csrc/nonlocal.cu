@@ -141,27 +141,30 @@ cudaError_t batch_project(const BatchItem *items, int nitems, const BatchNonloca
     return cudaGetLastError();
 }
 
-template <typename T, typename TC, bool ILV>
-static cudaError_t project(const DevHam &H, const T *Y, int ncols, long ld, const TC *chi,
-                           TC *C, TC alpha, cudaStream_t st)
-{
-    if (H.natoms == 0 || ncols <= 0) return cudaSuccess;
-    // FP32 accumulators leave room for 16 columns per CTA (32 loads of Y in flight per
-    // thread); FP64 ones for 8
-    constexpr int CB = sizeof(TC) == 4 ? 16 : 8, NT = 256;
-    dim3 grid(H.natoms, (ncols + CB - 1) / CB);
-    if (grid.y > 65535) return cudaErrorInvalidValue;
-    k_project<T, TC, CB, NT, ILV>
-        <<<grid, NT, 0, st>>>(Y, ld, ncols, H.atom_ptr, H.idx, chi, C, alpha, H.proj_order);
-    note_launch();
-    return cudaGetLastError();
-}
-
+// Columns per CTA: 16 (32 loads of Y in flight per thread, the support's tables read once for
+// them) while that gives every SM its two CTAs; below, fewer, so that the launch reaches all SMs
+// (12 atoms x 40 columns: 20.5 us with 36 CTAs of 16 columns, 13.2 us with 120 of 4;
+// 400 atoms x 256 columns of 160^3: 0.83 ms with 16, 0.95 ms with 4). A column's sums do not
+// depend on the choice.
 cudaError_t project_f32(const DevHam &H, const float *Y, int ncols, long ld, double alpha,
                         float *C, cudaStream_t st)
 {
-    return project<float, float, true>(H, Y, ncols, ld, H.chi_f, C, (float)alpha, st);
+    if (H.natoms == 0 || ncols <= 0) return cudaSuccess;
+    constexpr int NT = 256;
+    auto launch = [&](auto cb) {
+        constexpr int CB = decltype(cb)::value;
+        const dim3 grid(H.natoms, (ncols + CB - 1) / CB);
+        if (grid.y > 65535) return cudaErrorInvalidValue;
+        k_project<float, float, CB, NT, true><<<grid, NT, 0, st>>>(
+            Y, ld, ncols, H.atom_ptr, H.idx, H.chi_f, C, (float)alpha, H.proj_order);
+        note_launch();
+        return cudaGetLastError();
+    };
+    if ((long)H.natoms * ((ncols + 15) / 16) >= 2 * 152)
+        return launch(std::integral_constant<int, 16>{});
+    return launch(std::integral_constant<int, 4>{});
 }
+
 // ---- FP64 projection in exact integer arithmetic ---------------------------------------
 // Each column of Y is put on its 49-bit grid (fx_split: y = 2^(E-49) (d 2^23 + r), E from
 // the column bound) and each projector l of atom J on a 46-bit grid of its own (chi =
@@ -363,7 +366,7 @@ cudaError_t project_f32in_f64(const DevHam &H, const float *Y, int ncols, long l
 
 constexpr int kScatNodes = 256;     // covered nodes (threads) per CTA of the FP32 scatter
 constexpr int kScatF32Cols = 8;     // columns per group
-constexpr int kScatF32Groups = 4;   // column groups per thread
+constexpr int kScatF32Groups = 4;   // column groups per thread, most
 
 // FP32 blocks: Cs holds alpha chi^T Y as one float4 per (atom, column), Cs4[J * ncols + c],
 // and g4[q] the four h^3 gamma chi values of entry q. A thread owns one covered node and
@@ -490,12 +493,22 @@ cudaError_t scatter_f32(const DevHam &H, const float *Cs, float *out, int ncols,
                         cudaStream_t st)
 {
     if (H.natoms == 0 || H.nuniq == 0 || ncols <= 0) return cudaSuccess;
-    constexpr int NC = kScatF32Cols, NG = kScatF32Groups;
     const long nb = (H.nuniq + kScatNodes - 1) / kScatNodes;
-    dim3 grid((unsigned)((ncols + NC * NG - 1) / (NC * NG)), (unsigned)(nb < 65535 ? nb : 65535));
-    k_scatter_f32<NC, NG><<<grid, kScatNodes, 0, st>>>(out, ld, ncols, H.nuniq, H.uniq_node, H.uniq_ptr,
-                                               H.nl_atom, reinterpret_cast<const float4 *>(H.nl_gf),
-                                               reinterpret_cast<const float4 *>(Cs));
+    auto launch = [&](auto ng) {
+        constexpr int NC = kScatF32Cols, NG = decltype(ng)::value;
+        const dim3 grid((unsigned)((ncols + NC * NG - 1) / (NC * NG)),
+                        (unsigned)(nb < 65535 ? nb : 65535));
+        k_scatter_f32<NC, NG><<<grid, kScatNodes, 0, st>>>(
+            out, ld, ncols, H.nuniq, H.uniq_node, H.uniq_ptr, H.nl_atom,
+            reinterpret_cast<const float4 *>(H.nl_gf), reinterpret_cast<const float4 *>(Cs));
+    };
+    // As in the pair scatter below, groups that follow one another in a thread pay only in
+    // launches of many waves: 75 x 61 x 53 x 40, 12 atoms 12.8 us with four, 9.1 us with one;
+    // 160^3 x 256, 400 atoms 1.20 ms with four, 1.35 ms with two.
+    if (nb * ((ncols + kScatF32Cols - 1) / kScatF32Cols) <= 4 * 4 * 152)
+        launch(std::integral_constant<int, 1>{});
+    else
+        launch(std::integral_constant<int, kScatF32Groups>{});
     note_launch();
     return cudaGetLastError();
 }

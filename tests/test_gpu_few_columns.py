@@ -39,6 +39,27 @@ def test_nonlocal_columns(ncols, pad):
     assert np.all(np.abs(got - ref).max(axis=1) <= 1e-12 * np.abs(ref).max(axis=1))
 
 
+@pytest.mark.parametrize("ncols", [1, 5, 33, 100])
+def test_nonlocal_columns_f32(ncols):
+    # a column's FP32 sums are the same bits in every launch shape
+    n3, h = (37, 29, 23), 0.45
+    nd = n3[0] * n3[1] * n3[2]
+    g = np.random.default_rng(3)
+    R = np.array([n * h for n in n3]) * g.uniform(0.1, 0.9, (14, 3))
+    gamma = g.uniform(-2, 2, (14, 4))
+    V = g.uniform(-3.0, 0.5, nd)
+    ctx = sparc.Context(n3, h, R, None, gamma, veff=V)
+    X = torch.from_numpy(g.uniform(-0.5, 0.5, (480, nd))).to("cuda:0", torch.float32)
+    Y, Z = torch.empty_like(X), torch.empty_like(X[:ncols])
+    ctx.apply_H(X, Y)
+    ctx.apply_H(X[:ncols].contiguous(), Z)
+    ctx.close()
+    assert torch.equal(Y[:ncols], Z)
+    H = oracle.Hamiltonian(n3, h, V, R, gamma)
+    ref = H.apply(X[:ncols].double().cpu().numpy())
+    assert np.abs(Z.double().cpu().numpy() - ref).max() <= 2e-6 * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("n3", [(1, 1, 1), (7, 5, 3), (33, 17, 5), (40, 41, 43)])
 @pytest.mark.parametrize("k", [1, 3, 10])
 def test_lanczos_sizes(n3, k):
