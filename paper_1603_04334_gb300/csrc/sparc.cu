@@ -575,7 +575,7 @@ bool lap_weights_int(int no, double h, int *wint, double &wunit)
 void free_ctx(sparc_ctx *c)
 {
     if (!c) return;
-    void *ps[] = {c->V, c->Vf, c->uq, c->atom_ptr, c->idx, c->ent_atom, c->chi, c->gchi, c->chi_f,
+    void *ps[] = {c->V, c->atom_ptr, c->idx, c->ent_atom, c->chi, c->gchi, c->chi_f,
                   c->gchi_f, c->chi_q, c->chi_F, c->proj_order, c->uniq_node, c->uniq_ptr, c->ent_list, c->nl_atom, c->nl_gf, c->nl_gdf, c->C, c->hx, c->rotx, c->roth, c->part,
                   c->tcws, c->dm, c->lz, c->bnd, c->bsc, c->flags, c->obs, c->pois};
     for (void *p : ps) dfree(p);
@@ -653,14 +653,10 @@ sparc_status build_tables(sparc_ctx *ctx, const sparc_atoms *at)
     // inverse map node -> entries
     const long nd = H.nd;
     const long nu_max = tot < nd ? tot : nd;
-    int *node_cnt = nullptr, *node_start = nullptr, *cursor = nullptr, *flags = nullptr,
-        *rank = nullptr, *scan_tmp = nullptr;
-    TRY(dmalloc(ctx, node_cnt, nd));
-    TRY(dmalloc(ctx, node_start, nd + 1));
-    TRY(dmalloc(ctx, cursor, nd));
-    TRY(dmalloc(ctx, flags, nd));
-    TRY(dmalloc(ctx, rank, nd + 1));
-    TRY(dmalloc(ctx, scan_tmp, nd / 4096 + 2));
+    int *scratch = nullptr;  // the map's, one allocation
+    TRY(dmalloc(ctx, scratch, 5 * (size_t)nd + 2 + nd / 4096 + 2));
+    int *node_cnt = scratch, *node_start = node_cnt + nd, *cursor = node_start + nd + 1,
+        *flags = cursor + nd, *rank = flags + nd, *scan_tmp = rank + nd + 1;
     TRY(dmalloc(ctx, ctx->ent_list, tot));
     TRY(dmalloc(ctx, ctx->uniq_node, nu_max));
     TRY(dmalloc(ctx, ctx->uniq_ptr, nu_max + 1));
@@ -670,9 +666,7 @@ sparc_status build_tables(sparc_ctx *ctx, const sparc_atoms *at)
     CK(cudaMemcpyAsync(&nuniq, rank + nd, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     H.nuniq = nuniq;
-    for (void *p : {(void *)R, (void *)G, (void *)counts, (void *)node_cnt, (void *)node_start,
-                    (void *)cursor, (void *)flags, (void *)rank, (void *)scan_tmp})
-        CK(cudaFree(p));
+    for (void *p : {(void *)R, (void *)G, (void *)counts, (void *)scratch}) CK(cudaFree(p));
     // chi on its integer grid (FP64 projection) and the node-ordered entry tables of the
     // scatter kernels
     TRY(dmalloc(ctx, ctx->chi_q, 2 * tot));
@@ -750,8 +744,12 @@ sparc_status sparc_create(const sparc_grid *grid, const double *veff_host,
         TRY(dmalloc(ctx, ctx->flags, 16));
         CK(cudaMemsetAsync(ctx->flags, 0, sizeof(int) * 16, ctx->st));
         H.err = ctx->flags + 14;
-        TRY(dmalloc(ctx, ctx->V, nd));
-        TRY(dmalloc(ctx, ctx->Vf, nd));
+        {   // V_eff in its three forms, one allocation (parts at multiples of 256 bytes)
+            const size_t nv = ((size_t)nd + 63) & ~(size_t)63;
+            TRY(dmalloc(ctx, ctx->V, 2 * nv + nv / 2));
+            ctx->uq = reinterpret_cast<int2 *>(ctx->V + nv);
+            ctx->Vf = reinterpret_cast<float *>(ctx->V + 2 * nv);
+        }
         if (veff_host) {
             CK(cudaMemcpyAsync(ctx->V, veff_host, sizeof(double) * nd, cudaMemcpyHostToDevice,
                                ctx->st));
@@ -776,7 +774,6 @@ sparc_status sparc_create(const sparc_grid *grid, const double *veff_host,
         H.Vf = ctx->Vf;
         // the range words (flags 0, 1) are read at the end of the set-up
         H.vscale = -2.0 / H.wunit;
-        TRY(dmalloc(ctx, ctx->uq, nd));
         CK(potential_grid(ctx->V, H.vscale, ctx->uq, nd, ctx->flags, ctx->st));
         CK(cudaMemcpyAsync(ctx->pin_i, ctx->flags, sizeof(int) * 2, cudaMemcpyDeviceToHost,
                            ctx->st));
