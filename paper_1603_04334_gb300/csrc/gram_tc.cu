@@ -428,7 +428,10 @@ k_tc_digits_t(const T *__restrict__ Y, long ld, long nd, int ns, long nstep,
 // for kN of its 128 B columns. part: nsplit x ntiles x 128 x 128 doubles, element (r, c) of
 // a tile at r * 128 + c (r: A column, c: B column).
 // Work units: a unit is one tile half (kN of the tile's 128 B columns) over a range of
-// chunks. Gram mode: CTA b owns unit b (units = halves x tiles x splits). ROT (the rotation,
+// chunks. Gram mode: CTA b owns unit b (units = halves x tiles x splits); the tiles from ntiles1
+// on are those of a second Gram with the same A (M_s and H_s of a Rayleigh-Ritz step in one
+// launch: half as many splits to add up, and one launch and reduction less, a tenth of the step
+// at 24^3 x 12). ROT (the rotation,
 // see rotate_tc below): tile t is (t / mblk, t % mblk) over all chunks (mblk = B blocks, so
 // the units that share an A block run side by side and find it in L2), the CTAs are
 // persistent and walk units b, b + gridDim.x, ... with the ring, the MMAs and the epilogue
@@ -441,7 +444,8 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
           const __grid_constant__ CUtensorMap mapB, const int *__restrict__ EB, int ns_pad, long nstep,
           const int2 *__restrict__ tiles, int ntiles, int nsplit, double *__restrict__ part,
           int drop, int *err, const int *__restrict__ EXA, const int *__restrict__ EXB,
-          int eb_ld = 0, int mblk = 1, TO *__restrict__ out = nullptr, long ldo = 0,
+          const __grid_constant__ CUtensorMap mapB2, const int *__restrict__ EB2,
+          const int *__restrict__ EXB2, int ntiles1, int eb_ld = 0, int mblk = 1, TO *__restrict__ out = nullptr, long ldo = 0,
           long nrow = 0, int ncol = 0, long ea_ld = 0)
 {
     using Dm = TcDims<C>;
@@ -463,6 +467,7 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
     const int ustride = ROT ? (int)gridDim.x : nunits;
     struct Unit {
         int hf, tile, split;
+        bool second;  // of the two Grams A^T B, A^T B2
         int2 tb;
         long c0, c1;
     };
@@ -471,7 +476,9 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
         w.hf = u % Dm::kHalves;
         w.tile = (u / Dm::kHalves) % ntiles;
         w.split = u / (Dm::kHalves * ntiles);
-        w.tb = ROT ? make_int2(w.tile / mblk, w.tile % mblk) : tiles[w.tile];
+        w.second = !ROT && w.tile >= ntiles1;
+        w.tb = ROT ? make_int2(w.tile / mblk, w.tile % mblk)
+                   : tiles[w.second ? w.tile - ntiles1 : w.tile];
         w.c0 = ROT ? 0 : (long)w.split * nchunk / nsplit;
         w.c1 = ROT ? nchunk : (long)(w.split + 1) * nchunk / nsplit;
         return w;
@@ -528,7 +535,7 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
                     unsigned char *dst = smem + (size_t)s * kStageBytes;
                     mbar_arrive_expect_tx(&full[s], kStageBytes);
                     bulk_load(dst, src, kOperandBytes, &full[s]);
-                    tma_load_3d(dst + kOperandBytes, &mapB, &full[s], w.hf * (C::kN * 2), row, 0);
+                    tma_load_3d(dst + kOperandBytes, w.second ? &mapB2 : &mapB, &full[s], w.hf * (C::kN * 2), row, 0);
                 }
                 __syncwarp();
                 src += C::kDigits * Dm::kBlobElems;
@@ -632,12 +639,8 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
         for (int u = blockIdx.x; u < nunits && ok; u += ustride) {
             const Unit w = unit(u);
             const long colA = (long)w.tb.x * kTile + r;
-            const int *ebw = EB + (long)w.tb.y * kTile + w.hf * C::kN + hw * kEpiCols + lane;
-#pragma unroll
-            for (int x = 0; x < kEpiCols; ++x) {
-                H[x] = 0.0f;
-                Lw[x * 32] = 0.0f;
-            }
+            const int *ebw = (w.second ? EB2 : EB) + (long)w.tb.y * kTile + w.hf * C::kN +
+                             hw * kEpiCols + lane;
             int ea_n = EA[w.c0 * ea_stride + colA], eb_n[kEB];
 #pragma unroll
             for (int k = 0; k < kEB; ++k) eb_n[k] = ebw[w.c0 * eb_stride + 32 * k];
@@ -685,10 +688,15 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
                                              fmaf(c1, 0x1p-8f, c0 - h));
                         const float f =
                             fA * __shfl_sync(0xffffffffu, fb[(g * 4 + x) / 32], (g * 4 + x) % 32);
-                        float sh, se;
-                        two_sum_f(H[g * 4 + x], h * f, sh, se);
-                        H[g * 4 + x] = sh;
-                        Lw[(g * 4 + x) * 32] += fmaf(l, f, se);
+                        if (c == w.c0) {  // the unit's first chunk: the sums are its own
+                            H[g * 4 + x] = h * f;
+                            Lw[(g * 4 + x) * 32] = l * f;
+                        } else {
+                            float sh, se;
+                            two_sum_f(H[g * 4 + x], h * f, sh, se);
+                            H[g * 4 + x] = sh;
+                            Lw[(g * 4 + x) * 32] += fmaf(l, f, se);
+                        }
                     }
                 }
             }
@@ -724,7 +732,7 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
             const Unit w = unit(u);
             const long colA = (long)w.tb.x * kTile + r;
             const long colB = (long)w.tb.y * kTile + w.hf * C::kN + hw * kEpiCols + lane % kEpiCols;
-            const int *ebw = EB + colB;
+            const int *ebw = (w.second ? EB2 : EB) + colB;
 #pragma unroll
             for (int x = 0; x < kEpiCols; ++x) S[x] = 0;
             // largest exponents over the chunks (the rotation's few chunks are looked at here)
@@ -738,7 +746,7 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
                 }
             } else {
                 xa = max(xa, EXA[colA]);
-                xb = max(xb, EXB[colB]);
+                xb = max(xb, (w.second ? EXB2 : EXB)[colB]);
             }
             int ea_n = EA[w.c0 * ea_stride + colA], eb_n = ebw[w.c0 * eb_stride];
             for (long c = w.c0; c < w.c1; ++c, ++cc) {
@@ -821,23 +829,36 @@ k_gram_tc(const __nv_bfloat16 *__restrict__ DA, const int *__restrict__ EA,
     }
 }
 
-// G from the split partials, summed in split order; sym mirrors each off-diagonal tile.
+// G (tiles below ntiles1) and G2 from the split partials, summed in split order, eight loads in
+// flight; sym mirrors each off-diagonal tile.
 __global__ void k_gram_tc_reduce(const double *__restrict__ part, const int2 *__restrict__ tiles,
-                                 int ntiles, int nsplit, int ns, bool sym, double *G)
+                                 int ntiles, int ntiles1, int nsplit, int ns, bool sym, double *G,
+                                 double *G2)
 {
+    constexpr int kU = 8;
     const long tot = (long)ntiles * kTile * kTile;
     for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < tot;
          t += (long)gridDim.x * blockDim.x) {
         const int tile = (int)(t / (kTile * kTile));
         const int e = (int)(t % (kTile * kTile));
         const int r = e / kTile, c = e % kTile;
-        const int2 tb = tiles[tile];
+        const int2 tb = tiles[tile < ntiles1 ? tile : tile - ntiles1];
         const int i = tb.x * kTile + r, j = tb.y * kTile + c;
         if (i >= ns || j >= ns) continue;
+        const double *p = part + (long)tile * kTile * kTile + e;
+        const long step = (long)ntiles * kTile * kTile;
         double v = 0.0;
-        for (int s = 0; s < nsplit; ++s) v += part[((long)s * ntiles + tile) * kTile * kTile + e];
-        G[i + (long)j * ns] = v;
-        if (sym && tb.x != tb.y) G[j + (long)i * ns] = v;
+        for (int s0 = 0; s0 < nsplit; s0 += kU) {
+            double x[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) x[u] = s0 + u < nsplit ? p[(s0 + u) * step] : 0.0;
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (s0 + u < nsplit) v += x[u];
+        }
+        double *g = tile < ntiles1 ? G : G2;
+        g[i + (long)j * ns] = v;
+        if (sym && tb.x != tb.y) g[j + (long)i * ns] = v;
     }
 }
 
@@ -845,7 +866,7 @@ __global__ void k_gram_tc_reduce(const double *__restrict__ part, const int2 *__
 
 namespace {
 struct TcPlan {
-    int ns_pad, nblk, ntiles, nsplit;
+    int ns_pad, nblk, ntiles1, ntiles, nsplit;  // tiles of one Gram, of all
     int drop;  // right shift of a chunk's integer: the chunks of a unit add up below 2^63
     long nstep, nchunk;
     size_t digits_bytes, exps_bytes, part_bytes, tiles_bytes;
@@ -859,14 +880,15 @@ int log2_ceil(long n)
 }
 
 template <class C>
-TcPlan tc_plan(long nd, int ns, bool sym)
+TcPlan tc_plan(long nd, int ns, bool sym, int grams = 1)
 {
     TcPlan p;
     p.nblk = (ns + kTile - 1) / kTile;
     p.ns_pad = p.nblk * kTile;
     p.nchunk = (nd + C::kChunk - 1) / C::kChunk;
     p.nstep = p.nchunk * TcDims<C>::kStepsPerChunk;
-    p.ntiles = sym ? p.nblk * (p.nblk + 1) / 2 : p.nblk * p.nblk;
+    p.ntiles1 = sym ? p.nblk * (p.nblk + 1) / 2 : p.nblk * p.nblk;
+    p.ntiles = grams * p.ntiles1;
     // K splits: one CTA per SM (the ring and the class accumulators fill an SM), so the
     // kernel takes (waves of 152 CTAs) x (chunks per split). Pick the split count with the
     // fewest chunk-times, counting about two chunks of fixed cost per CTA (set-up and the
@@ -886,16 +908,16 @@ TcPlan tc_plan(long nd, int ns, bool sym)
     p.digits_bytes = (size_t)C::kDigits * p.ns_pad * p.nstep * C::kStep * 2;
     p.exps_bytes = (size_t)(p.nchunk + 1) * p.ns_pad * sizeof(int);  // then the largest per column
     p.part_bytes = (size_t)p.nsplit * p.ntiles * kTile * kTile * sizeof(double);
-    p.tiles_bytes = (size_t)p.ntiles * sizeof(int2);
+    p.tiles_bytes = (size_t)p.ntiles1 * sizeof(int2);
     return p;
 }
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 template <class C>
-size_t tc_workspace(long nd, int ns, bool same_operand, bool sym)
+size_t tc_workspace(long nd, int ns, bool same_operand, bool sym, int grams = 1)
 {
-    const TcPlan p = tc_plan<C>(nd, ns, sym);
+    const TcPlan p = tc_plan<C>(nd, ns, sym, grams);
     const int nops = same_operand ? 1 : 2;
     return nops * (align256(p.digits_bytes) + align256(p.exps_bytes)) + align256(p.part_bytes) +
            align256(p.tiles_bytes);
@@ -906,7 +928,7 @@ size_t gram_tc_workspace(long nd, int ns, bool same_operand, bool sym)
 {
     return tc_workspace<Tc23>(nd, ns, same_operand, sym);
 }
-size_t gram_tc47_workspace(long nd, int ns) { return tc_workspace<Tc47>(nd, ns, false, true); }
+size_t gram_tc47_workspace(long nd, int ns) { return tc_workspace<Tc47>(nd, ns, false, true, 2); }
 
 // 16-byte loads along a column
 template <typename T>
@@ -966,29 +988,34 @@ static cudaError_t tc_prepare(const TcPlan &p, bool sym, int2 *tiles, cudaStream
         attr_set.store(true, std::memory_order_release);
     }
     static thread_local int2 host_tiles[64 * 65 / 2 + 64 * 64];
-    if (p.ntiles > (int)(sizeof(host_tiles) / sizeof(int2))) return cudaErrorInvalidValue;
+    if (p.ntiles1 > (int)(sizeof(host_tiles) / sizeof(int2))) return cudaErrorInvalidValue;
     int n = 0;
     for (int a = 0; a < p.nblk; ++a)
         for (int b = (sym ? a : 0); b < p.nblk; ++b) host_tiles[n++] = make_int2(a, b);
     return cudaMemcpyAsync(tiles, host_tiles, p.tiles_bytes, cudaMemcpyHostToDevice, st);
 }
 
+// G = A^T B and, for a plan of two Grams, G2 = A^T B2
 template <class C>
 static cudaError_t tc_run(const TcPlan &p, const __nv_bfloat16 *DA, const int *EA,
-                          const __nv_bfloat16 *DB, const int *EB, const int2 *tiles,
-                          double *part, int ns, bool sym, double *G, int *err, cudaStream_t st)
+                          const __nv_bfloat16 *DB, const int *EB, const __nv_bfloat16 *DB2,
+                          const int *EB2, const int2 *tiles, double *part, int ns, bool sym,
+                          double *G, double *G2, int *err, cudaStream_t st)
 {
     const int ctas = p.ntiles * p.nsplit * TcDims<C>::kHalves;
-    CUtensorMap mapB;
+    const long ex = p.nchunk * p.ns_pad;
+    CUtensorMap mapB, mapB2;
     cudaError_t e = tc_map<C>(mapB, DB, p.nblk, p.nstep);
+    if (e == cudaSuccess) e = tc_map<C>(mapB2, DB2, p.nblk, p.nstep);
     if (e != cudaSuccess) return e;
     k_gram_tc<C, false><<<ctas, kThreads, TcDims<C>::kSmemBytes, st>>>(
-        DA, EA, mapB, EB, p.ns_pad, p.nstep, tiles, p.ntiles, p.nsplit, part, p.drop, err,
-        EA + p.nchunk * p.ns_pad, EB + p.nchunk * p.ns_pad);
+        DA, EA, mapB, EB, p.ns_pad, p.nstep, tiles, p.ntiles, p.nsplit, part, p.drop, err, EA + ex,
+        EB + ex, mapB2, EB2, EB2 + ex, p.ntiles1);
     note_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_gram_tc_reduce<<<152 * 4, 256, 0, st>>>(part, tiles, p.ntiles, p.nsplit, ns, sym, G);
+    k_gram_tc_reduce<<<152 * 4, 256, 0, st>>>(part, tiles, p.ntiles, p.ntiles1, p.nsplit, ns, sym,
+                                              G, G2);
     note_launch();
     return cudaGetLastError();
 }
@@ -1023,7 +1050,7 @@ static cudaError_t gram_tc_impl(const TA *A, long lda, const TB *B, long ldb, lo
     if ((e = tc_prepare<C>(p, sym, tiles, st)) != cudaSuccess) return e;
     if ((e = tc_digits<C, TA>(A, lda, nd, ns, p, DA, EA, st)) != cudaSuccess) return e;
     if (!same && (e = tc_digits<C, TB>(B, ldb, nd, ns, p, DB, EB, st)) != cudaSuccess) return e;
-    return tc_run<C>(p, DA, EA, DB, EB, tiles, part, ns, sym, G, err, st);
+    return tc_run<C>(p, DA, EA, DB, EB, DB, EB, tiles, part, ns, sym, G, nullptr, err, st);
 }
 
 template <class C, typename TA, typename TB>
@@ -1032,8 +1059,8 @@ static cudaError_t gram_tc_pair_impl(const TA *A, long lda, const TB *B, long ld
                                      int *err, cudaStream_t st)
 {
     if (ns <= 0 || nd <= 0) return cudaErrorInvalidValue;
-    const TcPlan p = tc_plan<C>(nd, ns, true);
-    if (ws_bytes < tc_workspace<C>(nd, ns, false, true)) return cudaErrorInvalidValue;
+    const TcPlan p = tc_plan<C>(nd, ns, true, 2);
+    if (ws_bytes < tc_workspace<C>(nd, ns, false, true, 2)) return cudaErrorInvalidValue;
     unsigned char *w = (unsigned char *)ws;
     auto take = [&](size_t b) {
         unsigned char *r = w;
@@ -1050,9 +1077,7 @@ static cudaError_t gram_tc_pair_impl(const TA *A, long lda, const TB *B, long ld
     if ((e = tc_prepare<C>(p, true, tiles, st)) != cudaSuccess) return e;
     if ((e = tc_digits<C, TA>(A, lda, nd, ns, p, DA, EA, st)) != cudaSuccess) return e;
     if ((e = tc_digits<C, TB>(B, ldb, nd, ns, p, DB, EB, st)) != cudaSuccess) return e;
-    if ((e = tc_run<C>(p, DA, EA, DA, EA, tiles, part, ns, true, M, err, st)) != cudaSuccess)
-        return e;
-    return tc_run<C>(p, DA, EA, DB, EB, tiles, part, ns, true, Hm, err, st);
+    return tc_run<C>(p, DA, EA, DA, EA, DB, EB, tiles, part, ns, true, M, Hm, err, st);
 }
 
 template <typename TA, typename TB>
@@ -1169,7 +1194,8 @@ cudaError_t rotate_tc_impl(const TY *Y, long ldy, long nd, int ns, const double 
     // the fastest tile index)
     k_gram_tc<C, true, TO><<<grid, kThreads, TcDims<C>::kSmemBytes, st>>>(
         DB, EB, mapB, EA, p.ns_pad, p.nstep, nullptr, (int)(p.mblk * p.nblk), 1, nullptr,
-        std::max(1, log2_ceil(p.nchunk)), err, nullptr, nullptr, p.ns_pad, p.mblk, out, ldo, nd, ns, p.nd_pad);
+        std::max(1, log2_ceil(p.nchunk)), err, nullptr, nullptr,
+        mapB, EA, nullptr, 0, p.ns_pad, p.mblk, out, ldo, nd, ns, p.nd_pad);
     note_launch();
     return cudaGetLastError();
 }
