@@ -320,7 +320,7 @@ k_project_fx(const T *__restrict__ Y, long ld, int ncols, const int *__restrict_
             double v = alpha * ldexp(fma(g, 0x1p-23, h), E[cb] + chi_F[4 * J + l] - 49 + sh);
             if (((u >> 20) & 0x7ffu) == 0x7ffu) v = __longlong_as_double(0x7ff8000000000000ll);
             const float vh = (float)v;
-            C[(long)(J * 4 + l) * ncols + c0 + cb] = make_float2(vh, (float)(v - (double)vh));
+            C[((long)J * ncols + c0 + cb) * 4 + l] = make_float2(vh, (float)(v - (double)vh));
         }
     }
 }
@@ -525,13 +525,15 @@ namespace {
 constexpr int kScatDfNodes = 256;
 constexpr int kScatDfCols = 4;    // columns per group
 constexpr int kScatDfGroups = 4;  // column groups per thread, most
+__device__ __forceinline__ float2 lo_pair(const float4 &v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi_pair(const float4 &v) { return make_float2(v.z, v.w); }
 }  // namespace
 
 template <int NG>
 __global__ void __launch_bounds__(kScatDfNodes, 4)
 k_scatter_df(double *out, long ld, int ncols, long nuniq, const int *__restrict__ uniq_node,
              const int *__restrict__ uniq_ptr, const int *__restrict__ nl_atom,
-             const float2 *__restrict__ g, const float2 *__restrict__ Cs, unsigned *bOut)
+             const float4 *__restrict__ g4, const float4 *__restrict__ Cs4, unsigned *bOut)
 {
     constexpr int K = kScatDfCols;
     const int c0 = blockIdx.x * K * NG;
@@ -562,14 +564,17 @@ k_scatter_df(double *out, long ld, int ncols, long nuniq, const int *__restrict_
 #pragma unroll
             for (int k = 0; k < K; ++k) vh[k] = vl[k] = 0.0f;
             for (int q = q0; q < q1; ++q) {
-                const float2 *cs = Cs + (long)nl_atom[q] * 4 * ncols + cg;
+                const float4 *cs = Cs4 + ((long)nl_atom[q] * ncols + cg) * 2;
+                const float4 ga = g4[2L * q], gb = g4[2L * q + 1];
 #pragma unroll
-                for (int l = 0; l < 4; ++l) {
-                    const float2 gl = g[4L * q + l];
-#pragma unroll
-                    for (int k = 0; k < K; ++k)
-                        if (cg + k < ncols) mac(gl, cs[(long)l * ncols + k], vh[k], vl[k]);
-                }
+                for (int k = 0; k < K; ++k)
+                    if (cg + k < ncols) {
+                        const float4 a = cs[2 * k], b = cs[2 * k + 1];
+                        mac(lo_pair(ga), lo_pair(a), vh[k], vl[k]);
+                        mac(hi_pair(ga), hi_pair(a), vh[k], vl[k]);
+                        mac(lo_pair(gb), lo_pair(b), vh[k], vl[k]);
+                        mac(hi_pair(gb), hi_pair(b), vh[k], vl[k]);
+                    }
             }
             unsigned om[K];
 #pragma unroll
@@ -603,7 +608,9 @@ cudaError_t scatter_f64_df(const DevHam &H, const float2 *Cs, double *out, int n
         constexpr int NG = decltype(ng)::value, cpb = kScatDfCols * NG;
         dim3 grid((unsigned)((ncols + cpb - 1) / cpb), (unsigned)(nb < 65535 ? nb : 65535));
         k_scatter_df<NG><<<grid, kScatDfNodes, 0, st>>>(out, ld, ncols, H.nuniq, H.uniq_node,
-                                                        H.uniq_ptr, H.nl_atom, H.nl_gdf, Cs, bOut);
+                                                        H.uniq_ptr, H.nl_atom,
+                                                        reinterpret_cast<const float4 *>(H.nl_gdf),
+                                                        reinterpret_cast<const float4 *>(Cs), bOut);
     };
     // A thread's groups follow one another, so while a launch of one group a thread is a few
     // waves of the chip (four CTAs an SM), it is the shorter: 24^3 x 12, 4 atoms 13.5 -> 7.6 us;
