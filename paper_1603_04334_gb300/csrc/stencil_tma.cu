@@ -114,6 +114,76 @@ __device__ __forceinline__ void plane_math(const float *row, const float4 (&q)[2
     }
 }
 
+// The x sums of radius r of a row's four nodes from the 20 values around them.
+template <int r>
+__device__ __forceinline__ void x_sums(const float (&f)[20], float2 &xA, float2 &xB)
+{
+    if constexpr (r % 2 == 0) {
+        xA = __fadd2_rn(make_float2(f[8 + r], f[9 + r]), make_float2(f[8 - r], f[9 - r]));
+        xB = __fadd2_rn(make_float2(f[10 + r], f[11 + r]), make_float2(f[10 - r], f[11 - r]));
+    } else {
+        xA = make_float2(f[8 + r] + f[8 - r], f[9 + r] + f[9 - r]);
+        xB = make_float2(f[10 + r] + f[10 - r], f[11 + r] + f[11 - r]);
+    }
+}
+
+// plane_math for two rows at once (row: the upper one's; q, vv and a: of the rows in turn): the
+// y neighbours of the pair are 12 loads instead of 24, and each is used by both rows. The values
+// are those of plane_math, operation by operation.
+template <int PH>
+__device__ __forceinline__ void plane_math2(const float *row, const float4 (&q)[2][2 * kR + 1],
+                                            const float4 (&vv)[2], const StepCoef2 &cf,
+                                            float2 (&a)[2][2])
+{
+    constexpr int Q = 2 * kR + 1;
+    float f[2][20];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+            const float4 v = *reinterpret_cast<const float4 *>(row + h * kW + 4 * m);
+            f[h][4 * m] = v.x;
+            f[h][4 * m + 1] = v.y;
+            f[h][4 * m + 2] = v.z;
+            f[h][4 * m + 3] = v.w;
+        }
+    const float4 c0 = q[0][(PH + kR) % Q], c1 = q[1][(PH + kR) % Q];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float4 c = h ? c1 : c0;
+        a[h][0] = __fmul2_rn(__ffma2_rn(cf.alpha, lo2(vv[h]), cf.c0), lo2(c));
+        a[h][1] = __fmul2_rn(__ffma2_rn(cf.alpha, hi2(vv[h]), cf.c0), hi2(c));
+    }
+    float4 up = c0, dn = c1;  // the rows at distance r - 1 above row 0 and below row 1
+    auto radius = [&](auto rr) {
+        constexpr int r = decltype(rr)::value;
+        const float4 un = *reinterpret_cast<const float4 *>(row - r * kW + 8);
+        const float4 dm = *reinterpret_cast<const float4 *>(row + (1 + r) * kW + 8);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 yp = h ? dm : dn, ym = h ? up : un;
+            const float4 zp = q[h][(PH + kR + r) % Q], zm = q[h][(PH + kR - r) % Q];
+            float2 xA, xB;
+            x_sums<r>(f[h], xA, xB);
+            const float2 tA = __fadd2_rn(__fadd2_rn(xA, __fadd2_rn(lo2(yp), lo2(ym))),
+                                         __fadd2_rn(lo2(zp), lo2(zm)));
+            const float2 tB = __fadd2_rn(__fadd2_rn(xB, __fadd2_rn(hi2(yp), hi2(ym))),
+                                         __fadd2_rn(hi2(zp), hi2(zm)));
+            a[h][0] = __ffma2_rn(cf.w[r], tA, a[h][0]);
+            a[h][1] = __ffma2_rn(cf.w[r], tB, a[h][1]);
+        }
+        up = un;
+        dn = dm;
+    };
+    radius(std::integral_constant<int, 1>{});
+    radius(std::integral_constant<int, 2>{});
+    radius(std::integral_constant<int, 3>{});
+    radius(std::integral_constant<int, 4>{});
+    radius(std::integral_constant<int, 5>{});
+    radius(std::integral_constant<int, 6>{});
+    static_assert(kR == 6, "the radii above");
+}
+
 // State of one thread of k_stencil_f32_tma.
 struct TmaThread {
     float *sm;
@@ -129,8 +199,10 @@ struct TmaThread {
     int sp;         // slot of its Y_{j-1} tile
     unsigned pn;    // parity of plane tc + 6's current use of its stage
     int tc;         // current compute plane
-    int ty, tx, tid;
-    bool act, hasP;
+    int row;        // offset of the thread's upper row and first node in a plane's box, less 8
+    int tile;       // the same in a Y_{j-1} tile
+    int n0, tid;
+    bool act[2], hasP;
 };
 
 // plane t of Y (z = k0 - 6 + t) into stage t % kStages, with the Y_{j-1} tile of the plane
@@ -147,30 +219,45 @@ __device__ __forceinline__ void tma_issue(TmaThread &s, int t)
                     s.i0, s.j0, s.k0 - 2 * kR + t, s.col);
 }
 
-template <int PH>
-__device__ __forceinline__ bool plane_step(TmaThread &s, float4 (&q)[2 * kR + 1], float4 &vv,
-                                           float4 &v1, const StepCoef2 &cf, int *timed_out)
+template <int PH, int NR>
+__device__ __forceinline__ bool plane_step(TmaThread &s, float4 (&q)[NR][2 * kR + 1],
+                                           float4 (&vv)[NR], float4 (&v1)[NR], const StepCoef2 &cf,
+                                           int *timed_out)
 {
     constexpr int Q = 2 * kR + 1;
-    float4 v2 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (s.act && s.k + 2 < s.k1) v2 = *reinterpret_cast<const float4 *>(s.V + s.p + 2 * s.plane);
-    const bool got = mbar_wait(&s.full[s.sn], s.pn, kWaitLimit);
-    const float *stn = s.sm + (long)s.sn * kStageFloats;
-    q[(PH + 2 * kR) % Q] = *reinterpret_cast<const float4 *>(stn + (kR + s.ty) * kW + 8 + 4 * s.tx);
-    const float *row = s.sm + (long)s.sc * kStageFloats + (kR + s.ty) * kW + 4 * s.tx;
-    float2 aA, aB;
-    plane_math<PH>(row, q, vv, cf, aA, aB);
-    if (s.act && got) {
-        if (s.hasP) {
-            const float4 pv = *reinterpret_cast<const float4 *>(
-                s.sm + kStages * kStageFloats + s.sp * kTileFloats + s.ty * kBX + 4 * s.tx);
-            aA = __ffma2_rn(cf.nbeta, lo2(pv), aA);
-            aB = __ffma2_rn(cf.nbeta, hi2(pv), aB);
-        }
-        *reinterpret_cast<float4 *>(s.Oc + s.p) = make_float4(aA.x, aA.y, aB.x, aB.y);
+    float4 v2[NR];
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+        v2[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s.act[h] && s.k + 2 < s.k1)
+            v2[h] = *reinterpret_cast<const float4 *>(s.V + s.p + h * s.n0 + 2 * s.plane);
     }
-    vv = v1;
-    v1 = v2;
+    const bool got = mbar_wait(&s.full[s.sn], s.pn, kWaitLimit);
+    const float *stn = s.sm + (long)s.sn * kStageFloats + s.row + 8;
+#pragma unroll
+    for (int h = 0; h < NR; ++h)
+        q[h][(PH + 2 * kR) % Q] = *reinterpret_cast<const float4 *>(stn + h * kW);
+    float2 a[NR][2];
+    const float *row = s.sm + (long)s.sc * kStageFloats + s.row;
+    if constexpr (NR == 2)
+        plane_math2<PH>(row, q, vv, cf, a);
+    else
+        plane_math<PH>(row, q[0], vv[0], cf, a[0][0], a[0][1]);
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+        if (s.act[h] && got) {
+            if (s.hasP) {
+                const float4 pv = *reinterpret_cast<const float4 *>(
+                    s.sm + kStages * kStageFloats + s.sp * kTileFloats + s.tile + h * kBX);
+                a[h][0] = __ffma2_rn(cf.nbeta, lo2(pv), a[h][0]);
+                a[h][1] = __ffma2_rn(cf.nbeta, hi2(pv), a[h][1]);
+            }
+            *reinterpret_cast<float4 *>(s.Oc + s.p + h * s.n0) =
+                make_float4(a[h][0].x, a[h][0].y, a[h][1].x, a[h][1].y);
+        }
+        vv[h] = v1[h];
+        v1[h] = v2[h];
+    }
     if (!got) *timed_out = 1;
     __syncthreads();  // every thread is done with plane tc's stage
     if (*(volatile int *)timed_out) return false;
@@ -187,11 +274,12 @@ __device__ __forceinline__ bool plane_step(TmaThread &s, float4 (&q)[2 * kR + 1]
     return true;
 }
 
-// Block: 8 x 16 threads (4 x-nodes each). Thread 0 keeps the ring kStages planes ahead:
+// Block: 8 x 16 / NR threads (4 x-nodes of NR neighbouring rows each). Thread 0 keeps the ring kStages planes ahead:
 // after the barrier that ends the compute of plane tc, it refills that plane's stage with
 // plane tc + kStages. The plane loop is unrolled 13 times, one copy per rotation of the z
 // queue, so the queue is never shifted.
-__global__ void __launch_bounds__(kTX *kTY, 4)
+template <int NR>
+__global__ void __launch_bounds__(kTX *kTY / NR, 4)
 k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmP,
                   bool hasP, float *out, const float *__restrict__ V, int n0, int n1, int n2,
                   long ld, int nzc, int zchunk, StepCoef2 cf, int *err)
@@ -202,8 +290,9 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
     __shared__ int timed_out;
     TmaThread s;
     s.tid = threadIdx.y * kTX + threadIdx.x;
-    s.tx = threadIdx.x;
-    s.ty = threadIdx.y;
+    s.row = (kR + NR * threadIdx.y) * kW + 4 * threadIdx.x;
+    s.tile = NR * threadIdx.y * kBX + 4 * threadIdx.x;
+    s.n0 = n0;
     s.i0 = blockIdx.x * kBX;
     s.j0 = blockIdx.y * kTY;
     s.col = blockIdx.z / nzc;
@@ -215,8 +304,9 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
     s.tmY = &tmY;
     s.tmP = &tmP;
     s.hasP = hasP;
-    const int i = s.i0 + 4 * s.tx, j = s.j0 + s.ty;
-    s.act = (i < n0) && (j < n1);
+    const int i = s.i0 + 4 * threadIdx.x, j = s.j0 + NR * threadIdx.y;
+#pragma unroll
+    for (int h = 0; h < NR; ++h) s.act[h] = (i < n0) && (j + h < n1);
     s.plane = (long)n0 * n1;
     s.k = s.k0;
     s.p = (long)i + (long)n0 * j + (long)s.k0 * s.plane;
@@ -232,17 +322,18 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
     __syncthreads();
     if (s.tid == 0)
         for (int t = 0; t < kStages && t < s.T; ++t) tma_issue(s, t);
-    auto center = [&](int t) -> float4 {
-        return *reinterpret_cast<const float4 *>(sm + (long)(t % kStages) * kStageFloats +
-                                                 (kR + s.ty) * kW + 8 + 4 * s.tx);
+    auto center = [&](int t, int h) -> float4 {
+        return *reinterpret_cast<const float4 *>(sm + (long)(t % kStages) * kStageFloats + s.row +
+                                                 h * kW + 8);
     };
     bool ok = true;
-    float4 q[2 * kR + 1];
+    float4 q[NR][2 * kR + 1];
     // planes 0..5 only feed the queue: read them, then hand their stages to planes
     // kStages .. kStages+5
     for (int t = 0; t < kR; ++t) {
         ok = ok && mbar_wait(&full[t % kStages], (unsigned)((t / kStages) & 1), kWaitLimit);
-        q[t] = center(t);
+#pragma unroll
+        for (int h = 0; h < NR; ++h) q[h][t] = center(t, h);
     }
     if (!ok) timed_out = 1;
     __syncthreads();
@@ -250,7 +341,8 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
         for (int t = kStages; t < kStages + kR && t < s.T; ++t) tma_issue(s, t);
     for (int t = kR; t < 2 * kR; ++t) {
         ok = ok && mbar_wait(&full[t % kStages], (unsigned)((t / kStages) & 1), kWaitLimit);
-        q[t] = center(t);
+#pragma unroll
+        for (int h = 0; h < NR; ++h) q[h][t] = center(t, h);
     }
     if (!ok) timed_out = 1;
     __syncthreads();
@@ -259,14 +351,19 @@ k_stencil_f32_tma(const __grid_constant__ CUtensorMap tmY, const __grid_constant
     s.pn = (unsigned)(((2 * kR) / kStages) & 1);
     s.sp = (2 * kR) % kPrev;
     s.tc = kR;
-    float4 vv = make_float4(0.f, 0.f, 0.f, 0.f), v1 = vv;
-    if (s.act) vv = *reinterpret_cast<const float4 *>(V + s.p);
-    if (s.act && s.k0 + 1 < s.k1) v1 = *reinterpret_cast<const float4 *>(V + s.p + s.plane);
+    float4 vv[NR], v1[NR];
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+        vv[h] = v1[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float *v = V + s.p + h * n0;
+        if (s.act[h]) vv[h] = *reinterpret_cast<const float4 *>(v);
+        if (s.act[h] && s.k0 + 1 < s.k1) v1[h] = *reinterpret_cast<const float4 *>(v + s.plane);
+    }
     const int tend = s.T - kR;
     if (!timed_out) {
 #define SPARC_PLANE(PH)                                                                  \
     if (s.tc >= tend) break;                                                             \
-    if (!plane_step<PH>(s, q, vv, v1, cf, &timed_out)) break;
+    if (!plane_step<PH, NR>(s, q, vv, v1, cf, &timed_out)) break;
         for (;;) {
             SPARC_PLANE(0) SPARC_PLANE(1) SPARC_PLANE(2) SPARC_PLANE(3) SPARC_PLANE(4)
             SPARC_PLANE(5) SPARC_PLANE(6) SPARC_PLANE(7) SPARC_PLANE(8) SPARC_PLANE(9)
@@ -735,9 +832,13 @@ cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev,
     static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
     const int smem = kSmemBytes;
     if (!attr_set.load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(k_stencil_f32_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem);
-        if (e != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(k_stencil_f32_tma<1>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
+                cudaSuccess ||
+            (e = cudaFuncSetAttribute(k_stencil_f32_tma<2>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
+                cudaSuccess)
+            return e;
         attr_set.store(true, std::memory_order_release);
     }
     // both maps view a block as (x, y, z, column); they differ in base and box
@@ -763,9 +864,21 @@ cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev,
     int nzc, zchunk;
     f32_z_split(H.n2, (long)gx * gy, ncols, nzc, zchunk);
     dim3 grid(gx, gy, ncols * nzc);
-    k_stencil_f32_tma<<<grid, dim3(kTX, kTY), smem, st>>>(mapY, mapP, Yprev != nullptr, out,
-                                                          H.Vf, H.n0, H.n1, H.n2, ld, nzc,
-                                                          zchunk, pair_coef(cf), err);
+    // Two rows per thread read 26 16-byte values from shared memory for eight nodes where one
+    // row reads 19 for four, which is what bounds a full chip; a launch of one wave is
+    // bound by its planes' latency, and the more threads are the faster: 96^3 x 128 380 -> 335 us,
+    // 128^3 x 64 444 -> 403, 160^3 x 256 3.22 -> 3.07 ms; 32^3 x 16 (256 CTAs) 9.3 us with one
+    // row, 9.8 with two, 48 x 40 x 36 x 60 (720 CTAs) 34 either way.
+    auto launch = [&](auto nr) {
+        constexpr int NR = decltype(nr)::value;
+        k_stencil_f32_tma<NR><<<grid, dim3(kTX, kTY / NR), smem, st>>>(
+            mapY, mapP, Yprev != nullptr, out, H.Vf, H.n0, H.n1, H.n2, ld, nzc, zchunk,
+            pair_coef(cf), err);
+    };
+    if ((long)gx * gy * ncols * nzc > 4 * 152)
+        launch(std::integral_constant<int, 2>{});
+    else
+        launch(std::integral_constant<int, 1>{});
     note_launch();
     return cudaGetLastError();
 }
