@@ -553,19 +553,91 @@ k_stencil_f32_copy(const float *Yb, const float *Pb, float *out, const float *__
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+namespace {
+// State of one thread of k_batch_stencil_tma within an item.
+struct BatchThread {
+    float *Oc;
+    const float *V;
+    long p, plane;  // p: the thread's node offset at the current plane
+    int k, k1;      // current z, end of the range
+    int sn;         // stage of the plane entering the queue (its Y_{j-1} slot is sn mod kPrev)
+    unsigned pn;    // parity of its current use
+    int row, tile;  // offsets of the thread's rows in a plane's box (less 8) and in a tile
+    int n0;
+    bool act[2], hasP;
+};
+static_assert(kStages % kPrev == 0, "a plane's Y_{j-1} slot follows from its stage");
+
+template <int PH, int NR>
+__device__ __forceinline__ bool batch_plane(BatchThread &s, float4 (&q)[NR][2 * kR + 1],
+                                            float4 (&vv)[NR], float4 (&v1)[NR], const StepCoef2 &cf,
+                                            float *sm, uint64_t *full, int *timed_out)
+{
+    constexpr int Q = 2 * kR + 1;
+    float4 v2[NR];
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+        v2[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s.act[h] && s.k + 2 < s.k1)
+            v2[h] = *reinterpret_cast<const float4 *>(s.V + s.p + h * s.n0 + 2 * s.plane);
+    }
+    const bool got = mbar_wait(&full[s.sn], s.pn, kWaitLimit);
+#pragma unroll
+    for (int h = 0; h < NR; ++h)
+        q[h][(PH + 2 * kR) % Q] = *reinterpret_cast<const float4 *>(
+            sm + s.sn * kStageFloats + s.row + h * kW + 8);
+    const int sc = s.sn >= kR ? s.sn - kR : s.sn + kStages - kR;
+    float2 a[NR][2];
+    const float *row = sm + sc * kStageFloats + s.row;
+    if constexpr (NR == 2)
+        plane_math2<PH>(row, q, vv, cf, a);
+    else
+        plane_math<PH>(row, q[0], vv[0], cf, a[0][0], a[0][1]);
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+        if (s.act[h] && got) {
+            if (s.hasP) {
+                const float4 pv = *reinterpret_cast<const float4 *>(
+                    sm + kStages * kStageFloats + s.sn % kPrev * kTileFloats + s.tile + h * kBX);
+                a[h][0] = __ffma2_rn(cf.nbeta, lo2(pv), a[h][0]);
+                a[h][1] = __ffma2_rn(cf.nbeta, hi2(pv), a[h][1]);
+            }
+            *reinterpret_cast<float4 *>(s.Oc + s.p + h * s.n0) =
+                make_float4(a[h][0].x, a[h][0].y, a[h][1].x, a[h][1].y);
+        }
+        vv[h] = v1[h];
+        v1[h] = v2[h];
+    }
+    if (!got) *timed_out = 1;
+    if (++s.sn == kStages) {
+        s.sn = 0;
+        s.pn ^= 1u;
+    }
+    ++s.k;
+    s.p += s.plane;
+    __syncthreads();  // the plane's stage is free
+    return !*(volatile int *)timed_out;
+}
+}  // namespace
+
 // Work-list form for a batch of clusters: a persistent CTA walks its items (cluster,
 // column, 32 x 16 tile, z range) in order, and its ring runs on across item boundaries: the
 // planes of all its items form one sequence (item i contributes (k1 - k0) + 12 planes),
 // thread 0 issues that sequence kStages planes ahead of the planes released, and the
 // consumers take the planes in the same order. Each cluster's tensor maps (Y_j with halo,
 // Y_{j-1} tile) live in device memory, its sizes, pointers and coefficients in its
-// BatchTma entry. Same per-point arithmetic as k_stencil_f32_tma.
-__global__ void __launch_bounds__(kTX *kTY, 4)
+// BatchTma entry (the current item's coefficients in shared memory). A plane is computed as in
+// k_stencil_f32_tma, two rows per thread where the launch is more than a wave (the scalar form
+// with a shifted queue it replaces: 445 us a step for 12 clusters of 32 to 48 nodes an edge, 400 us
+// so; one cluster 31.7 -> 27.7 us, 40 clusters 1.28 -> 1.12 ms).
+template <int NR>
+__global__ void __launch_bounds__(kTX *kTY / NR, NR == 1 ? 2 : 4)
 k_batch_stencil_tma(const BatchItem *__restrict__ items, int nitems, const BatchTma *cs, int *err)
 {
     extern __shared__ __align__(128) float sm[];
     __shared__ __align__(8) uint64_t full[kStages];
     __shared__ int timed_out;
+    __shared__ __align__(16) StepCoef2 cf;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int tid = ty * kTX + tx;
     if (tid == 0) {
@@ -619,88 +691,77 @@ k_batch_stencil_tma(const BatchItem *__restrict__ items, int nitems, const Batch
         const BatchTma &C = cs[w.cluster];
         const int n0 = C.n0, n1 = C.n1;
         const int T = (w.k1 - w.k0) + 2 * kR;
-        const int i0 = w.a * kBX, j0 = w.b * kTY;
-        const int i = i0 + 4 * tx, j = j0 + ty;
-        const bool act = (i < n0) && (j < n1);
-        const long plane = (long)n0 * n1;
-        const long pij = (long)i + (long)n0 * j;
-        float *Oc = C.out + (long)w.col * C.ld;
-        const float *V = C.V;
-        const StepCoef<float> cf = C.cf;
-        const bool hasP = C.mP != nullptr;
-        auto center = [&](unsigned g) -> float4 {
-            return *reinterpret_cast<const float4 *>(sm + (g % kStages) * kStageFloats +
-                                                     (kR + ty) * kW + 8 + 4 * tx);
+        const int i = w.a * kBX + 4 * tx, j = w.b * kTY + NR * ty;
+        if (tid <= kR) cf.w[tid] = make_float2(C.cf.w[tid], C.cf.w[tid]);
+        if (tid == 0) {
+            cf.c0 = make_float2(C.cf.c0, C.cf.c0);
+            cf.alpha = make_float2(C.cf.alpha, C.cf.alpha);
+            cf.nbeta = make_float2(-C.cf.beta, -C.cf.beta);
+        }
+        BatchThread b;
+        b.row = (kR + NR * ty) * kW + 4 * tx;
+        b.tile = NR * ty * kBX + 4 * tx;
+        auto center = [&](unsigned g, int h) -> float4 {
+            return *reinterpret_cast<const float4 *>(sm + (g % kStages) * kStageFloats + b.row +
+                                                     h * kW + 8);
         };
         bool ok = true;
-        float4 q[2 * kR + 1];
+        float4 q[NR][2 * kR + 1];
         for (int t = 0; t < kR; ++t) {
             ok = ok && wait(g0 + t);
-            q[t] = center(g0 + t);
+#pragma unroll
+            for (int h = 0; h < NR; ++h) q[h][t] = center(g0 + t, h);
         }
         if (!ok) timed_out = 1;
         __syncthreads();
         if (tid == 0 && !timed_out) issue_upto(g0 + kR + kStages);
         for (int t = kR; t < 2 * kR; ++t) {
             ok = ok && wait(g0 + t);
-            q[t] = center(g0 + t);
+#pragma unroll
+            for (int h = 0; h < NR; ++h) q[h][t] = center(g0 + t, h);
         }
         if (!ok) timed_out = 1;
         __syncthreads();
-        float4 vv = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (act) vv = *reinterpret_cast<const float4 *>(V + pij + (long)w.k0 * plane);
-        for (int tc = kR; tc < T - kR && !timed_out; ++tc) {
-            const int k = w.k0 - kR + tc;
-            const long p = pij + (long)k * plane;
-            float4 vn = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (act && k + 1 < w.k1) vn = *reinterpret_cast<const float4 *>(V + p + plane);
-            if (!wait(g0 + tc + kR)) timed_out = 1;
-            q[2 * kR] = center(g0 + tc + kR);
-            const float *pl = sm + ((g0 + tc) % kStages) * kStageFloats;
-            const float *row = pl + (kR + ty) * kW + 4 * tx;
-            float f[20];
+        b.n0 = n0;
+        b.Oc = C.out + (long)w.col * C.ld;
+        b.V = C.V;
+        b.plane = (long)n0 * n1;
+        b.p = (long)i + (long)n0 * j + (long)w.k0 * b.plane;
+        b.k = w.k0;
+        b.k1 = w.k1;
+        b.sn = (int)((g0 + 2 * kR) % kStages);
+        b.pn = (g0 + 2 * kR) / kStages & 1u;
+        b.hasP = C.mP != nullptr;
+        float4 vv[NR], v1[NR];
 #pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                const float4 v = *reinterpret_cast<const float4 *>(row + 4 * m);
-                f[4 * m] = v.x;
-                f[4 * m + 1] = v.y;
-                f[4 * m + 2] = v.z;
-                f[4 * m + 3] = v.w;
-            }
-            float acc[4];
-            const float *c4 = &q[kR].x;
-            const float *v4 = &vv.x;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = (cf.c0 + cf.alpha * v4[u]) * c4[u];
-#pragma unroll
-            for (int r = 1; r <= kR; ++r) {
-                const float4 yp = *reinterpret_cast<const float4 *>(row + r * kW + 8);
-                const float4 ym = *reinterpret_cast<const float4 *>(row - r * kW + 8);
-                const float *a = &yp.x, *b = &ym.x, *zp = &q[kR + r].x, *zm = &q[kR - r].x;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float t = (f[8 + u + r] + f[8 + u - r]) + (a[u] + b[u]) + (zp[u] + zm[u]);
-                    acc[u] += cf.w[r] * t;
-                }
-            }
-            if (act) {
-                float4 o = make_float4(acc[0], acc[1], acc[2], acc[3]);
-                if (hasP) {
-                    const float4 pv = *reinterpret_cast<const float4 *>(
-                        sm + kStages * kStageFloats + (g0 + tc + kR) % kPrev * kTileFloats +
-                        ty * kBX + 4 * tx);
-                    o.x -= cf.beta * pv.x;
-                    o.y -= cf.beta * pv.y;
-                    o.z -= cf.beta * pv.z;
-                    o.w -= cf.beta * pv.w;
-                }
-                *reinterpret_cast<float4 *>(Oc + p) = o;
-            }
-            vv = vn;
-#pragma unroll
-            for (int t = 0; t < 2 * kR; ++t) q[t] = q[t + 1];
-            __syncthreads();  // plane tc's stage is free
-            if (tid == 0 && !timed_out) issue_upto(g0 + tc + 1 + kStages);
+        for (int h = 0; h < NR; ++h) {
+            b.act[h] = (i < n0) && (j + h < n1);
+            vv[h] = v1[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float *v = b.V + b.p + h * n0;
+            if (b.act[h]) vv[h] = *reinterpret_cast<const float4 *>(v);
+            if (b.act[h] && b.k + 1 < b.k1)
+                v1[h] = *reinterpret_cast<const float4 *>(v + b.plane);
+        }
+        for (bool more = !timed_out && b.k < b.k1; more;) {
+            // (each plane that is done makes room for one)
+#define SPARC_BATCH_STEP(PH)                                                                   \
+    more = batch_plane<PH, NR>(b, q, vv, v1, cf, sm, full, &timed_out);                             \
+    if (tid == 0 && more) issue_upto(issued + 1);                                               \
+    if (!(more = more && b.k < b.k1)) break
+            SPARC_BATCH_STEP(0);
+            SPARC_BATCH_STEP(1);
+            SPARC_BATCH_STEP(2);
+            SPARC_BATCH_STEP(3);
+            SPARC_BATCH_STEP(4);
+            SPARC_BATCH_STEP(5);
+            SPARC_BATCH_STEP(6);
+            SPARC_BATCH_STEP(7);
+            SPARC_BATCH_STEP(8);
+            SPARC_BATCH_STEP(9);
+            SPARC_BATCH_STEP(10);
+            SPARC_BATCH_STEP(11);
+            SPARC_BATCH_STEP(12);
+#undef SPARC_BATCH_STEP
         }
         g0 += T;
         __syncthreads();  // the item's last planes (z halo) are free
@@ -757,12 +818,19 @@ cudaError_t batch_stencil_tma(const BatchItem *items, int nitems, const BatchTma
     static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
     const int smem = kSmemBytes;
     if (!attr_set.load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(k_batch_stencil_tma,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(
+            k_batch_stencil_tma<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_batch_stencil_tma<2>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         attr_set.store(true, std::memory_order_release);
     }
-    k_batch_stencil_tma<<<grid, dim3(kTX, kTY), smem, st>>>(items, nitems, cs, err);
+    // one row per thread while all items are resident at two CTAs per SM (as in stencil_f32_tma)
+    if (nitems <= 2 * 152)
+        k_batch_stencil_tma<1><<<grid, dim3(kTX, kTY), smem, st>>>(items, nitems, cs, err);
+    else
+        k_batch_stencil_tma<2><<<grid, dim3(kTX, kTY / 2), smem, st>>>(items, nitems, cs, err);
     note_launch();
     return cudaGetLastError();
 }
