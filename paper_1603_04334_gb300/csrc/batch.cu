@@ -30,7 +30,7 @@ constexpr int kDefaultVariant = kTmaItemForm * 3;  // TMA, one CTA per item, who
 // Persistent grids: enough resident CTAs to fill the 152 SMs several times.
 constexpr int kGridStencil = 152 * 8;
 constexpr int kGridTma = 152 * 4;
-constexpr int kGridProject = 152 * 2;
+constexpr int kGridProject = 152 * 4;
 constexpr int kGridScatter = 152 * 6;
 
 struct Key {
@@ -123,7 +123,7 @@ sparc_status build_items(sparc_batch *b, const int *ncols)
         if (H.natoms > 0) {
             b->any_atoms = true;
             for (int J = 0; J < H.natoms; ++J)
-                for (int col = 0; col < ncols[c]; col += kBatchCols)
+                for (int col = 0; col < ncols[c]; col += kBatchProjCols)
                     pr.push_back({(int)c, col, J, 0, 0, 0});
             const long chunks = (H.nuniq + kBatchNodes - 1) / kBatchNodes;
             for (long u = 0; u < chunks; ++u)

@@ -1,6 +1,5 @@
-// bounds.cu -- helpers of the FP64 path that run once per block or per context:
-// per-column magnitude bounds (the FP64 stencil's fixed-point grid), V_eff - shift as FP32
-// pairs, and FP64 arrays as FP32 pairs.
+// bounds.cu -- per-column magnitude bounds of a block (the FP64 stencil's and projection's
+// fixed-point grid).
 #include "fx.cuh"
 #include "internal.cuh"
 

@@ -162,7 +162,11 @@ StepCoef<float> coef_f32(const DevHam &H, double alpha, double shift, double bet
 const DevHam *ctx_ham(const sparc_ctx *ctx);
 cudaStream_t ctx_stream(const sparc_ctx *ctx);
 float *ctx_coef_buffer(sparc_ctx *ctx, int ncols);  // grows the context's C buffer
-constexpr int kBatchCols = 16;     // columns per nonlocal work item
+// columns per projection and scatter work item: few enough that the accumulators stay in registers
+// and the items of small clusters reach all SMs (12 clusters of 32 to 48 nodes an edge: projection
+// 105 us with 16 columns, which spilled, 64 with 8, 59 with 4 at four CTAs per SM; scatter 115 us
+// with 16, 103 with 8, 124 with 4)
+constexpr int kBatchProjCols = 4, kBatchCols = 8;
 constexpr int kBatchNodes = 256;   // covered nodes per scatter work item
 
 cudaError_t stencil_f32(const DevHam &H, const float *Y, const float *Yprev, float *out,

@@ -25,48 +25,42 @@ __device__ __forceinline__ T warp_sum(T v)
 
 // One CTA per (atom, column block of CB). Each thread accumulates 4*CB partial sums over
 // a strided share of the atom's support; the block reduces them in a fixed order.
-// C layout: ILV = false: C[(J * 4 + l) * ncols + c]; ILV = true: C[(J * ncols + c) * 4 + l]
-// (the four channels of one atom and column contiguous, one 16-byte load in the scatter).
+// C layout: C[(J * ncols + c) * 4 + l] (the four channels of one atom and column contiguous, one
+// 16-byte load in the scatter).
 // project_block: atom J (support entries b .. e-1), columns c0 .. c0+CB-1; ends with a CTA
 // barrier so the caller may reuse the shared memory.
-template <typename T, typename TC, int CB, int NT, bool ILV>
-__device__ __forceinline__ void project_block(const T *__restrict__ Y, long ld, int ncols, int J,
+template <int CB, int NT>
+__device__ __forceinline__ void project_block(const float *__restrict__ Y, long ld, int ncols, int J,
                                               int b, int e, int c0,
                                               const int *__restrict__ idx,
-                                              const TC *__restrict__ chi, TC *__restrict__ C,
-                                              TC alpha)
+                                              const float *__restrict__ chi, float *__restrict__ C,
+                                              float alpha)
 {
-    __shared__ TC red[NT / 32][4 * CB];
-    TC acc[4][CB];
+    __shared__ float red[NT / 32][4 * CB];
+    float acc[4][CB];
 #pragma unroll
     for (int l = 0; l < 4; ++l)
 #pragma unroll
-        for (int cb = 0; cb < CB; ++cb) acc[l][cb] = (TC)0;
+        for (int cb = 0; cb < CB; ++cb) acc[l][cb] = 0;
     // Two support points per trip, their node indices loaded one trip ahead, so a thread
     // has 2 * CB independent loads of Y in flight instead of an index -> value chain.
-    auto load_chi = [&](int s, TC x[4]) {
-        if constexpr (sizeof(TC) == 4) {
-            const float4 v = reinterpret_cast<const float4 *>(chi)[s];
-            x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
-        } else {
-            const double2 a = reinterpret_cast<const double2 *>(chi)[2 * (long)s];
-            const double2 q = reinterpret_cast<const double2 *>(chi)[2 * (long)s + 1];
-            x[0] = a.x, x[1] = a.y, x[2] = q.x, x[3] = q.y;
-        }
+    auto load_chi = [&](int s, float x[4]) {
+        const float4 v = reinterpret_cast<const float4 *>(chi)[s];
+        x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
     };
     int s = b + threadIdx.x;
     long pa = s < e ? idx[s] : 0, pb = s + NT < e ? idx[s + NT] : 0;
     for (; s < e; s += 2 * NT) {
         const bool vb = s + NT < e;
-        TC xa[4], xb[4] = {(TC)0, (TC)0, (TC)0, (TC)0};
-        TC ya[CB], yb[CB];
+        float xa[4], xb[4] = {0, 0, 0, 0};
+        float ya[CB], yb[CB];
         load_chi(s, xa);
         if (vb) load_chi(s + NT, xb);
 #pragma unroll
         for (int cb = 0; cb < CB; ++cb) {
             const bool vc = c0 + cb < ncols;
-            ya[cb] = vc ? (TC)Y[pa + (long)(c0 + cb) * ld] : (TC)0;
-            yb[cb] = (vc && vb) ? (TC)Y[pb + (long)(c0 + cb) * ld] : (TC)0;
+            ya[cb] = vc ? Y[pa + (long)(c0 + cb) * ld] : 0;
+            yb[cb] = (vc && vb) ? Y[pb + (long)(c0 + cb) * ld] : 0;
         }
         const int sn = s + 2 * NT;
         pa = sn < e ? idx[sn] : 0;
@@ -85,19 +79,17 @@ __device__ __forceinline__ void project_block(const T *__restrict__ Y, long ld, 
     for (int l = 0; l < 4; ++l)
 #pragma unroll
         for (int cb = 0; cb < CB; ++cb) {
-            const TC v = warp_sum(acc[l][cb]);
+            const float v = warp_sum(acc[l][cb]);
             if (lane == 0) red[wid][l * CB + cb] = v;
         }
     __syncthreads();
     if (threadIdx.x < 4 * CB) {
         const int l = threadIdx.x / CB, cb = threadIdx.x % CB;
-        TC v = (TC)0;
+        float v = 0;
 #pragma unroll
         for (int w = 0; w < NT / 32; ++w) v += red[w][threadIdx.x];
         if (c0 + cb < ncols) {
-            const long o = ILV ? ((long)J * ncols + c0 + cb) * 4 + l
-                               : (long)(J * 4 + l) * ncols + c0 + cb;
-            C[o] = alpha * v;
+            C[((long)J * ncols + c0 + cb) * 4 + l] = alpha * v;
         }
     }
     __syncthreads();
@@ -108,25 +100,25 @@ __device__ __forceinline__ void project_block(const T *__restrict__ Y, long ld, 
 // DRAM about once), y = column block. order (optional): the atoms in a spatial order, so
 // that CTAs dispatched together gather overlapping supports (and the DRAM granules that the
 // short x-runs of one support fetch only in part serve its neighbours).
-template <typename T, typename TC, int CB, int NT, bool ILV>
+template <int CB, int NT>
 __global__ void __launch_bounds__(NT)
-k_project(const T *__restrict__ Y, long ld, int ncols, const int *__restrict__ atom_ptr,
-          const int *__restrict__ idx, const TC *__restrict__ chi, TC *__restrict__ C, TC alpha,
+k_project(const float *__restrict__ Y, long ld, int ncols, const int *__restrict__ atom_ptr,
+          const int *__restrict__ idx, const float *__restrict__ chi, float *__restrict__ C, float alpha,
           const int *__restrict__ order)
 {
     const int J = order ? order[blockIdx.x] : (int)blockIdx.x;
-    project_block<T, TC, CB, NT, ILV>(Y, ld, ncols, J, atom_ptr[J], atom_ptr[J + 1],
+    project_block<CB, NT>(Y, ld, ncols, J, atom_ptr[J], atom_ptr[J + 1],
                                       blockIdx.y * CB, idx, chi, C, alpha);
 }
 
 // Work-list form for a batch of clusters (items: cluster, atom, first column).
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 4)
 k_batch_project(const BatchItem *__restrict__ items, int nitems, const BatchNonlocal *cs)
 {
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const BatchItem w = items[it];
         const BatchNonlocal &P = cs[w.cluster];
-        project_block<float, float, kBatchCols, 256, true>(
+        project_block<kBatchProjCols, 256>(
             P.Y, P.ld, P.ncols, w.a, P.atom_ptr[w.a], P.atom_ptr[w.a + 1], w.col, P.idx,
             P.chi_f, P.C, P.alpha);
     }
@@ -155,7 +147,7 @@ cudaError_t project_f32(const DevHam &H, const float *Y, int ncols, long ld, dou
         constexpr int CB = decltype(cb)::value;
         const dim3 grid(H.natoms, (ncols + CB - 1) / CB);
         if (grid.y > 65535) return cudaErrorInvalidValue;
-        k_project<float, float, CB, NT, true><<<grid, NT, 0, st>>>(
+        k_project<CB, NT><<<grid, NT, 0, st>>>(
             Y, ld, ncols, H.atom_ptr, H.idx, H.chi_f, C, (float)alpha, H.proj_order);
         note_launch();
         return cudaGetLastError();
@@ -514,8 +506,8 @@ cudaError_t scatter_f32(const DevHam &H, const float *Cs, float *out, int ncols,
 }
 
 // Nonlocal scatter for FP64 blocks in pair arithmetic: out(p, c) += sum_{q at p} sum_l
-// g(q, l) Cs(atom(q), l, c), Cs = alpha chi^T Y as pairs (k_project_df). A thread owns one
-// covered node and kScatDfGroups groups of kScatDfCols columns; the grid's x dimension
+// g(q, l) Cs(atom(q), l, c), Cs = alpha chi^T Y as pairs (k_project_fx), the four l of a column
+// side by side. A thread owns one covered node and NG groups of kScatDfCols columns; the grid's x dimension
 // (dispatched first) runs over the column ranges, so the CTAs resident at one time share
 // their covered nodes (the node's entry tables are read from L1/L2, not once per column
 // group from DRAM), and y over blocks of covered nodes (strided when there are more than the

@@ -225,8 +225,6 @@ sparc_status check_block(sparc_ctx *ctx, const void *X, int ncols, long ld, cons
     return SPARC_OK;
 }
 
-size_t esize(sparc_dtype t) { return t == SPARC_F32 ? 4 : 8; }
-
 // --- H applications --------------------------------------------------------------------
 sparc_status ensure_C(sparc_ctx *ctx, int ncols)
 {

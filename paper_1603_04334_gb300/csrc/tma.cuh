@@ -208,18 +208,8 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar)
         : "memory");
 }
 
-// Eight consecutive 32-bit columns of this thread's tensor-memory lane (warp-wide; a warp
+// Four consecutive 32-bit columns of this thread's tensor-memory lane (warp-wide; a warp
 // reaches the 32 lanes of its quarter, warp index mod 4).
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                   "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-}
-
-// Four of them.
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
