@@ -58,7 +58,7 @@
 // formed descriptors and tested barriers for longer than a step's MMAs took, B's 1 KB pieces
 // came in twelve requests a step, and every chunk waited for the epilogue's sums of pairs.
 // Uniform issue, one copy for B, 32-row steps and 64-bit integer sums of which only the
-// combination is waited for: 0.46 ms (128^3 x 512, two slabs, M and H: 33.8 -> 20.9 ms). What
+// combination is waited for: 0.46 ms (128^3 x 512, two slabs, M and H: 33.8 -> 20.6 ms). What
 // is left is that wait, about 2000 cycles a chunk beside 5400 of MMAs (the class accumulators
 // fill 384 of the 512 columns, so no second set fits).
 #include "internal.cuh"

@@ -607,7 +607,8 @@ cudaError_t scatter_f64_df(const DevHam &H, const float2 *Cs, double *out, int n
     // A thread's groups follow one another, so while a launch of one group a thread is a few
     // waves of the chip (four CTAs an SM), it is the shorter: 24^3 x 12, 4 atoms 13.5 -> 7.6 us;
     // 70 x 61 x 53 x 33, 12 atoms (2.3 waves) 26.3 -> 18.6 us; 96^3 x 128, 40 atoms (27 waves)
-    // 133 us with four groups, whose output reads run ahead, 146 us with one.
+    // 133 us with four groups, whose output reads run ahead, 146 us with one (126 us since the
+    // coefficients come by 16-byte loads).
     const long groups = (ncols + kScatDfCols - 1) / kScatDfCols;
     if (nb * groups <= 4 * 4 * 152)
         launch(std::integral_constant<int, 1>{});
