@@ -224,7 +224,7 @@ cudaError_t chi_fixed(int natoms, const int *atom_ptr, const double *chi, int4 *
 // mixed-precision Rayleigh-Ritz step applies H in FP64). bY: the columns' bounds.
 // Grid as k_project: x = atom (in the spatial order), y = column block.
 template <typename T, int CB, int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1)
+__global__ void __launch_bounds__(NT, 1024 / NT)
 k_project_fx(const T *__restrict__ Y, long ld, int ncols, const int *__restrict__ atom_ptr,
              const int *__restrict__ idx, const int4 *__restrict__ chi_q,
              const int *__restrict__ chi_F, const unsigned *__restrict__ bY, double alpha,
@@ -323,24 +323,27 @@ static cudaError_t project_fx(const DevHam &H, const T *Y, int ncols, long ld, d
 {
     if (H.natoms == 0 || ncols <= 0) return cudaSuccess;
     if (!bY) return cudaErrorInvalidValue;
-    auto launch = [&](auto cb, auto nt) {
-        constexpr int CB = decltype(cb)::value, NT = decltype(nt)::value;
-        const dim3 grid(H.natoms, (ncols + CB - 1) / CB);
-        if (grid.y > 65535) return cudaErrorInvalidValue;
+    auto launch = [&](auto nt) {
+        constexpr int CB = 1, NT = decltype(nt)::value;
+        const dim3 grid(H.natoms, ncols);
         k_project_fx<T, CB, NT><<<grid, NT, 0, st>>>(Y, ld, ncols, H.atom_ptr, H.idx, H.chi_q,
                                                      H.chi_F, bY, alpha, C, H.proj_order);
         note_launch();
-        return cudaSuccess;
     };
-    // Two columns a CTA of 256 threads, three CTAs an SM. A single vector (the Lanczos steps) has
-    // one CTA per atom, whose time is its trips over the support: 1024 threads make a quarter of
-    // them (20 atoms, 4189 entries each: 18.9 us with 256 threads and two columns, 11.5 us so).
-    cudaError_t e;
+    if (ncols > 65535) return cudaErrorInvalidValue;
+    // One column a CTA (two, whose accumulators left three CTAs of 256 threads an SM, 110 us at
+    // 96^3 x 128 FP64 with 40 atoms, 18.2 at 70 x 61 x 53 x 33 with 12, 7.9 at 24^3 x 12 with 4).
+    // The threads that walk one support are few where the CTAs fill the chip more than
+    // twice, since each CTA ends in a reduction (128 threads 98 us at 96^3; 256 threads 109),
+    // and more where they do not, since a CTA's time is its trips over the support (256 threads
+    // 15.6 and 6.3 us at the smaller sizes; 128 threads 18.6 and 7.2). A single vector, as in the
+    // Lanczos steps, has one CTA per atom: 20 atoms of 4189 entries 11.5 us with 1024 threads.
     if (ncols == 1)
-        e = launch(std::integral_constant<int, 1>{}, std::integral_constant<int, 1024>{});
+        launch(std::integral_constant<int, 1024>{});
+    else if ((long)H.natoms * ncols >= 2 * 8 * 152)
+        launch(std::integral_constant<int, 128>{});
     else
-        e = launch(std::integral_constant<int, 2>{}, std::integral_constant<int, 256>{});
-    if (e != cudaSuccess) return e;
+        launch(std::integral_constant<int, 256>{});
     return cudaGetLastError();
 }
 
