@@ -240,7 +240,10 @@ sparc_status sparc_nonlocal_force(sparc_ctx *ctx, sparc_dtype dtype, const void 
  *       of Eq. (phi:BC:discrete), l_max = 6 (Sec. 4), |x| measured from the box centre
  *       ((n_d - 1) h / 2 per axis).
  * Conjugate gradients with a Jacobi preconditioner (the paper's block-Jacobi on one block
- * per processor; here the diagonal) from phi = 0, until ||r|| <= tol ||rhs||.
+ * per processor; here the diagonal) from phi = 0, until ||r|| <= tol ||rhs||, r the
+ * iteration's recursive residual. As in any conjugate gradients in 64 bits, rhs + (1/4 pi)
+ * L_h phi formed from phi itself parts from r at some 1e-14 ||rhs|| (3e-14 on 40^3 nodes),
+ * which a tol below that does not improve.
  * rho: Nd doubles (device, x fastest) or NULL for rho = 0; phi: Nd doubles (device,
  * caller-owned) for the result; b_out: Nd doubles (device) for b, or NULL. Writes the
  * iteration count and the final relative residual to *iters_host / *relres_host (each may

@@ -276,10 +276,17 @@ k_poisson_rhs(const double *__restrict__ rho, const double *__restrict__ b,
 //   A  A p on bricks of 16 x 16 x bz nodes, one or more per CTA, and partial sums of p.Ap;
 //   B  r -= alpha A p, partial sums of r.r and the largest |r|;
 //   C  x += alpha p, p = r + beta p, p's grid form and its largest magnitude.
-// The operator works on p's fixed-point grid (d, r) as the FP64 stencil does (stencil_df.cu):
-// exact integer neighbour sums and an FP32 remainder, two FP64 operations a node instead of 37.
-// Phase C writes that form, with the exponent from |p_new| <= max |r| + beta max |p|, so phase A
-// converts nothing. Every CTA adds the CTAs' partial sums itself, in the same order.
+// The operator works on a fixed-point grid, as the FP64 stencil does (stencil_df.cu), but p is
+// kept to 2^-57 of its largest value, as two whole numbers d and r of 28 bits, both summed over
+// the neighbours and weighted in integers without rounding; the result is rounded to 2^-61 of
+// the largest term and then to FP64. That is two FP64 operations a node instead of 37, and closer
+// to the exact operator than those (40^3, radius 6, relative error in the 2-norm: over CG's
+// own p 6e-17 in the median and 2e-15 at most, FP64 5e-16 and 2.7e-15), which CG needs: the
+// recursion follows the operator it is given, so a coarser one (26 bits and an FP32
+// remainder: 7e-15 and 1.9e-13) leaves f - A x at 2.2e-13 of f whatever tol, and this one,
+// like FP64, at 3e-14. Phase C writes that form, with the exponent from |p_new| <= max |r| +
+// beta max |p|, so phase A converts nothing. Every CTA adds the CTAs' partial sums itself, in
+// the same order.
 //
 // Bound by latency: three barriers, the brick's loads from L2 and short FP64 chains (an FP64
 // warp instruction holds its quarter of the SM for 64 cycles). 64^3: 85 us an iteration with
@@ -313,7 +320,6 @@ struct CgArgs {
     CgState *s;
     int n0, n1, n2, bz;
     int W[kRadius + 1];
-    float Wf[kRadius + 1];
     double scale;       // -(1/4 pi) / (D h^2)
     double tol2;
     int first, last;    // iterations of this launch
@@ -385,11 +391,27 @@ __device__ __forceinline__ void cg_get(const double *part, const unsigned *pa, c
     __syncthreads();
 }
 
-// scale 2^(E - 32): the operator's factor for T in 1/64 of a grid unit
+// y on the grid of exponent E, |y| < 2^E: y 2^(28-E) = d + 2^-28 r, both of y's sign, |d| < 2^28,
+// |r| <= 2^28 (rounded to nearest). With the significand at the top of 64 bits, y = (h:l)
+// 2^(e-1086), and (h:l) >> (1026 + E - e) (4 or more) is |y| 2^(60-E). Zero and subnormal y give 0.
+__device__ __forceinline__ int2 cg_grid(double y, int E)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(y);
+    const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
+    const int e = (int)((hw >> 20) & 0x7ffu);
+    const unsigned h = e ? __funnelshift_l(lw, hw, 11) | 0x80000000u : 0u;
+    const unsigned l = e ? lw << 11 : 0u;
+    const unsigned long long N = (((unsigned long long)h << 32) | l) >> min(1026 + E - e, 63);
+    const unsigned f = (unsigned)N;
+    const int sm = (int)hw >> 31;  // 0 or -1
+    return make_int2(((int)(N >> 32) ^ sm) - sm, ((int)((f >> 4) + ((f >> 3) & 1u)) ^ sm) - sm);
+}
+
+// scale 2^(E - 38): the operator's factor for T in 2^-10 of a grid unit 2^(E-28)
 __device__ __forceinline__ double cg_scale(double scale, int E)
 {
-    const int e = E - 32 + 1023;
-    return e > 0 && e < 2047 ? scale * __hiloint2double(e << 20, 0) : ldexp(scale, E - 32);
+    const int e = E - 38 + 1023;
+    return e > 0 && e < 2047 ? scale * __hiloint2double(e << 20, 0) : ldexp(scale, E - 38);
 }
 
 // E with |y| < 2^E for |y| <= a + b c, from the high words of a and c (each at most 2^-20
@@ -445,7 +467,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgArgs g)
             if (gt == 0) s->ff = s->rr = 0.0, s->done = 1, s->iters = 0;
             return;
         }
-        for (long t = gt; t < nd; t += gs) g.q[t] = to_grid(g.p[t], S.E);
+        for (long t = gt; t < nd; t += gs) g.q[t] = cg_grid(g.p[t], S.E);
         if (!grid_barrier(&s->bar, nb, epoch)) return;
     } else {
         if (tid == 0) {
@@ -542,24 +564,17 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgArgs g)
                         if (z >= bz) break;
                         const int2 *c = sm + z * slab + (y + R) * kBrH + hx + R;
                         const int2 *cz = zc + (z * kBr + y) * kBr + hx;
-                        long long A = 0;
-                        float rs = 0.0f;
+                        // (six terms of 28 bits fit 32; the weights' sum is below 2^24.1)
+                        long long A = (long long)g.W[0] * c->x, B = (long long)g.W[0] * c->y;
 #pragma unroll
                         for (int r = R; r >= 1; --r) {
                             const int2 xa = c[r], xb = c[-r], ya = c[r * kBrH], yb = c[-r * kBrH];
                             const int2 za = cz[r * kBr * kBr], zb = cz[-r * kBr * kBr];
-                            const int sd = (xa.x + xb.x + ya.x) + (yb.x + za.x + zb.x);
-                            const float sr = ((__int_as_float(xa.y) + __int_as_float(xb.y)) +
-                                              (__int_as_float(ya.y) + __int_as_float(yb.y))) +
-                                             (__int_as_float(za.y) + __int_as_float(zb.y));
-                            A += (long long)g.W[r] * sd;
-                            rs = fmaf(g.Wf[r], sr, rs);
+                            A += (long long)g.W[r] * ((xa.x + xb.x + ya.x) + (yb.x + za.x + zb.x));
+                            B += (long long)g.W[r] * ((xa.y + xb.y + ya.y) + (yb.y + za.y + zb.y));
                         }
-                        A += (long long)g.W[0] * c->x;
-                        rs = fmaf(g.Wf[0], __int_as_float(c->y), rs);
-                        // T in 1/64 of a unit (the r sum, below 2^25 units, fits 32 bits so)
-                        A = A * 64 + (long long)__float2int_rn(rs * 0x1p-26f);
-                        const double T = (double)A;
+                        // T = (A + 2^-28 B) 2^10, below 2^62.2
+                        const double T = (double)(A * 1024 + ((B + (1 << 17)) >> 18));
                         g.Ap[o0 + plane * z] = T;
                         v = fma(pv[u], T, v);
                     }
@@ -625,7 +640,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgArgs g)
                 g.x[t] = fma(alpha, po[u], x[u]);
                 const double pn = fma(beta, po[u], r[u]);
                 g.p[t] = pn;
-                g.q[t] = to_grid(pn, E);
+                g.q[t] = cg_grid(pn, E);
                 m = max(m, abs_hi_word(pn));
             }
         }
@@ -748,7 +763,6 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
     g.bz = cg_brick_height(n0, n1, n2);
     for (int t = 0; t <= kRadius; ++t) {
         g.W[t] = H.wint[t];
-        g.Wf[t] = (float)H.wint[t];
     }
     g.scale = -kInv4Pi * H.wunit;
     g.tol2 = tol * tol;
