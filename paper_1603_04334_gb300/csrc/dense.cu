@@ -20,13 +20,13 @@
 // FP64 rate), refined to FP64 by products, and checked by the multi-SM FP64 Jacobi, which
 // does what is left. Matrices are column-major in global memory (L2-resident for the sizes
 // used). All loops and waits are bounded.
+#include "device_once.cuh"
 #include "df.cuh"
 #include "fx.cuh"
 #include "grid.cuh"
 #include "internal.cuh"
 #include "rotation.cuh"
 
-#include <atomic>
 #include <type_traits>
 
 namespace sparc {
@@ -397,13 +397,9 @@ static cudaError_t eig_small(const double *A, int n, const int *n_dev, double *e
                              int *status, cudaStream_t st)
 {
     const int smem = kEigArrays * NMAX * (NMAX + 1) * (int)sizeof(double);
-    static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
-    if (!attr_set.load(std::memory_order_acquire)) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            k_eig_small<NMAX, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set.store(true, std::memory_order_release);
-    }
+    static DeviceOnce once;
+    const cudaError_t e = once.allow_smem(smem, k_eig_small<NMAX, NT>);
+    if (e != cudaSuccess) return e;
     k_eig_small<NMAX, NT><<<1, NT, smem, st>>>(A, n, n_dev, ev, Q, status);
     note_launch();
     return cudaGetLastError();
@@ -807,8 +803,6 @@ __global__ void k_refine_rotation(const double *__restrict__ A, double *__restri
     }
 }
 
-static std::atomic<int> g_chol_blocks{0};  // co-resident CTAs of k_chol_grid (queried once)
-
 cudaError_t dense_rr(double *M, double *Hs, int ns, double *ritz, double *Cf, double *work,
                      int *status, cudaStream_t st)
 {
@@ -816,12 +810,8 @@ cudaError_t dense_rr(double *M, double *Hs, int ns, double *ritz, double *Cf, do
     cudaError_t e;
     if ((e = cudaMemsetAsync(status, 0, sizeof(int), st)) != cudaSuccess) return e;
     if (ns <= kSmallEig) {
-        static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
-        if (!attr_set.load(std::memory_order_acquire)) {
-            e = cudaFuncSetAttribute(k_rr_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kRrSmem);
-            if (e != cudaSuccess) return e;
-            attr_set.store(true, std::memory_order_release);
-        }
+        static DeviceOnce once;
+        if ((e = once.allow_smem(kRrSmem, k_rr_small)) != cudaSuccess) return e;
         k_rr_small<<<1, kRrThreads, kRrSmem, st>>>(M, Hs, ns, ritz, Cf, status);
         note_launch();
         return cudaGetLastError();
@@ -840,19 +830,14 @@ cudaError_t dense_rr(double *M, double *Hs, int ns, double *ritz, double *Cf, do
     void *scratch = diag + 8L * ns + 64;
     GridBarrier *bar = (GridBarrier *)(status + 8);
     unsigned *mx = (unsigned *)(status + 13);
-    if (g_chol_blocks.load(std::memory_order_acquire) == 0) {
-        int dev = 0, sms = 0, per = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-            return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_chol_grid, CT, 0)) !=
-            cudaSuccess)
-            return e;
-        g_chol_blocks.store(sms * (per > 0 ? per : 1), std::memory_order_release);
-    }
+    static DeviceOnce coop;
+    int cb;  // co-resident CTAs of k_chol_grid
+    if ((e = coop.get(cb, [](int dev, int &n) {
+             return coop_blocks((const void *)k_chol_grid, CT, dev, n);
+         })) != cudaSuccess)
+        return e;
     long want = (nn / 2 + CT - 1) / CT;
     if (want < 1) want = 1;
-    const int cb = g_chol_blocks.load(std::memory_order_acquire);
     int G0 = (int)(want < cb ? want : cb);
     if (G0 > 152) G0 = 152;
     if ((e = cudaMemsetAsync(bar, 0, sizeof(GridBarrier), st)) != cudaSuccess) return e;

@@ -61,10 +61,10 @@
 // combination is waited for: 0.46 ms (128^3 x 512, two slabs, M and H: 33.8 -> 20.6 ms). What
 // is left is that wait, about 2000 cycles a chunk beside 5400 of MMAs (the class accumulators
 // fill 384 of the 512 columns, so no second set fits).
+#include "device_once.cuh"
 #include "internal.cuh"
 
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include "tma.cuh"
 
@@ -979,14 +979,9 @@ static cudaError_t tc_map(CUtensorMap &m, const __nv_bfloat16 *D, long nblk, lon
 template <class C>
 static cudaError_t tc_prepare(const TcPlan &p, bool sym, int2 *tiles, cudaStream_t st)
 {
-    static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
-    cudaError_t e;
-    if (!attr_set.load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(k_gram_tc<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)TcDims<C>::kSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_set.store(true, std::memory_order_release);
-    }
+    static DeviceOnce once;
+    const cudaError_t e = once.allow_smem((int)TcDims<C>::kSmemBytes, k_gram_tc<C, false>);
+    if (e != cudaSuccess) return e;
     static thread_local int2 host_tiles[64 * 65 / 2 + 64 * 64];
     if (p.ntiles1 > (int)(sizeof(host_tiles) / sizeof(int2))) return cudaErrorInvalidValue;
     int n = 0;
@@ -1163,15 +1158,9 @@ cudaError_t rotate_tc_impl(const TY *Y, long ldy, long nd, int ns, const double 
     int *EA = (int *)take(p.ea_bytes);
     __nv_bfloat16 *DB = (__nv_bfloat16 *)take(p.db_bytes);
     int *EB = (int *)take(p.eb_bytes);
-    static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
-    cudaError_t e;
-    if (!attr_set.load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(k_gram_tc<C, true, TO>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)TcDims<C>::kSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_set.store(true, std::memory_order_release);
-    }
+    static DeviceOnce once;
+    cudaError_t e = once.allow_smem((int)TcDims<C>::kSmemBytes, k_gram_tc<C, true, TO>);
+    if (e != cudaSuccess) return e;
     {   // A = C: K = Ns rows, M = Ns columns
         dim3 grid(p.ns_pad / (2048 / C::kChunk), (unsigned)p.nchunk);
         int *EX = EA + p.nchunk * p.ns_pad;  // (not used by the rotation)

@@ -22,12 +22,12 @@
 // cooperatively (all CTAs co-resident), and every wait is bounded: after kBarrierSpins
 // polls the waiting CTA raises an error flag, every CTA leaves at its next barrier and the
 // host reports SPARC_ERR_TIMEOUT.
+#include "device_once.cuh"
 #include "fx.cuh"
 #include "grid.cuh"
 #include "internal.cuh"
 #include "rotation.cuh"
 
-#include <atomic>
 
 namespace sparc {
 
@@ -188,29 +188,22 @@ static cudaError_t jacobi_grid_t(T *A0, T *A1, T *V, T *diag, int n, GridBarrier
                                  int *status, int *sweeps_out, double eps, int max_sweeps,
                                  cudaStream_t st)
 {
-    static std::atomic<int> coop_blocks{0};  // co-resident CTAs of this instance (queried once)
     if (n <= 0 || n > kMaxDense) return cudaErrorInvalidValue;
-    if (coop_blocks.load(std::memory_order_acquire) == 0) {
-        int dev = 0, sms = 0, per = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_jacobi_grid<T>, NT, 0);
-        if (e != cudaSuccess) return e;
-        coop_blocks.store(sms * (per > 0 ? per : 1), std::memory_order_release);
-    }
+    static DeviceOnce coop;
+    int cb;  // co-resident CTAs of this instance
+    cudaError_t e = coop.get(cb, [](int dev, int &n) {
+        return coop_blocks((const void *)k_jacobi_grid<T>, NT, dev, n);
+    });
+    if (e != cudaSuccess) return e;
     const long half = (n + 1) / 2;
     // a round's FP64 work (the 2 x 2 blocks and the columns of V) spread over four times
     // the CTAs that one block per thread would take: the FP64 pipes of more SMs, at the
     // cost of a barrier over more CTAs
     long want = 4 * ((half * half + NT - 1) / NT);
     if (want < 1) want = 1;
-    const int cb = coop_blocks.load(std::memory_order_acquire);
     int G = (int)(want < cb ? want : cb);
     if (G > kJacobiCtas) G = kJacobiCtas;
-    cudaError_t e = cudaMemsetAsync(bar, 0, sizeof(GridBarrier), st);
-    if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(bar, 0, sizeof(GridBarrier), st)) != cudaSuccess) return e;
     void *args[] = {&A0, &A1, &V, &diag, &n, &bar, &status, &sweeps_out, &eps, &max_sweeps};
     e = cudaLaunchCooperativeKernel((const void *)k_jacobi_grid<T>, dim3(G), dim3(NT), args, 0,
                                     st);

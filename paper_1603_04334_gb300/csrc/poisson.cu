@@ -15,13 +15,13 @@
 //
 // Every reduction (moments, CG dot products) runs in a fixed order: a block-level tree,
 // then one CTA over the block partials, so results repeat bit for bit.
+#include "device_once.cuh"
 #include "fx.cuh"
 #include "grid.cuh"
 #include "internal.cuh"
 #include "rotation.cuh"
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 
 namespace sparc {
@@ -766,22 +766,17 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
     }
     g.scale = -kInv4Pi * H.wunit;
     g.tol2 = tol * tol;
-    static std::atomic<int> sms{0};  // set once (several host threads may launch)
-    if (!sms.load(std::memory_order_acquire)) {
-        int dev = 0, n = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-            return e;
-        if ((e = cudaFuncSetAttribute(k_cg, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kCgSmemMax)) != cudaSuccess)
-            return e;
-        sms.store(n, std::memory_order_release);
-    }
+    static DeviceOnce smem, count;
+    int sms;
+    if ((e = smem.allow_smem(kCgSmemMax, k_cg)) != cudaSuccess) return e;
+    if ((e = count.get(sms, [](int dev, int &n) {
+             return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+         })) != cudaSuccess)
+        return e;
     // enough CTAs for the bricks, and for the vector phases (four nodes per thread)
     const long bricks = (long)((n0 + kBr - 1) / kBr) * ((n1 + kBr - 1) / kBr) * ((n2 + g.bz - 1) / g.bz);
     const long vec = (nd + 4 * kCgThreads - 1) / (4 * kCgThreads);
-    const int grid = (int)std::min<long>(std::min(kCgMaxGrid, sms.load(std::memory_order_acquire)),
-                                         std::max(bricks, vec));
+    const int grid = (int)std::min<long>(std::min(kCgMaxGrid, sms), std::max(bricks, vec));
     if ((e = cudaMemsetAsync(cs, 0, sizeof(CgState), st)) != cudaSuccess) return e;
     CgState h;
     for (int it = 0; it < maxit; it += kCgPerLaunch) {

@@ -29,9 +29,9 @@
 //
 // Requirements (checked on the host, else k_stencil_f32_copy runs): n0 and ld
 // multiples of 4 and 16-byte aligned block pointers (TMA strides and float4 accesses).
+#include "device_once.cuh"
 #include "internal.cuh"
 
-#include <atomic>
 #include <type_traits>
 #include "tma.cuh"
 
@@ -815,17 +815,10 @@ cudaError_t batch_stencil_tma(const BatchItem *items, int nitems, const BatchTma
                               int *err, cudaStream_t st)
 {
     if (nitems <= 0) return cudaSuccess;
-    static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
+    static DeviceOnce once;
     const int smem = kSmemBytes;
-    if (!attr_set.load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(
-            k_batch_stencil_tma<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_batch_stencil_tma<2>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set.store(true, std::memory_order_release);
-    }
+    const cudaError_t e = once.allow_smem(smem, k_batch_stencil_tma<1>, k_batch_stencil_tma<2>);
+    if (e != cudaSuccess) return e;
     // one row per thread while all items are resident at two CTAs per SM (as in stencil_f32_tma)
     if (nitems <= 2 * 152)
         k_batch_stencil_tma<1><<<grid, dim3(kTX, kTY), smem, st>>>(items, nitems, cs, err);
@@ -874,13 +867,9 @@ cudaError_t stencil_f32_copy(const DevHam &H, const float *Y, const float *Yprev
 {
     if (ncols <= 0) return cudaSuccess;
     if (ncols > 65535) return cudaErrorInvalidValue;
-    static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
-    if (!attr_set.load(std::memory_order_acquire)) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            k_stencil_f32_copy, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_set.store(true, std::memory_order_release);
-    }
+    static DeviceOnce once;
+    const cudaError_t e = once.allow_smem(kSmemBytes, k_stencil_f32_copy);
+    if (e != cudaSuccess) return e;
     const int gx = (H.n0 + kBX - 1) / kBX, gy = (H.n1 + kTY - 1) / kTY;
     int nzc, zchunk;
     f32_z_split(H.n2, (long)gx * gy, ncols, nzc, zchunk);
@@ -897,18 +886,10 @@ cudaError_t stencil_f32_tma(const DevHam &H, const float *Y, const float *Yprev,
     PFN_cuTensorMapEncodeTiled_v12000 enc;
     cudaError_t e = tensor_map_encoder(enc);
     if (e != cudaSuccess) return e;
-    static std::atomic<bool> attr_set{false};  // set once (several host threads may launch)
+    static DeviceOnce once;
     const int smem = kSmemBytes;
-    if (!attr_set.load(std::memory_order_acquire)) {
-        if ((e = cudaFuncSetAttribute(k_stencil_f32_tma<1>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
-                cudaSuccess ||
-            (e = cudaFuncSetAttribute(k_stencil_f32_tma<2>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
-                cudaSuccess)
-            return e;
-        attr_set.store(true, std::memory_order_release);
-    }
+    e = once.allow_smem(smem, k_stencil_f32_tma<1>, k_stencil_f32_tma<2>);
+    if (e != cudaSuccess) return e;
     // both maps view a block as (x, y, z, column); they differ in base and box
     auto encode = [&](CUtensorMap *m, const float *base, cuuint32_t bx, cuuint32_t by) {
         cuuint64_t dims[4] = {(cuuint64_t)H.n0, (cuuint64_t)H.n1, (cuuint64_t)H.n2,
