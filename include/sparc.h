@@ -243,7 +243,8 @@ sparc_status sparc_nonlocal_force(sparc_ctx *ctx, sparc_dtype dtype, const void 
  * per processor; here the diagonal) from phi = 0, until ||r|| <= tol ||rhs||, r the
  * iteration's recursive residual. As in any conjugate gradients in 64 bits, rhs + (1/4 pi)
  * L_h phi formed from phi itself parts from r at some 1e-14 ||rhs|| (3e-14 on 40^3 nodes),
- * which a tol below that does not improve.
+ * which a tol below that does not improve. NaN in rho is no error: phi is NaN, with maxit
+ * iterations and a relative residual of 0.
  * rho: Nd doubles (device, x fastest) or NULL for rho = 0; phi: Nd doubles (device,
  * caller-owned) for the result; b_out: Nd doubles (device) for b, or NULL. Writes the
  * iteration count and the final relative residual to *iters_host / *relres_host (each may

@@ -793,9 +793,11 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
         if (h.done || h.bar.err) break;
     }
-    *iters_host = h.iters;
-    // a barrier that gave up counts as no convergence
-    *relres_host = h.bar.err ? INFINITY : h.ff > 0.0 ? std::sqrt(h.rr / h.ff) : h.rr;
+    // a NaN never meets the tolerance: the iterations left after it would change nothing
+    *iters_host = std::isnan(h.rr) ? maxit : h.iters;
+    // a barrier that gave up counts as no convergence; with a right-hand side of zeros, or with NaN
+    // in it, there is nothing to compare with
+    *relres_host = h.bar.err ? INFINITY : h.ff > 0.0 ? std::sqrt(h.rr / h.ff) : 0.0;
     return cudaGetLastError();
 }
 
