@@ -414,6 +414,15 @@ __device__ __forceinline__ double cg_scale(double scale, int E)
     return e > 0 && e < 2047 ? scale * __hiloint2double(e << 20, 0) : ldexp(scale, E - 38);
 }
 
+// tol^2 |f|^2, or -1 (never reached) where f is so small (its norm below 1e-144) that this
+// vanishes: the last values of r.r would be a few units of the smallest number and then 0, which
+// is no residual below the tolerance
+__device__ __forceinline__ double cg_stop(double tol2, double ff)
+{
+    const double s = tol2 * ff;
+    return s < 0x1p-1060 && ff < 0x1p-960 ? -1.0 : s;
+}
+
 // E with |y| < 2^E for |y| <= a + b c, from the high words of a and c (each at most 2^-20
 // above its value's truncation) and b >= 0
 __device__ __forceinline__ int cg_exponent(unsigned a, double b, unsigned c)
@@ -439,7 +448,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgArgs g)
     // the iteration's scalars; thread 0 writes them between barriers that all threads pass
     // before they read or after they have read them
     __shared__ struct {
-        double rr, ff, alpha, as, beta, sc, stop;  // sc: Ap = sc T; stop = tol^2 |f|^2
+        double rr, ff, alpha, as, beta, sc, stop;  // sc: Ap = sc T; stop: of r.r
         int E, done;
     } S;
     unsigned m, epoch = 0;
@@ -459,7 +468,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgArgs g)
         if (!grid_barrier(&s->bar, nb, epoch)) return;
         cg_get(part1, pmax2, pmax2, [&](double u, unsigned x, unsigned) {
             S.rr = S.ff = u;
-            S.stop = g.tol2 * u;
+            S.stop = cg_stop(g.tol2, u);
             S.E = bound_exponent(x);
             S.sc = cg_scale(g.scale, S.E);
         });
@@ -473,7 +482,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgArgs g)
         if (tid == 0) {
             S.rr = s->rr;
             S.ff = s->ff;
-            S.stop = g.tol2 * S.ff;
+            S.stop = cg_stop(g.tol2, S.ff);
             S.E = s->E;
             S.sc = cg_scale(g.scale, S.E);
         }
@@ -798,6 +807,8 @@ cudaError_t poisson_solve(const DevHam &H, const double *R, const double *Z, int
     // a barrier that gave up counts as no convergence; with a right-hand side of zeros, or with NaN
     // in it, there is nothing to compare with
     *relres_host = h.bar.err ? INFINITY : h.ff > 0.0 ? std::sqrt(h.rr / h.ff) : 0.0;
+    // and below cg_stop's range r.r says nothing any more
+    if (!h.done && *relres_host <= tol) *relres_host = NAN;
     return cudaGetLastError();
 }
 

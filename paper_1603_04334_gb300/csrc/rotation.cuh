@@ -43,9 +43,12 @@ __device__ __forceinline__ double fast_reciprocal(double d)
     return y * __hiloint2double((2046 - e) << 20, 0);
 }
 
-// a / b to about an ulp (a short chain; b as for fast_reciprocal, else a plain division)
+// a / b to about an ulp (a short chain; b as for fast_reciprocal, else a plain division: the
+// reciprocal of a subnormal b may overflow where the quotient does not)
 __device__ __forceinline__ double fast_quotient(double a, double b)
 {
+    const int e = (__double2hiint(b) >> 20) & 0x7ff;
+    if (e < 2 || e > 2044) return a / b;
     const double y = fast_reciprocal(fabs(b));
     const double q = a * y, d = fabs(b);
     const double z = isfinite(q) ? fma(y, fma(-q, d, a), q) : q;
