@@ -151,8 +151,9 @@ sparc_status sparc_cheb_filter(sparc_ctx *ctx, sparc_dtype dtype, void *X, void 
  * FP32 results (the block's own precision; residuals good to about 1e-7 of ||H x_n||).
  * HXf_or_null: optional FP64 device
  * block (ncols x ld) used as the H Xf workspace; when NULL the context allocates one.
- * Fails with SPARC_ERR_NOT_SPD if M_s is not numerically positive definite and with
- * SPARC_ERR_NONFINITE on NaN/Inf, leaving Xf unrotated. ncols <= 1024. Synchronises. */
+ * Fails with SPARC_ERR_NOT_SPD if M_s is not numerically positive definite (a column's norm
+ * below 2^-68 counts as zero) and with SPARC_ERR_NONFINITE on NaN/Inf (or entries of M_s or
+ * H_s above 2^136), leaving Xf unrotated. ncols <= 1024. Synchronises. */
 sparc_status sparc_orth_rr(sparc_ctx *ctx, sparc_dtype dtype, void *Xf, void *HXf_or_null,
                            int ncols, long ld, double *ritz_host, double *resid_host);
 

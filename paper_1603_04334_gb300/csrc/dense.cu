@@ -40,6 +40,16 @@ constexpr int kEigArrays = 6;   // shared-memory matrices of the one-CTA eigenso
 constexpr int kMaxSweeps32 = 20;
 constexpr int kRefine = 2;
 
+// M_s and H_s are taken between 2^-136 (M_s's diagonal; below: status 1, no basis) and 2^136 (any
+// entry; beyond, and NaN: status 2), which is the range of FP32 products. Blocks beyond it are
+// not orbitals, and the squares of their overlaps in the Cholesky step would leave FP64's range
+// (columns of 1e-140 came out 1e-2 from orthonormal), as their FP32 values do H's.
+__device__ __forceinline__ bool in_range(double x) { return fabs(x) <= 0x1p136; }
+__device__ __forceinline__ bool pivot_ok(double pivot, double diag, int n)
+{
+    return pivot > 4.0 * n * kEps * diag && diag >= 0x1p-136 && isfinite(pivot);
+}
+
 // Entry (i, j) of the refinement rotation: a / (a_jj - a_ii), or 0 where the two are too close
 // for two Newton-Schulz steps to make I + E orthogonal again: |E_ij| > 1/64, or a gap below
 // 2^-16 of the matrix (mx: high word of its largest entry), where whole multiplets of
@@ -437,7 +447,7 @@ k_rr_small(const double *__restrict__ M, const double *__restrict__ Hs, int n,
         A[i + j * LD] = m;
         B[i + j * LD] = h;
         if (i == j) od[i] = m;
-        if (!isfinite(m) || !isfinite(h)) bad = 1;
+        if (!in_range(m) || !in_range(h)) bad = 1;
     }
     __syncthreads();
     if (bad) {
@@ -448,7 +458,7 @@ k_rr_small(const double *__restrict__ M, const double *__restrict__ Hs, int n,
     // pivot; L_rj = A_rj / sqrt(piv_j)
     for (int j = 0; j < n; ++j) {
         const double d = A[j + j * LD];
-        if (!(d > 4.0 * n * kEps * od[j]) || !isfinite(d)) {
+        if (!pivot_ok(d, od[j], n)) {
             if (tid == 0) *status = 1;
             return;
         }
@@ -539,8 +549,8 @@ constexpr int CT = 256;       // threads per CTA of the cooperative Cholesky
 constexpr int kInvWarps = 4;  // columns per CTA of the triangular inverse
 }  // namespace
 
-// Symmetrise M_s and H_s and check them for non-finite entries (status 2); Cholesky with
-// the pivot rule pivot_j > 4 n eps M_jj (status 1 otherwise); writes L row-major into Lr
+// Symmetrise M_s and H_s and check them for entries out of range (status 2); Cholesky with
+// the pivot rule pivot_j > 4 n eps M_jj (pivot_ok; status 1 otherwise); writes L row-major into Lr
 // (Lr[k + r n] = L_rk, zero above the diagonal) and 1 / L_jj into dinv. Every CTA reads
 // the same pivot after the barrier, so all take the same decision. M is overwritten by the
 // Schur complements; odiag holds the original diagonal. A barrier that times out sets
@@ -567,9 +577,9 @@ k_chol_grid(double *M, double *Hs, int n, double *Lr, double *dinv, double *odia
             M[tt] = m;
             Hs[t] = h;
             Hs[tt] = h;
-            if (!isfinite(m) || !isfinite(h)) atomicExch(status, 2);
+            if (!in_range(m) || !in_range(h)) atomicExch(status, 2);
         } else if (i == j) {
-            if (!isfinite(M[t]) || !isfinite(Hs[t])) atomicExch(status, 2);
+            if (!in_range(M[t]) || !in_range(Hs[t])) atomicExch(status, 2);
             odiag[i] = M[t];
         }
     }
@@ -577,7 +587,7 @@ k_chol_grid(double *M, double *Hs, int n, double *Lr, double *dinv, double *odia
     if (*((volatile int *)status) != 0) return;
     for (int j = 0; j < n; ++j) {
         const double d = __ldcg(M + j + (long)j * n);
-        if (!(d > 4.0 * n * kEps * __ldcg(odiag + j)) || !isfinite(d)) {
+        if (!pivot_ok(d, __ldcg(odiag + j), n)) {
             if (gtid == 0) atomicExch(status, 1);
             return;
         }
