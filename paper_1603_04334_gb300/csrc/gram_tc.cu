@@ -36,7 +36,10 @@
 // along Nd; the FP32-pair Gram of gram_df.cu remains the exact one. The 47-bit form combines a
 // chunk's accumulators into one 64-bit integer, shifts it right by the chunk's exponents'
 // distance from the columns' largest (E_i - e_i + E_j - e_j, rounded) and adds it to a 64-bit
-// integer sum.
+// integer sum. One unit of that sum is 2^(E_i + E_j - 54 + drop) (drop: log2 of a split's
+// chunks, at most 7 at 96^3 x 128), also for two columns whose large values lie in different
+// chunks: the entry's error is absolute, about 2^-45 max|x_i| max|x_j|, which against the
+// columns' norms is below FP64's rounding once they spread over some 256 nodes.
 //
 // Layout and pipeline. A pre-pass (k_tc_digits) writes the digits of an operand in the
 // shared-memory order the MMA reads (no swizzle, K-major, 8-row x 16-byte core matrices)
@@ -341,7 +344,10 @@ __device__ __forceinline__ double scaled_to_double(long long a, int sc)
 
 // The chunk's integer T from Tc47's class sums (exact integers in FP32, below 2^21, 2^22, 2^22.6,
 // 2^23, 2^23.4, 2^23.6). Integers up to 2^22 come out of the significand of 1.5 2^23 + v, larger
-// ones by conversion; the last two classes are rounded together to 2^10 (2^-51 of T's range).
+// ones by conversion; the last two classes, as 2^8 f4 + f5 = 2^10 t + g with t = f4 / 4 rounded
+// and the exact remainder g, are rounded to 4 units, 2^-50 of the largest product (rounded to
+// 2^10 in one step they cost four operations less, and columns whose largest values stand out by
+// 2^20 and more, where the sums are far below T's range, lost bits that the digits hold).
 __device__ __forceinline__ long long class_sum47(const uint32_t (&v)[6])
 {
     constexpr float kM = 12582912.0f;
@@ -349,9 +355,12 @@ __device__ __forceinline__ long long class_sum47(const uint32_t (&v)[6])
     const int b0 = __float_as_int(f(0) + kM), b1 = __float_as_int(f(1) + kM);
     const int i1 = (int)(((unsigned)b0 << 8) + (unsigned)b1 - (0x40000000u + 0x4B400000u));
     const int i2 = (int)(((unsigned)__float2int_rn(f(2)) << 8) + (unsigned)__float2int_rn(f(3)));
-    const float l = fmaf(f(5), 0x1p-10f, fmaf(f(4), 0x1p-2f, kM));
-    const int i3 = __float_as_int(l) - 0x4B400000;
-    return ((long long)i1 << 32) + ((long long)i2 * 65536 + (long long)i3 * 1024);
+    const float t = fmaf(f(4), 0.25f, kM);
+    const float g = fmaf(fmaf(t - kM, -4.0f, f(4)), 256.0f, f(5));  // below 2^23.7: exact
+    const float l = fmaf(g, 0.25f, kM);
+    const int i3 = (int)(((unsigned)__float_as_int(t) << 8) + (unsigned)__float_as_int(l) -
+                         (0x40000000u + 0x4B400000u));
+    return ((long long)i1 << 32) + ((long long)i2 * 65536 + (long long)i3 * 4);
 }
 
 // Digits of the transposed operand: B = Y^T for the rotation, so the K dimension runs over
