@@ -15,11 +15,11 @@
 // Eigenvalues are sorted ascending and each eigenvector column is signed so that its
 // largest-magnitude entry is positive (lowest index on ties).
 //
-// Up to kSmallEig states (and the k x k Lanczos problem) the FP64 Jacobi runs in one CTA's
-// shared memory. Larger problems are solved approximately in FP32 (jacobi.cu, 64 times the
-// FP64 rate), refined to FP64 by products, and checked by the multi-SM FP64 Jacobi, which
-// does what is left. Matrices are column-major in global memory (L2-resident for the sizes
-// used). All loops and waits are bounded.
+// At every size the problem is solved approximately in FP32 (64 times the FP64 rate), refined
+// to FP64 by products, and checked by the FP64 Jacobi, which does what is left: up to kSmallEig
+// states (and the k x k Lanczos problem) in one CTA's shared memory, above on many SMs
+// (jacobi.cu). Matrices are column-major in global memory (L2-resident for the sizes used). All
+// loops and waits are bounded.
 #include "device_once.cuh"
 #include "df.cuh"
 #include "fx.cuh"
@@ -415,10 +415,10 @@ static cudaError_t eig_small(const double *A, int n, const int *n_dev, double *e
     return cudaGetLastError();
 }
 
-// The whole reduction and eigensolve for n <= kSmallEig states in one CTA, all in FP64 and
-// shared memory: M_s and H_s symmetrised and checked (status 2), Cholesky with the pivot rule
-// of k_chol_grid (status 1), U = L^-T, A = U^T H_s U, Jacobi (status 3), sort and sign, and
-// Cf = U Q. Six launches and a grid barrier per column and per rotation round otherwise: 12
+// The whole reduction and eigensolve for n <= kSmallEig states in one CTA and its shared memory,
+// in FP64 but for the eigensolve's FP32 start (eig_cta): M_s and H_s symmetrised and checked
+// (status 2), Cholesky with the pivot rule of k_chol_grid (status 1), U = L^-T, A = U^T H_s U, the
+// eigensolve (status 3), sort and sign, and Cf = U Q. Six launches and a grid barrier per column and per rotation round otherwise: 12
 // states, 380 us -> 100 us.
 namespace {
 constexpr int kRrThreads = 256;

@@ -186,23 +186,4 @@ cudaError_t resid_f32(const float *X, const float *HX, long ld, long nd, int nco
     return resid<float>(X, HX, ld, nd, ncols, ritz, part, out, st);
 }
 
-__global__ void k_check_finite(const double *a, long n, int *flag)
-{
-    int bad = 0;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-         q += (long)gridDim.x * blockDim.x)
-        if (!isfinite(a[q])) bad = 1;
-    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
-}
-
-cudaError_t check_finite(const double *a, long n, int *flag, cudaStream_t st)
-{
-    int b = (int)((n + 255) / 256);
-    if (b > 152 * 4) b = 152 * 4;
-    if (b < 1) b = 1;
-    k_check_finite<<<b, 256, 0, st>>>(a, n, flag);
-    note_launch();
-    return cudaGetLastError();
-}
-
 }  // namespace sparc

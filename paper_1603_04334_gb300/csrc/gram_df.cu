@@ -3,7 +3,7 @@
 //
 // GB300's FP64 pipe issues at 1/64 of the FP32 rate, so a native FP64 Gram of a
 // 884736 x 128 block takes ~23 ms. Here every FP64 input is split into an FP32 pair
-// (hi, lo) (see split_double in stencil_df.cu) and each product a*b is accumulated as
+// (hi, lo) (split_double in df.cuh) and each product a*b is accumulated as
 //   p = ah*bh exactly via TwoProduct (FMA), p added to the running sum with TwoSum, and
 //   the product error, the TwoSum error and the cross terms ah*bl + al*bh collected in a
 //   second FP32 accumulator

@@ -36,10 +36,11 @@
 // along Nd; the FP32-pair Gram of gram_df.cu remains the exact one. The 47-bit form combines a
 // chunk's accumulators into one 64-bit integer, shifts it right by the chunk's exponents'
 // distance from the columns' largest (E_i - e_i + E_j - e_j, rounded) and adds it to a 64-bit
-// integer sum. One unit of that sum is 2^(E_i + E_j - 54 + drop) (drop: log2 of a split's
-// chunks, at most 7 at 96^3 x 128), also for two columns whose large values lie in different
-// chunks: the entry's error is absolute, about 2^-45 max|x_i| max|x_j|, which against the
-// columns' norms is below FP64's rounding once they spread over some 256 nodes.
+// integer sum. A chunk is rounded to one unit of that sum, 2^(E_i + E_j - 54 + drop) (drop:
+// log2 of a split's chunks, 8 at 96^3 x 128), also where the large values of the two columns
+// lie in different chunks: the entry's error is absolute, over 6912 chunks about 2^-41 max|x_i|
+// max|x_j|, which against the columns' norms is below FP64's rounding once they spread over some
+// thousands of nodes.
 //
 // Layout and pipeline. A pre-pass (k_tc_digits) writes the digits of an operand in the
 // shared-memory order the MMA reads (no swizzle, K-major, 8-row x 16-byte core matrices)
@@ -61,7 +62,7 @@
 // formed descriptors and tested barriers for longer than a step's MMAs took, B's 1 KB pieces
 // came in twelve requests a step, and every chunk waited for the epilogue's sums of pairs.
 // Uniform issue, one copy for B, 32-row steps and 64-bit integer sums of which only the
-// combination is waited for: 0.46 ms (128^3 x 512, two slabs, M and H: 33.8 -> 20.6 ms). What
+// combination is waited for: 0.47 ms (128^3 x 512, two slabs, M and H: 33.8 -> 21 ms). What
 // is left is that wait, about 2000 cycles a chunk beside 5400 of MMAs (the class accumulators
 // fill 384 of the 512 columns, so no second set fits).
 #include "device_once.cuh"

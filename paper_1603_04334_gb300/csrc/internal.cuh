@@ -107,8 +107,8 @@ cudaError_t scatter_f32(const DevHam &H, const float *Cs, float *out, int ncols,
                         cudaStream_t st);
 // ---- batched FP32 filter steps over many clusters (batch.cu) --------------------------
 // One unit of work of a batched launch. stencil: column `col`, tile (a, b) of the x-y
-// plane, planes k0 .. k1-1; projection: atom a, columns col .. col+15; scatter: covered
-// nodes a*256 .. a*256+255, columns col .. col+15.
+// plane, planes k0 .. k1-1; projection: atom a, kBatchProjCols columns from col on; scatter:
+// covered nodes a*kBatchNodes .., kBatchCols columns from col on.
 struct BatchItem {
     int cluster, col, a, b, k0, k1;
 };
@@ -316,9 +316,7 @@ cudaError_t dense_syev(const double *A, int ns, const int *ns_dev, double *ev, d
 // Grid-wide barrier state (zeroed before each cooperative launch).
 struct GridBarrier {
     unsigned count;  // arrivals since the barrier was zeroed (grid.cuh)
-    unsigned gen;    // unused
     int err;
-    int pad;
 };
 // Multi-SM cyclic Jacobi of A0 (n x n, column-major; A1 is a second n x n buffer):
 // eigenvalues (unsorted) in diag, eigenvectors in V. Skipped if *status != 0 on entry;
@@ -328,7 +326,8 @@ cudaError_t jacobi_grid(double *A0, double *A1, double *V, double *diag, int n, 
 // Block Jacobi in FP32 (jacobi.cu): V = approximate eigenvectors of the symmetric A64 (n x n,
 // column-major); A: n x n FP32 workspace; mx: a device word; scratch of
 // block_jacobi_f32_scratch(n) bytes (device, 8-byte aligned); *sweeps_out (device) = sweeps
-// used or -1. Synchronises the stream once per sweep from the fourth on.
+// used or -1. Synchronises the stream once per sweep: from the fourth on, or from the first where
+// one pair of blocks is the whole matrix (n <= 64).
 size_t block_jacobi_f32_scratch(int n);
 cudaError_t block_jacobi_f32(const double *A64, float *A, float *V, int n, unsigned *mx,
                              void *scratch, int *sweeps_out, int max_sweeps, cudaStream_t st);
@@ -369,8 +368,6 @@ cudaError_t resid_f64(const double *X, const double *HX, long ld, long nd, int n
                       const double *ritz, double *part, double *resid, cudaStream_t st);
 cudaError_t resid_f32(const float *X, const float *HX, long ld, long nd, int ncols,
                       const double *ritz, double *part, double *resid, cudaStream_t st);
-// flag |= 1 if any of n values is NaN or Inf
-cudaError_t check_finite(const double *a, long n, int *flag, cudaStream_t st);
 
 // ---- observables.cu -----------------------------------------------------------------
 // Fermi level of Eq. (FermiEnergyConstraintFormulation): *mu with 2 sum g_n = nelec, g

@@ -278,7 +278,8 @@ k_project_fx(const T *__restrict__ Y, long ld, int ncols, const int *__restrict_
     }
     // |a d| and |a r + b d| are below 2^50: a thread's sums stay below 2^(50 + log2 t) for t
     // entries; before the 32-way warp sum they are shifted right by max(0, log2 t - 7) so that
-    // it stays below 2^62 (for supports up to 32768 entries per atom no shift is needed)
+    // it stays below 2^62 (no shift up to 128 NT entries per atom: 16384 with 128 threads, 131072
+    // with 1024)
     const int t = (e - b + NT - 1) / NT;
     const int sh = t > 128 ? (32 - __clz(t - 1)) - 7 : 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;

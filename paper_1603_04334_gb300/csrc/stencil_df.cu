@@ -1,13 +1,12 @@
 // stencil_df.cu -- the FP64 fused stencil step on the integer, FP32 and FP64 pipes.
 //
-// Same operation and blocking as k_stencil in stencil.cu (Eq. FD:Laplacian with the
-// weights of Eq. weightsLap, zero-Dirichlet boundaries, V_eff and the Chebyshev
-// three-term recurrence of Algorithm ChebychevFilter, Sec. 3.4), for FP64 blocks. GB300
-// issues FP64 at 1/64 of its FP32 rate, so a native FP64 stencil (37 FP64 multiply-adds
-// per point) is bound by the FP64 pipe at a few per cent of HBM bandwidth. This kernel
-// spends three FP64 operations per point:
+// The operation of stencil.cu (Eq. FD:Laplacian with the weights of Eq. weightsLap,
+// zero-Dirichlet boundaries, V_eff and the Chebyshev three-term recurrence of Algorithm
+// ChebychevFilter, Sec. 3.4), for FP64 blocks. GB300 issues FP64 at 1/64 of its FP32 rate, so a
+// native FP64 stencil (37 FP64 multiply-adds per point) is bound by the FP64 pipe at a few per
+// cent of HBM bandwidth. This kernel spends three FP64 operations per point:
 //   * The Laplacian weights of radius n_o are rationals with one small common
-//     denominator D (h^2 w_p = W_p / D, W_p integers, D = 831600 for n_o = 6), so
+//     denominator D (h^2 w_p = W_p / D, W_p integers, D = 831600 for every n_o), so
 //     h^2 D L_h y = sum_p W_p S_p is an integer combination of the neighbour sums S_p.
 //   * Every value of a column is put on a fixed-point grid: with |y| < 2^E over the
 //     column (E from a per-column bound), y 2^(26-E) = d + 2^-32 r with d an integer truncated
@@ -23,8 +22,11 @@
 //     more FP64 operations a point. Where that does not fit (a kinetic scale other than 1, a
 //     potential beyond 2^25 units) the general form computes alpha (V_p - shift) y_p in FP64.
 // Error: the rounding of r (2^-51 of the column's largest value per value) and the FP32
-// rounding of the r sum (about a unit of 2^(E-26), weighted by g ~ 1e-5 at h = 0.3): about
-// 2^-42 of the column's largest value in the worst case, FP64 rounding elsewhere. A column
+// rounding of the r sum and of the potential's product (about a unit of 2^(E-26), weighted by g ~
+// 1e-5 at h = 0.3, at every radius): about 2^-42 of the column's largest value in the worst case,
+// 1.3e-15 to 1.8e-15 of the largest |H X| measured at radii 1 to 6. The potential term, an FP64
+// product of y itself in the general form, is thereby absolute in the column, as the
+// Laplacian's part always is. A column
 // whose bound is not finite (Inf or NaN anywhere in Y_j) gives NaN in every output value of
 // the column. Each launch can raise the output's column bounds (atomicMax), which is how
 // the filter hands the bound of Y_{j+1} to the next step without another pass over the
@@ -107,18 +109,20 @@ __device__ __forceinline__ float2 r_pair(const int4 &v)
 // row above and below: 288 for 256 threads) are loaded and converted by all threads, the
 // last 32 by warp 0 alone. The next plane's halo pairs, queue entry, potential and Y_{j-1}
 // are loaded during the current plane's compute (loading the potential and Y_{j-1} of the same
-// plane at the start of its step instead took 1.6 ms against 1.03 for 96^3 x 128).
+// plane at the start of its step instead took 1.6 ms against 1.13 for 96^3 x 128).
 //
 // What bounds it: latency (shared-memory reads and the FP64 pipe; issue slots 42% busy, the
-// shared-memory pipe 58%, FP64 50%) at the 16 warps that 128 registers leave. The pair
+// shared-memory pipe 58%, FP64 50%) at the 16 warps that 128 registers leave, which is also less
+// than it wants: the usual form spills 128 bytes of stores and 312 of loads a thread over the 13
+// unrolled planes (FP32 input 148 and 468, the general form 136 and 340). The pair
 // form reads 18 16-byte values for the neighbours of two nodes (a thread per node: 48 of 8
 // bytes), the r sums run on packed FP32 pairs, addresses, predicates and the barrier are shared
 // by two nodes and the loads and stores are 16 bytes wide: about 162 thread instructions per
 // node against 282. VINT (the integer potential, the usual form) takes alpha (V - shift) y out
 // of the FP64 pipe: V / g on a 2^-30 grid of the weights' units (DevHam::uq) joins the centre
 // weight, so a point costs three FP64 operations instead of four and no second read of y.
-// A launch of 96^3 x 128: 1.435 ms with one node per thread, 1.12 ms in this form; the degree-20
-// filter's error against 64-bit arithmetic went from 2.0e-14 to 1.5e-14 of its norm.
+// A filter step of 96^3 x 128: 1.435 ms with one node per thread, 1.13 ms in this form; the
+// degree-20 filter's error against 64-bit arithmetic went from 2.0e-14 to 1.4e-14 of its norm.
 template <typename TI, bool VEC, bool VINT>
 __global__ void __launch_bounds__(kDfPX *kDfBY, 2)
 k_stencil_df(const TI *__restrict__ Yb, const double *Yprev, double *outb,
